@@ -1172,165 +1172,225 @@ __global__ void __launch_bounds__(128) patch_apply_f64(int npatch, const int* __
 // One ASM sweep with factored saddle inverses (saddle_core's factored form):
 //   t = r_p - W^T r_u,  s = Si t,  z_u = blockdiag(Li) r_u + W s,  z_p = -s,
 //   Y[poff[i] + a] = w[dof_a] z_a.
-// One CTA of SADDLE_APPLY_THREADS threads per patch.  The gathered residual
-// and W are staged in shared memory (W is used twice); Li is streamed from
-// HBM once, as in patch_apply_body: a thread owns VEC consecutive rows and
-// accumulates them for the d components at once, G groups of row owners
-// split the columns, eight 16-byte loads in flight per thread, the groups'
-// partial sums added in a fixed order.
-__device__ __forceinline__ float vcomp(const float4& v, int e) { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
-__device__ __forceinline__ double vcomp(const double2& v, int e) { return e == 0 ? v.x : v.y; }
-__device__ __forceinline__ float4 mkvec(const float* a, float4*) { return make_float4(a[0], a[1], a[2], a[3]); }
-__device__ __forceinline__ double2 mkvec(const double* a, double2*) { return make_double2(a[0], a[1]); }
+// One CTA of SADDLE_APPLY_THREADS threads per patch.  Only vectors live in
+// shared memory; Li, W and Si stream from global memory into registers, so
+// that seven CTAs share an SM and one's loads cover the others' barriers and
+// dependent loads.  Staging W in shared memory, to read it once, left one to
+// three CTAs per SM: 584 us against 162 us on the FP64 P6 level of the 32 x 32
+// square (1089 patches; bound by the FP64 pipe at 116 us), 176 against 135 us on
+// 3D P3 16^3 (3.9 TB/s), 155 against 130 us on P8 (5.4 TB/s: there W, 220 KB a
+// patch, comes from DRAM both times), 184 against 131 us on the SV P4 disk.
+// Fewer, larger CTAs (256 or 512 threads), 64 threads, and a bulk prefetch of
+// the block into L2 were each measured no faster.
+template <typename T, int D> struct ColVec;              // x of one column, all components
+template <> struct __align__(4) ColVec<float, 1> { float v[1]; };
+template <> struct __align__(8) ColVec<float, 2> { float v[2]; };
+template <> struct __align__(16) ColVec<float, 3> { float v[4]; };
+template <> struct __align__(8) ColVec<double, 1> { double v[1]; };
+template <> struct __align__(16) ColVec<double, 2> { double v[2]; };
+template <> struct __align__(16) ColVec<double, 3> { double v[4]; };
+template <typename T> struct Vec16;                      // 16 bytes of consecutive rows
+template <> struct Vec16<float> {
+    static constexpr int N = 4;
+    float4 v;
+    __device__ __forceinline__ float at(int e) const { return e == 0 ? v.x : e == 1 ? v.y : e == 2 ? v.z : v.w; }
+    __device__ __forceinline__ void set(const float* a) { v = make_float4(a[0], a[1], a[2], a[3]); }
+};
+template <> struct Vec16<double> {
+    static constexpr int N = 2;
+    double2 v;
+    __device__ __forceinline__ double at(int e) const { return e == 0 ? v.x : v.y; }
+    __device__ __forceinline__ void set(const double* a) { v = make_double2(a[0], a[1]); }
+};
+// streaming (read once) and cached 16-byte loads
+template <bool ONCE, typename T>
+__device__ __forceinline__ Vec16<T> load16(const Vec16<T>* p) {
+    Vec16<T> r;
+    r.v = ONCE ? __ldcs(&p->v) : __ldg(&p->v);
+    return r;
+}
 
-template <typename T, typename V, int VEC>
-__device__ __forceinline__ void saddle_apply_body(int p, int d, const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                                  const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                                  const T* __restrict__ fac, const T* __restrict__ r,
-                                                  const T* __restrict__ wt, T* __restrict__ Y, int xs_len, int ws_len,
-                                                  unsigned char* smem) {
-    constexpr int NT = SADDLE_APPLY_THREADS;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int s0 = poff[p], n = poff[p + 1] - s0, nv = pnv[p], dnv = d * nv, np = n - dnv;
-    if (n == 0) return;
-    const int ldl = (nv + VEC - 1) / VEC * VEC, ldw = (dnv + VEC - 1) / VEC * VEC;
-    const T* Li = fac + foff[p];
-    const T* Wg = Li + (long long)ldl * nv;
-    const T* Sg = Wg + (long long)ldw * np;
-    V* red = reinterpret_cast<V*>(smem);                         // [NT][3]
-    T* ws = reinterpret_cast<T*>(smem + sizeof(V) * NT * 3);     // [ws_len]   W, column-major
-    T* xs = ws + ws_len;                                         // [xs_len]   gathered r
-    T* ys = xs + xs_len;                                         // [xs_len]   blockdiag(Li) r_u
-    T* tq = ys + xs_len;                                         // [xs_len]   t
-    T* sq = tq + xs_len;                                         // [xs_len]   s
-    for (int a = tid; a < n; a += NT) xs[a] = r[pdofs[s0 + a]];
-    // W is staged in shared memory when the level's largest fits (ws_len > 0),
-    // else both of its uses read it from global memory (the second from cache)
-    const T* wsrc = ws_len > 0 ? ws : Wg;
-    if (ws_len > 0) {
-        const V* wv = reinterpret_cast<const V*>(Wg);
-        V* wsv = reinterpret_cast<V*>(ws);
-        const int nvec = ldw * np / VEC;
-        for (int t = tid; t < nvec; t += NT) wsv[t] = __ldcs(wv + t);
-    }
-    __syncthreads();
-    // t = r_p - W^T r_u: one warp per pressure row, lanes over the velocity DoFs
-    for (int q = warp; q < np; q += NT / 32) {
-        const T* wc = wsrc + (long long)q * ldw;
-        T acc = 0;
-        for (int a = lane; a < dnv; a += 32) acc += wc[a] * xs[a];
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) tq[q] = xs[dnv + q] - acc;
-    }
-    __syncthreads();
-    // s = Si t (Si symmetric: entry (q, x) at Sg[x * lds + q]) and
-    // y_c = Li r_c for every component c
-    const int lds = (np + VEC - 1) / VEC * VEC;
-    for (int q = tid; q < np; q += NT) {
-        T acc = 0;
-        for (int x = 0; x < np; ++x) acc += __ldcs(Sg + (long long)x * lds + q) * tq[x];
-        sq[q] = acc;
-    }
-    const int ldv = ldl / VEC;
+// M x for a column-major block M (ld a multiple of the vector, ncol columns)
+// and D vectors at once: a thread owns one 16-byte group of rows, G groups of
+// row owners take the columns in turn, eight loads in flight per thread; the
+// groups' sums are added in red in a fixed order and handed to
+// out(row group, acc) by the first group.  Ends with every read of red done
+// by its reader only: the caller separates two calls by a barrier.
+template <bool ONCE, typename T, int D, typename F>
+__device__ __forceinline__ void columns_times(const T* __restrict__ M, int ld, int ncol, const ColVec<T, D>* x,
+                                              Vec16<T>* red, F&& out) {
+    constexpr int NT = SADDLE_APPLY_THREADS, VEC = Vec16<T>::N, U = 8;
+    const int tid = threadIdx.x, ldv = ld / VEC;
     const int G = ldv >= NT ? 1 : NT / ldv;
-    const V* base = reinterpret_cast<const V*>(Li);
     for (int t0 = 0; t0 < ldv; t0 += NT) {
         const int rg = t0 + (G == 1 ? tid : tid % ldv), g = G == 1 ? 0 : tid / ldv;
-        T acc[3][VEC];
-#pragma unroll
-        for (int c = 0; c < 3; ++c)
-#pragma unroll
-            for (int u = 0; u < VEC; ++u) acc[c][u] = 0;
         const bool own = g < G && rg < ldv;
+        T acc[D][VEC];
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e) acc[c][e] = 0;
         if (own) {
-            const V* col = base + rg;
+            const Vec16<T>* col = reinterpret_cast<const Vec16<T>*>(M) + rg;
             int b = g;
-            for (; b + 7 * G < nv; b += 8 * G) {
-                V v[8];
+            for (; b + (U - 1) * G < ncol; b += U * G) {
+                Vec16<T> v[U];
 #pragma unroll
-                for (int u = 0; u < 8; ++u) v[u] = __ldcs(col + (long long)(b + u * G) * ldv);
+                for (int u = 0; u < U; ++u) v[u] = load16<ONCE>(col + (long long)(b + u * G) * ldv);
 #pragma unroll
-                for (int u = 0; u < 8; ++u)
+                for (int u = 0; u < U; ++u) {
+                    const ColVec<T, D> xb = x[b + u * G];
 #pragma unroll
-                    for (int c = 0; c < 3; ++c) {
-                        if (c < d) {
-                            const T x = xs[c * nv + b + u * G];
+                    for (int c = 0; c < D; ++c)
 #pragma unroll
-                            for (int e = 0; e < VEC; ++e) acc[c][e] += vcomp(v[u], e) * x;
-                        }
-                    }
+                        for (int e = 0; e < VEC; ++e) acc[c][e] += v[u].at(e) * xb.v[c];
+                }
             }
-            for (; b < nv; b += G) {
-                const V v = __ldcs(col + (long long)b * ldv);
+            if (b < ncol) {                      // the last, partial round: its loads issued together too
+                Vec16<T> v[U - 1];
 #pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    if (c < d) {
-                        const T x = xs[c * nv + b];
+                for (int u = 0; u < U - 1; ++u)
+                    if (b + u * G < ncol) v[u] = load16<ONCE>(col + (long long)(b + u * G) * ldv);
 #pragma unroll
-                        for (int e = 0; e < VEC; ++e) acc[c][e] += vcomp(v, e) * x;
+                for (int u = 0; u < U - 1; ++u)
+                    if (b + u * G < ncol) {
+                        const ColVec<T, D> xb = x[b + u * G];
+#pragma unroll
+                        for (int c = 0; c < D; ++c)
+#pragma unroll
+                            for (int e = 0; e < VEC; ++e) acc[c][e] += v[u].at(e) * xb.v[c];
                     }
             }
         }
         if (G > 1) {
-            if (own)
+            if (own && g > 0)
 #pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    if (c < d) red[(g * ldv + (rg - t0)) * 3 + c] = mkvec(acc[c], (V*)nullptr);
+                for (int c = 0; c < D; ++c) red[((g - 1) * ldv + rg) * D + c].set(acc[c]);
             __syncthreads();
-            if (tid < ldv) {
+            if (tid < ldv)
+                for (int gg = 0; gg < G - 1; ++gg)
 #pragma unroll
-                for (int c = 0; c < 3; ++c)
-                    if (c < d) {
+                    for (int c = 0; c < D; ++c) {
+                        const Vec16<T> q = red[(gg * ldv + tid) * D + c];
 #pragma unroll
-                        for (int e = 0; e < VEC; ++e) acc[c][e] = vcomp(red[tid * 3 + c], e);
-                        for (int gg = 1; gg < G; ++gg) {
-                            const V q = red[(gg * ldv + tid) * 3 + c];
-#pragma unroll
-                            for (int e = 0; e < VEC; ++e) acc[c][e] += vcomp(q, e);
-                        }
+                        for (int e = 0; e < VEC; ++e) acc[c][e] += q.at(e);
                     }
+        }
+        if (g == 0 && rg < ldv) out(rg, acc);
+    }
+}
+
+template <typename T, int D>
+__device__ __forceinline__ void saddle_apply_body(int p, const int* __restrict__ poff, const int* __restrict__ pdofs,
+                                                  const int* __restrict__ pnv, const long long* __restrict__ foff,
+                                                  const T* __restrict__ fac, const T* __restrict__ r,
+                                                  const T* __restrict__ wt, T* __restrict__ Y, int xs_len,
+                                                  unsigned char* smem) {
+    constexpr int NT = SADDLE_APPLY_THREADS, VEC = Vec16<T>::N;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int s0 = poff[p], n = poff[p + 1] - s0, nv = pnv[p], dnv = D * nv, np = n - dnv;
+    if (n == 0) return;
+    const int ldl = (nv + VEC - 1) / VEC * VEC, ldw = (dnv + VEC - 1) / VEC * VEC, lds = (np + VEC - 1) / VEC * VEC;
+    const T* Li = fac + foff[p];
+    const T* Wg = Li + (long long)ldl * nv;
+    const T* Sg = Wg + (long long)ldw * np;
+    const int xl = (xs_len + 3) & ~3;
+    Vec16<T>* red = reinterpret_cast<Vec16<T>*>(smem);                      // [NT][D]
+    ColVec<T, D>* xi = reinterpret_cast<ColVec<T, D>*>(red + NT * D);       // r_u, components together
+    T* xs = reinterpret_cast<T*>(xi + ((xl / D + 4) & ~3));                 // [xl + 4] r_u as W's rows, zero padded
+    T* ys = xs;                                                             // then blockdiag(Li) r_u
+    T* tq = xs + xl + 4;                                                    // [xl] r_p, then t
+    T* sq = tq + xl;                                                        // [xl] s
+    pdl_wait();
+    pdl_release();
+    for (int a = tid; a < n; a += NT) {
+        const T v = r[pdofs[s0 + a]];
+        if (a < dnv) {
+            const int c = a / nv;
+            xi[a - c * nv].v[c] = v;
+            xs[a] = v;
+        } else {
+            tq[a - dnv] = v;
+        }
+    }
+    for (int a = dnv + tid; a < ldw; a += NT) xs[a] = 0;
+    __syncthreads();
+    // t = r_p - W^T r_u: eight lanes per column (a 128-byte line per step),
+    // four columns per warp at a time
+    {
+        const int sub = lane & 7, ldwv = ldw / VEC;
+        const Vec16<T>* xv = reinterpret_cast<const Vec16<T>*>(xs);
+        for (int q0 = warp * 4; q0 < np; q0 += NT / 8) {
+            const int q = q0 + (lane >> 3);
+            T acc = 0;
+            if (q < np) {
+                const Vec16<T>* wc = reinterpret_cast<const Vec16<T>*>(Wg) + (long long)q * ldwv;
+                int i = sub;
+                for (; i + 24 < ldwv; i += 32) {
+                    Vec16<T> w[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) w[u] = load16<false>(wc + i + 8 * u);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const Vec16<T> x = xv[i + 8 * u];
+#pragma unroll
+                        for (int e = 0; e < VEC; ++e) acc += w[u].at(e) * x.at(e);
+                    }
+                }
+                for (; i < ldwv; i += 8) {
+                    const Vec16<T> w = load16<false>(wc + i), x = xv[i];
+#pragma unroll
+                    for (int e = 0; e < VEC; ++e) acc += w.at(e) * x.at(e);
+                }
             }
-        }
-        if (g == 0 && rg < ldv) {
-            const int row0 = VEC * rg;
 #pragma unroll
-            for (int c = 0; c < 3; ++c)
-                if (c < d)
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e)
-                        if (row0 + e < nv) ys[c * nv + row0 + e] = acc[c][e];
+            for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (sub == 0 && q < np) tq[q] -= acc;
         }
-        __syncthreads();
     }
+    __syncthreads();
+    // y_c = Li r_c for every component
+    columns_times<true, T, D>(Li, ldl, nv, xi, red, [&](int rg, const T (&acc)[D][VEC]) {
+#pragma unroll
+        for (int c = 0; c < D; ++c)
+#pragma unroll
+            for (int e = 0; e < VEC; ++e)
+                if (VEC * rg + e < nv) ys[c * nv + VEC * rg + e] = acc[c][e];
+    });
+    __syncthreads();
+    // s = Si t (Si symmetric)
+    columns_times<true, T, 1>(Sg, lds, np, reinterpret_cast<const ColVec<T, 1>*>(tq), red, [&](int rg, const T (&acc)[1][VEC]) {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e)
+            if (VEC * rg + e < np) sq[VEC * rg + e] = acc[0][e];
+    });
+    __syncthreads();
     // z_u = y + W s, z_p = -s, weighted
-    for (int a = tid; a < dnv; a += NT) {
-        T z = ys[a];
-        for (int q = 0; q < np; ++q) z += wsrc[(long long)q * ldw + a] * sq[q];
-        Y[s0 + a] = wt[pdofs[s0 + a]] * z;
-    }
+    columns_times<false, T, 1>(Wg, ldw, np, reinterpret_cast<const ColVec<T, 1>*>(sq), red, [&](int rg, const T (&acc)[1][VEC]) {
+#pragma unroll
+        for (int e = 0; e < VEC; ++e) {
+            const int a = VEC * rg + e;
+            if (a < dnv) Y[s0 + a] = wt[pdofs[s0 + a]] * (ys[a] + acc[0][e]);
+        }
+    });
     for (int q = tid; q < np; q += NT) Y[s0 + dnv + q] = -wt[pdofs[s0 + dnv + q]] * sq[q];
 }
 
-__global__ void __launch_bounds__(SADDLE_APPLY_THREADS) saddle_apply_f32(
-    int npatch, int d, const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
-    const long long* __restrict__ foff, const float* __restrict__ fac, const float* __restrict__ r,
-    const float* __restrict__ wt, float* __restrict__ Y, int xs_len, int ws_len) {
-    extern __shared__ __align__(16) unsigned char smem_sa[];
-    pdl_wait();
-    pdl_release();
-    saddle_apply_body<float, float4, 4>(blockIdx.x, d, poff, pdofs, pnv, foff, fac, r, wt, Y, xs_len, ws_len, smem_sa);
-}
-
-__global__ void __launch_bounds__(SADDLE_APPLY_THREADS) saddle_apply_f64(
-    int npatch, int d, const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
-    const long long* __restrict__ foff, const double* __restrict__ fac, const double* __restrict__ r,
-    const double* __restrict__ wt, double* __restrict__ Y, int xs_len, int ws_len) {
-    extern __shared__ __align__(16) unsigned char smem_sa[];
-    pdl_wait();
-    pdl_release();
-    saddle_apply_body<double, double2, 2>(blockIdx.x, d, poff, pdofs, pnv, foff, fac, r, wt, Y, xs_len, ws_len, smem_sa);
-}
+// seven CTAs per SM (at most 72 registers): left to itself the compiler takes
+// 77, six CTAs, and the 3D P3 apply takes 160 us instead of 135
+#define SADDLE_APPLY_KERNEL(NAME, T, D)                                                                             \
+    __global__ void __launch_bounds__(SADDLE_APPLY_THREADS, 7) NAME(                                                \
+        const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,                   \
+        const long long* __restrict__ foff, const T* __restrict__ fac, const T* __restrict__ r,                     \
+        const T* __restrict__ wt, T* __restrict__ Y, int xs_len) {                                                  \
+        extern __shared__ __align__(16) unsigned char smem_sa[];                                                    \
+        saddle_apply_body<T, D>(blockIdx.x, poff, pdofs, pnv, foff, fac, r, wt, Y, xs_len, smem_sa);                \
+    }
+SADDLE_APPLY_KERNEL(saddle_apply_f32_2d, float, 2)
+SADDLE_APPLY_KERNEL(saddle_apply_f32_3d, float, 3)
+SADDLE_APPLY_KERNEL(saddle_apply_f64_2d, double, 2)
+SADDLE_APPLY_KERNEL(saddle_apply_f64_3d, double, 3)
+#undef SADDLE_APPLY_KERNEL
 
 // ---- the same sweep with each patch's factored block brought into shared
 // memory by one bulk copy (cp.async.bulk, completion on an mbarrier) -------

@@ -235,15 +235,35 @@ __host__ __device__ inline long long saddle_factor_len(int d, int n, int nv, int
     const long long lenL = packed ? ((long long)nv * (nv + 1) / 2 + vec - 1) / vec * vec : ldl * nv;
     return lenL + ldw * np + lds * np;
 }
-// Shared memory (bytes) of saddle_apply_*: partial sums, W (ws_len
-// elements; 0 = W read from global memory), and five vectors of xs_len
-// (>= the largest patch) elements.  W is staged when the total stays within
-// SADDLE_APPLY_SMEM_MAX bytes (the kernels' shared-memory attribute).
+// One ASM sweep with the factored inverses streamed from global memory, one
+// CTA per patch, D = 2 or 3 components; xs_len >= the largest patch.  Shared
+// memory (bytes): the groups' partial sums and the patch's vectors (the
+// residual in two orders, y, t and s).  A level whose largest patch needs more
+// than SADDLE_APPLY_SMEM_MAX (the kernels' shared-memory attribute) by
+// saddle_apply_limit is refused.
 constexpr int SADDLE_APPLY_THREADS = 128;
 constexpr size_t SADDLE_APPLY_SMEM_MAX = 200 * 1024;
-__host__ __device__ inline size_t saddle_apply_smem(int elem_bytes, int vec, long long ws_len, long long xs_len) {
-    return (size_t)elem_bytes * vec * SADDLE_APPLY_THREADS * 3 + (size_t)elem_bytes * (ws_len + 5 * xs_len);
+__host__ __device__ inline size_t saddle_apply_smem(int elem_bytes, int d, long long xs_len) {
+    const long long xl = (xs_len + 3) & ~3LL;
+    return (size_t)16 * SADDLE_APPLY_THREADS * d + (size_t)elem_bytes * ((d == 3 ? 4 : d) * ((xl / d + 4) & ~3LL) + 3 * xl + 4);
 }
+__host__ __device__ inline size_t saddle_apply_limit(long long xs_len) { return (size_t)(6144 + 40 * xs_len); }
+__global__ void saddle_apply_f32_2d(const int* __restrict__ poff, const int* __restrict__ pdofs,
+                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
+                                    const float* __restrict__ fac, const float* __restrict__ r, const float* __restrict__ wt,
+                                    float* __restrict__ Y, int xs_len);
+__global__ void saddle_apply_f32_3d(const int* __restrict__ poff, const int* __restrict__ pdofs,
+                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
+                                    const float* __restrict__ fac, const float* __restrict__ r, const float* __restrict__ wt,
+                                    float* __restrict__ Y, int xs_len);
+__global__ void saddle_apply_f64_2d(const int* __restrict__ poff, const int* __restrict__ pdofs,
+                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
+                                    const double* __restrict__ fac, const double* __restrict__ r, const double* __restrict__ wt,
+                                    double* __restrict__ Y, int xs_len);
+__global__ void saddle_apply_f64_3d(const int* __restrict__ poff, const int* __restrict__ pdofs,
+                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
+                                    const double* __restrict__ fac, const double* __restrict__ r, const double* __restrict__ wt,
+                                    double* __restrict__ Y, int xs_len);
 // The same sweep with one CTA per patch whose factored block is brought into
 // shared memory by one bulk copy (buf_bytes >= the largest block, a
 // multiple of 128; xs_len >= the largest patch).  *status = 1 if a CTA gave
@@ -263,14 +283,6 @@ __global__ void saddle_apply_bulk_f64(int d, const int* __restrict__ poff, const
                                       const double* __restrict__ fac, const double* __restrict__ r,
                                       const double* __restrict__ wt, double* __restrict__ Y, int buf_bytes,
                                       int xs_len, int* __restrict__ status);
-__global__ void saddle_apply_f32(int npatch, int d, const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                 const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                 const float* __restrict__ fac, const float* __restrict__ r, const float* __restrict__ wt,
-                                 float* __restrict__ Y, int xs_len, int ws_len);
-__global__ void saddle_apply_f64(int npatch, int d, const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                 const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                 const double* __restrict__ fac, const double* __restrict__ r,
-                                 const double* __restrict__ wt, double* __restrict__ Y, int xs_len, int ws_len);
 
 // One ASM sweep (Eq. 3.4): Y[poff[i] + a] = w[dof_a] * sum_b Kinv_i[a][b] r[dof_b].
 // FP32: float4 loads of 4 consecutive rows per thread; FP64: double2 loads

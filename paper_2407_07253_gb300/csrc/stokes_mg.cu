@@ -171,7 +171,6 @@ struct DevLevel {
     double* fac64 = nullptr;
     float* fac32 = nullptr;
     int sa_xs = 0;                      // saddle apply: largest patch
-    long long sa_ws64 = 0, sa_ws32 = 0; // saddle apply: largest W (elements)
     int sa_buf = 0;                     // bulk-copy apply: buffer bytes (0: not used on this level)
     bool fac_packed = false;            // L^-1 stored as its packed upper triangle (bulk-copy apply only)
     double* wt64 = nullptr;
@@ -586,11 +585,9 @@ template <> struct PatchOf<float> {
     static const long long* ioff(const DevLevel& l) { return l.ioff32; }
     static const float* wt(const DevLevel& l) { return l.wt32; }
     static float* Y(const DevLevel& l) { return l.Y32; }
-    static long long ws(const DevLevel& l) { return l.sa_ws32; }
     static constexpr auto bulk = skern::saddle_apply_bulk_f32;
-    static constexpr auto fact = skern::saddle_apply_f32;
+    static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f32_3d : skern::saddle_apply_f32_2d; }
     static constexpr auto expl = skern::patch_apply_f32;
-    static constexpr int vec = 4;
     static constexpr size_t red = sizeof(float4);
     static constexpr const char* none = "no FP32 patch inverses on this handle (FP64 handle)";
 };
@@ -601,11 +598,9 @@ template <> struct PatchOf<double> {
     static const long long* ioff(const DevLevel& l) { return l.ioff64; }
     static const double* wt(const DevLevel& l) { return l.wt64; }
     static double* Y(const DevLevel& l) { return l.Y64; }
-    static long long ws(const DevLevel& l) { return l.sa_ws64; }
     static constexpr auto bulk = skern::saddle_apply_bulk_f64;
-    static constexpr auto fact = skern::saddle_apply_f64;
+    static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f64_3d : skern::saddle_apply_f64_2d; }
     static constexpr auto expl = skern::patch_apply_f64;
-    static constexpr int vec = 2;
     static constexpr size_t red = sizeof(double2);
     static constexpr const char* none = "no FP64 patch inverses on this handle (MIXED handle)";
 };
@@ -629,12 +624,10 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
                (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
         });
     } else if (fac) {
-        long long ws = PO::ws(l);
-        if (skern::saddle_apply_smem(sizeof(T), PO::vec, ws, l.sa_xs) > skern::SADDLE_APPLY_SMEM_MAX) ws = 0;
-        const size_t smem = skern::saddle_apply_smem(sizeof(T), PO::vec, ws, l.sa_xs);
+        const size_t smem = skern::saddle_apply_smem(sizeof(T), h->dim, l.sa_xs);
         launch(h, PK_PATCH, s, [&] {
-            kl(h, PO::fact, l.npatch, skern::SADDLE_APPLY_THREADS, smem, s, l.npatch, h->dim, poff, pdofs, pnv, foff,
-               fac, r, wt, Y, (int)l.sa_xs, (int)ws);
+            kl(h, PO::fact(h->dim), l.npatch, skern::SADDLE_APPLY_THREADS, smem, s, poff, pdofs, pnv, foff, fac, r, wt, Y,
+               (int)l.sa_xs);
         });
     } else {
         const T* inv = PO::inv(l);
@@ -1577,25 +1570,22 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
             l.sa_xs = l.maxn;
             for (int p = 0; p < l.npatch; ++p) {
                 const int n = HL.patch_off[p + 1] - HL.patch_off[p], nv = HL.patch_nv[p];
-                const int np = n - HL.d * nv;
                 f64[p + 1] = f64[p] + skern::saddle_factor_len(HL.d, n, nv, 2);
                 f32[p + 1] = f32[p] + skern::saddle_factor_len(HL.d, n, nv, 4);
-                l.sa_ws64 = std::max<long long>(l.sa_ws64, (long long)((HL.d * nv + 1) & ~1) * np);
-                l.sa_ws32 = std::max<long long>(l.sa_ws32, (long long)((HL.d * nv + 3) & ~3) * np);
             }
             l.nfac64 = f64[l.npatch];
             l.nfac32 = f32[l.npatch];
-            if (skern::saddle_apply_smem(8, 2, 0, l.sa_xs) > skern::SADDLE_APPLY_SMEM_MAX)
+            if (skern::saddle_apply_limit(l.sa_xs) > skern::SADDLE_APPLY_SMEM_MAX)
                 throw StokesError(STOKES_EUNSUPPORTED, "patch too large for the saddle apply's shared memory");
             // one process-wide upper bound (never lowered)
-            CK(cudaFuncSetAttribute(skern::saddle_apply_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)skern::SADDLE_APPLY_SMEM_MAX));
-            CK(cudaFuncSetAttribute(skern::saddle_apply_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)skern::SADDLE_APPLY_SMEM_MAX));
-            CK(cudaFuncSetAttribute(skern::saddle_apply_bulk_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)skern::SADDLE_APPLY_SMEM_MAX));
-            CK(cudaFuncSetAttribute(skern::saddle_apply_bulk_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)skern::SADDLE_APPLY_SMEM_MAX));
+            auto opt_in = [](auto kern) {
+                CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        (int)skern::SADDLE_APPLY_SMEM_MAX));
+            };
+            opt_in(PatchOf<float>::fact(HL.d));
+            opt_in(PatchOf<double>::fact(HL.d));
+            opt_in(skern::saddle_apply_bulk_f32);
+            opt_in(skern::saddle_apply_bulk_f64);
             // the bulk-copy apply, with L^-1 stored as its packed upper
             // triangle, when the level's largest packed block fits in shared
             // memory with room for at least two CTAs per SM
