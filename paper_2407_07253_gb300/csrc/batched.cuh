@@ -84,13 +84,19 @@ void spmm64(int mode, int nr, int m, const int* rp, const int* ci, const double*
             const double* B, cudaStream_t s);
 // doubles of the partial-sum workspace of col_dots at width m
 size_t col_partial_doubles(int m);
-// out[i][c] (+)= sum_r V_i[r][c] W[r][c] for i < nb (<= 32), basis vectors
+// out[i][c] = sum_r V_i[r][c] W[r][c] for i < nb (<= 32), basis vectors
 // ldv doubles apart; sqrt_out takes the square root (column norms with
 // V = W); deterministic (fixed-order two-stage reduction)
 void col_dots(int n, int m, int nb, const double* V, long long ldv, const double* W, double* partial, double* out,
-              int sqrt_out, int add, cudaStream_t s);
-// W[r][c] -= sum_{i < nb} H[i][c] V_i[r][c]
-void col_update(int n, int m, int nb, const double* V, long long ldv, const double* H, double* W, cudaStream_t s);
+              int sqrt_out, cudaStream_t s);
+// W[r][c] -= sum_{i < nb} H[i][c] V_i[r][c]; of the new W, out[i][c] as
+// col_dots and out[nb][c] = sum_r W[r][c]^2; acc[i][c] += out[i][c] (i < nb)
+void col_update_dots(int n, int m, int nb, const double* V, long long ldv, const double* H, double* W, double* partial,
+                     double* out, double* acc, cudaStream_t s);
+// Vout = (W - V H) / nu per column, hn[c] = nu = sqrt(H[nb][c] - sum_{i < nb} H[i][c]^2)
+// with H[nb][c] = |W_c|^2 (0 where nu == 0)
+void col_normalise(int n, int m, int nb, const double* V, long long ldv, const double* H, const double* W, double* Vout,
+                   double* hn, cudaStream_t s);
 // Vout = W / h[c] per column (0 where h[c] == 0)
 void col_scale(int n, int m, const double* W, const double* h, double* Vout, cudaStream_t s);
 // per column: Hessenberg column j, Givens rotations, g, |residual estimate|;

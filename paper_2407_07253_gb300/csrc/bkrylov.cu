@@ -4,14 +4,16 @@
 // run, and every column is an independent FGMRES (Sec. 4) in lockstep.
 #include "batched.cuh"
 
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 namespace sbat {
 
 namespace {
 
 constexpr int NBMAX = 32;           // basis vectors in one multi-dot (restart + 1 <= 32)
-constexpr int DOT_CTAS = 152 * 4;
+constexpr int DOT_CTAS = 152 * 4;   // the most CTAs of a multi-dot
 
 // Y = A X (MODE 0) or Y = B - A X (MODE 2), FP64; M / 2 lanes per row, one
 // double2 of right-hand sides per lane.
@@ -46,59 +48,168 @@ __global__ void __launch_bounds__(256) k_spmm64(int nr, int m, const int* __rest
     }
 }
 
-// partial[blk][i][c] = sum over the CTA's rows of V_i[r][c] W[r][c], i < nb:
-// W is read once, every basis vector once; 256 / M row lanes per CTA.
-template <int M>
-__global__ void __launch_bounds__(256) k_col_dots(int n, int nb, const double* __restrict__ V, long long ldv,
-                                                  const double* __restrict__ W, double* __restrict__ partial) {
-    constexpr int RL = 256 / M;
-    __shared__ double red[RL][M];
-    const int c = threadIdx.x % M, rl = threadIdx.x / M;
-    double acc[NBMAX];
+// ---- classical Gram-Schmidt twice, per column ---------------------------
+// Three passes over the basis for the new vector w (the single-vector cgs2's
+// fusion): h1 = V^T w;  w <- w - V h1, h2 = V^T w, |w|^2;  w <- (w - V h2) / nu.
+// The FP64 pipe bounds them (2 FMA lanes per SM and clock: 4 FMAs per basis
+// entry take 1.8 times what reading it three times takes), so the
+// accumulators are unrolled to NB, the smallest class (with_nb) that holds nb:
+// unrolled to 32 for every nb, the dots of 32 columns on 128 x 128 P3 took
+// 838 us, now 311 us at nb = 9 to 12 (86% of the FP64 peak's 268 us at 12);
+// the whole orthogonalisation of a step went from 2.5 to 1.0 ms on average.
+// A thread keeps one column c for all its rows (m divides the CTA's 256 threads).
+template <int NB>
+constexpr int dot_ctas_per_sm() { return NB <= 8 ? 4 : 2; }
+
+// The CTA's sums of acc[0 .. na) over its row lanes -> partial[blk][i][c] (and
+// of extra as i = na with EXTRA), 16 accumulators at a time through shared memory.
+template <bool EXTRA, int NB>
+__device__ __forceinline__ void col_block_partials(int m, int na, const double (&acc)[NB], double extra,
+                                                   double* __restrict__ partial) {
+    constexpr int NA = NB + (EXTRA ? 1 : 0), CH = NA < 16 ? NA : 16;
+    const int mc = na + (EXTRA ? 1 : 0);
+    __shared__ double red[CH][256];
+    const int rl = 256 / m;
 #pragma unroll
-    for (int i = 0; i < NBMAX; ++i) acc[i] = 0.0;
-    for (long long r = (long long)blockIdx.x * RL + rl; r < n; r += (long long)gridDim.x * RL) {
-        const double w = W[r * M + c];
+    for (int i0 = 0; i0 < NA; i0 += CH) {
+        if (i0 >= mc) break;
 #pragma unroll
-        for (int i = 0; i < NBMAX; ++i)
-            if (i < nb) acc[i] = fma(V[i * ldv + r * M + c], w, acc[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < NBMAX; ++i) {
-        if (i < nb) {                       // nb is uniform over the CTA
-            red[rl][c] = acc[i];
-            __syncthreads();
-            if (rl == 0) {
-                double s = 0.0;
-                for (int q = 0; q < RL; ++q) s += red[q][c];
-                partial[((long long)blockIdx.x * NBMAX + i) * M + c] = s;
+        for (int q = 0; q < CH; ++q)
+            if (i0 + q < NA) {
+                double v = acc[i0 + q < NB ? i0 + q : 0];
+                if (EXTRA && i0 + q == na) v = extra;
+                red[q][threadIdx.x] = v;
             }
-            __syncthreads();
+        __syncthreads();
+        for (int t = threadIdx.x; t < CH * m; t += 256) {
+            const int q = t / m, c = t - q * m;
+            if (i0 + q < mc) {
+                double s = 0.0;
+                for (int x = 0; x < rl; ++x) s += red[q][x * m + c];
+                partial[((long long)blockIdx.x * (NBMAX + 1) + i0 + q) * m + c] = s;
+            }
         }
+        __syncthreads();
     }
 }
 
-// out[i][c] = sum_blk partial[blk][i][c] in block order (deterministic);
-// sqrt_out: out = sqrt(out) (column norms); add: out += that sum
-__global__ void k_col_reduce(int nblk, int nb, int m, const double* __restrict__ partial, double* __restrict__ out,
-                             int sqrt_out, int add) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nb * m) return;
-    const int i = t / m, c = t - i * m;
-    double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += partial[((long long)b * NBMAX + i) * m + c];
-    if (sqrt_out) s = sqrt(s);
-    out[t] = add ? out[t] + s : s;
+// partial[blk][i][c] = sum over the CTA's rows of V_i[r][c] W[r][c], i < nb
+template <int NB>
+__global__ void __launch_bounds__(256, dot_ctas_per_sm<NB>()) k_col_dots(int n, int m, int nb,
+                                                                         const double* __restrict__ V, long long ldv,
+                                                                         const double* __restrict__ W,
+                                                                         double* __restrict__ partial) {
+    double acc[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) acc[i] = 0.0;
+    const long long nm = (long long)n * m;
+    for (long long t = blockIdx.x * 256LL + threadIdx.x; t < nm; t += gridDim.x * 256LL) {
+        const double w = W[t];
+#pragma unroll
+        for (int i = 0; i < NB; ++i)
+            if (i < nb) acc[i] = fma(V[i * ldv + t], w, acc[i]);
+    }
+    col_block_partials<false>(m, nb, acc, 0.0, partial);
 }
 
-// W[r][c] -= sum_{i < nb} H[i][c] V_i[r][c]
-__global__ void k_col_update(long long nm, int m, int nb, const double* __restrict__ V, long long ldv,
-                             const double* __restrict__ H, double* __restrict__ W) {
-    for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nm; t += (long long)gridDim.x * blockDim.x) {
-        const int c = (int)(t % m);
+// W <- W - V H, then the dots of the new W with the basis (i < nb) and itself (i = nb)
+template <int NB>
+__global__ void __launch_bounds__(256, dot_ctas_per_sm<NB>()) k_col_update_dots(int n, int m, int nb,
+                                                                                const double* __restrict__ V, long long ldv,
+                                                                                const double* __restrict__ H,
+                                                                                double* __restrict__ W,
+                                                                                double* __restrict__ partial) {
+    extern __shared__ double hs[];                // [nb][m]
+    for (int t = threadIdx.x; t < nb * m; t += 256) hs[t] = H[t];
+    __syncthreads();
+    double acc[NB];
+#pragma unroll
+    for (int i = 0; i < NB; ++i) acc[i] = 0.0;
+    const int c = threadIdx.x % m;
+    const long long nm = (long long)n * m;
+    double nrm = 0.0;
+    for (long long t = blockIdx.x * 256LL + threadIdx.x; t < nm; t += gridDim.x * 256LL) {
+        double w = W[t];
+        if constexpr (NB <= 16) {
+            // V's entries stay in registers between the two uses
+            double v[NB];
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (i < nb) v[i] = V[i * ldv + t];
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (i < nb) w = fma(-hs[i * m + c], v[i], w);
+            W[t] = w;
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (i < nb) acc[i] = fma(v[i], w, acc[i]);
+        } else {
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (i < nb) w = fma(-hs[i * m + c], V[i * ldv + t], w);
+            W[t] = w;
+#pragma unroll
+            for (int i = 0; i < NB; ++i)
+                if (i < nb) acc[i] = fma(V[i * ldv + t], w, acc[i]);
+        }
+        nrm = fma(w, w, nrm);
+    }
+    col_block_partials<true>(m, nb, acc, nrm, partial);   // the norm behind the nb dots
+}
+
+// out[i][c] = sum_blk partial[blk][i][c] (fixed order: 1024 / m interleaved
+// block sums, then those in turn), acc[i][c] += out[i][c] for i < nacc;
+// sqrt_out: out = sqrt(out) (column norms).  One CTA per i.
+__global__ void __launch_bounds__(1024) k_col_reduce(int nblk, int m, const double* __restrict__ partial,
+                                                     double* __restrict__ out, double* __restrict__ acc, int nacc,
+                                                     int sqrt_out) {
+    __shared__ double red[1024];
+    const int i = blockIdx.x, c = threadIdx.x % m, g = threadIdx.x / m, G = 1024 / m;
+    double s = 0.0;
+#pragma unroll 8
+    for (int b = g; b < nblk; b += G) s += partial[((long long)b * (NBMAX + 1) + i) * m + c];
+    red[threadIdx.x] = s;
+    __syncthreads();
+    if (g > 0) return;
+    for (int q = 1; q < G; ++q) s += red[q * m + c];
+    if (sqrt_out) s = sqrt(s);
+    out[i * m + c] = s;
+    if (i < nacc) acc[i * m + c] += s;
+}
+
+// Vout = (W - V H) / nu, hn[c] = nu = sqrt(max(H[nb][c] - sum_i H[i][c]^2, 0))
+// (H[nb] = |W|^2 before the update; Pythagoras: the second pass's H is O(eps)
+// relative to W, so the difference loses no accuracy); 0 where nu = 0 (a
+// column already exact, or padding).
+__global__ void __launch_bounds__(256) k_col_normalise(int n, int m, int nb, const double* __restrict__ V, long long ldv,
+                                                       const double* __restrict__ H, const double* __restrict__ W,
+                                                       double* __restrict__ Vout, double* __restrict__ hn) {
+    extern __shared__ double hs[];                // [nb][m], then [m] 1 / nu
+    for (int t = threadIdx.x; t < nb * m; t += 256) hs[t] = H[t];
+    __syncthreads();
+    if (threadIdx.x < m) {
+        double q = H[nb * m + threadIdx.x];
+        for (int i = 0; i < nb; ++i) q = fma(-hs[i * m + threadIdx.x], hs[i * m + threadIdx.x], q);
+        const double nu = sqrt(q > 0.0 ? q : 0.0);
+        hs[nb * m + threadIdx.x] = nu > 0.0 ? 1.0 / nu : 0.0;
+        if (blockIdx.x == 0) hn[threadIdx.x] = nu;
+    }
+    __syncthreads();
+    const int c = threadIdx.x % m;
+    const double inv = hs[nb * m + c];
+    const long long nm = (long long)n * m;
+    for (long long t = blockIdx.x * 256LL + threadIdx.x; t < nm; t += gridDim.x * 256LL) {
         double s = W[t];
-        for (int i = 0; i < nb; ++i) s = fma(-H[i * m + c], V[i * ldv + t], s);
-        W[t] = s;
+        int i = 0;
+        for (; i + 4 <= nb; i += 4) {
+            double v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = V[(i + u) * ldv + t];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s = fma(-hs[(i + u) * m + c], v[u], s);
+        }
+        for (; i < nb; ++i) s = fma(-hs[i * m + c], V[i * ldv + t], s);
+        Vout[t] = inv > 0.0 ? s * inv : 0.0;
     }
 }
 
@@ -209,16 +320,24 @@ inline int grid_of(long long n, int block = 256) {
     return (int)(g < 1 ? 1 : g);
 }
 
-template <int M>
-void col_dots_m(int n, int nb, const double* V, long long ldv, const double* W, double* partial, double* out,
-                int sqrt_out, int add, cudaStream_t s) {
-    k_col_dots<M><<<DOT_CTAS, 256, 0, s>>>(n, nb, V, ldv, W, partial);
-    k_col_reduce<<<(nb * M + 255) / 256, 256, 0, s>>>(DOT_CTAS, nb, M, partial, out, sqrt_out, add);
+// calls f(integral constant NB) with the smallest unrolling that holds nb
+template <typename F>
+void with_nb(int nb, F&& f) {
+    if (nb <= 2) f(std::integral_constant<int, 2>{});
+    else if (nb <= 4) f(std::integral_constant<int, 4>{});
+    else if (nb <= 6) f(std::integral_constant<int, 6>{});
+    else if (nb <= 8) f(std::integral_constant<int, 8>{});
+    else if (nb <= 12) f(std::integral_constant<int, 12>{});
+    else if (nb <= 16) f(std::integral_constant<int, 16>{});
+    else if (nb <= 24) f(std::integral_constant<int, 24>{});
+    else f(std::integral_constant<int, 32>{});
 }
+template <int NB>
+int dot_grid() { return 152 * dot_ctas_per_sm<NB>(); }
 
 }  // namespace
 
-size_t col_partial_doubles(int m) { return (size_t)DOT_CTAS * NBMAX * m; }
+size_t col_partial_doubles(int m) { return (size_t)DOT_CTAS * (NBMAX + 1) * m; }
 
 void spmm64(int mode, int nr, int m, const int* rp, const int* ci, const double* av, const double* X, double* Y,
             const double* B, cudaStream_t s) {
@@ -231,18 +350,27 @@ void spmm64(int mode, int nr, int m, const int* rp, const int* ci, const double*
 }
 
 void col_dots(int n, int m, int nb, const double* V, long long ldv, const double* W, double* partial, double* out,
-              int sqrt_out, int add, cudaStream_t s) {
-    switch (m) {
-        case 8: col_dots_m<8>(n, nb, V, ldv, W, partial, out, sqrt_out, add, s); break;
-        case 16: col_dots_m<16>(n, nb, V, ldv, W, partial, out, sqrt_out, add, s); break;
-        case 32: col_dots_m<32>(n, nb, V, ldv, W, partial, out, sqrt_out, add, s); break;
-        default: col_dots_m<64>(n, nb, V, ldv, W, partial, out, sqrt_out, add, s); break;
-    }
+              int sqrt_out, cudaStream_t s) {
+    with_nb(nb, [&](auto nbc) {
+        constexpr int NB = decltype(nbc)::value;
+        k_col_dots<NB><<<dot_grid<NB>(), 256, 0, s>>>(n, m, nb, V, ldv, W, partial);
+        k_col_reduce<<<nb, 1024, 0, s>>>(dot_grid<NB>(), m, partial, out, nullptr, 0, sqrt_out);
+    });
 }
 
-void col_update(int n, int m, int nb, const double* V, long long ldv, const double* H, double* W, cudaStream_t s) {
-    const long long nm = (long long)n * m;
-    k_col_update<<<grid_of(nm), 256, 0, s>>>(nm, m, nb, V, ldv, H, W);
+void col_update_dots(int n, int m, int nb, const double* V, long long ldv, const double* H, double* W, double* partial,
+                     double* out, double* acc, cudaStream_t s) {
+    with_nb(nb, [&](auto nbc) {
+        constexpr int NB = decltype(nbc)::value;
+        k_col_update_dots<NB><<<dot_grid<NB>(), 256, sizeof(double) * nb * m, s>>>(n, m, nb, V, ldv, H, W, partial);
+        k_col_reduce<<<nb + 1, 1024, 0, s>>>(dot_grid<NB>(), m, partial, out, acc, nb, 0);
+    });
+}
+
+void col_normalise(int n, int m, int nb, const double* V, long long ldv, const double* H, const double* W, double* Vout,
+                   double* hn, cudaStream_t s) {
+    const int grid = std::min(grid_of((long long)n * m), 152 * 8);
+    k_col_normalise<<<grid, 256, sizeof(double) * (nb + 1) * m, s>>>(n, m, nb, V, ldv, H, W, Vout, hn);
 }
 
 void col_scale(int n, int m, const double* W, const double* h, double* Vout, cudaStream_t s) {

@@ -2821,7 +2821,7 @@ void ensure_bkrylov(stokes_mg* h, int m) {
     K.X = halloc<double>(h, nm);
     K.partial = halloc<double>(h, sbat::col_partial_doubles(m));
     K.hcol = halloc<double>(h, (size_t)32 * m);
-    K.hcol2 = halloc<double>(h, (size_t)32 * m);
+    K.hcol2 = halloc<double>(h, (size_t)33 * m);
     K.hn = halloc<double>(h, m);
     K.Hc = halloc<double>(h, (size_t)m * ldh * ldh);
     K.cs = halloc<double>(h, (size_t)m * ldh);
@@ -2852,7 +2852,7 @@ int fgmres_batched(stokes_mg* h, int nrhs, int mode, const double* B_dev, double
     const long long nm = (long long)n * m;
     launch(h, -1, s, [&] { sbat::pack64(n, nrhs, m, B_dev, K.B, s); });
     CK(cudaMemsetAsync(K.X, 0, sizeof(double) * nm, s));
-    launch(h, -1, s, [&] { sbat::col_dots(n, m, 1, K.B, 0, K.B, K.partial, K.beta0, 1, 0, s); });
+    launch(h, -1, s, [&] { sbat::col_dots(n, m, 1, K.B, 0, K.B, K.partial, K.beta0, 1, s); });
     CK(cudaMemcpyAsync(K.host, K.beta0, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
     std::vector<double> beta0(K.host, K.host + m), res(m, 0.0);
@@ -2876,14 +2876,13 @@ int fgmres_batched(stokes_mg* h, int nrhs, int mode, const double* B_dev, double
             double* Zj = K.Z + (long long)j * nm;
             batched_precond(h, mode, Vj, Zj, s);
             launch(h, PK_SPMV, s, [&] { sbat::spmm64(0, n, m, l0.K.rp, l0.K.ci, l0.K.v64, Zj, K.W, nullptr, s); });
-            // CGS2
-            launch(h, -1, s, [&] { sbat::col_dots(n, m, j + 1, K.V, nm, K.W, K.partial, K.hcol, 0, 0, s); });
-            launch(h, -1, s, [&] { sbat::col_update(n, m, j + 1, K.V, nm, K.hcol, K.W, s); });
-            launch(h, -1, s, [&] { sbat::col_dots(n, m, j + 1, K.V, nm, K.W, K.partial, K.hcol2, 0, 0, s); });
-            launch(h, -1, s, [&] { sbat::col_update(n, m, j + 1, K.V, nm, K.hcol2, K.W, s); });
-            axpby_l<double>(h, (j + 1) * m, 1.0, K.hcol2, 1.0, K.hcol, s);
-            launch(h, -1, s, [&] { sbat::col_dots(n, m, 1, K.W, 0, K.W, K.partial, K.hn, 1, 0, s); });
-            launch(h, -1, s, [&] { sbat::col_scale(n, m, K.W, K.hn, K.V + (long long)(j + 1) * nm, s); });
+            // CGS2, three passes over the basis
+            launch(h, -1, s, [&] { sbat::col_dots(n, m, j + 1, K.V, nm, K.W, K.partial, K.hcol, 0, s); });
+            launch(h, -1, s, [&] { sbat::col_update_dots(n, m, j + 1, K.V, nm, K.hcol, K.W, K.partial, K.hcol2, K.hcol, s); });
+            launch(h, -1, s, [&] {
+                sbat::col_normalise(n, m, j + 1, K.V, nm, K.hcol2, K.W, K.V + (long long)(j + 1) * nm, K.hn, s);
+            });
+            h->launches += 2;              // the two reductions
             launch(h, -1, s, [&] { sbat::col_givens(j, m, ldh, K.Hc, K.hcol, K.hn, K.cs, K.sn, K.g, K.resid, s); });
             CK(cudaMemcpyAsync(K.host, K.resid, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
@@ -2900,7 +2899,7 @@ int fgmres_batched(stokes_mg* h, int nrhs, int mode, const double* B_dev, double
         if (converged) break;
         // restart: the true residual of every column
         launch(h, PK_SPMV, s, [&] { sbat::spmm64(2, n, m, l0.K.rp, l0.K.ci, l0.K.v64, K.X, K.R, K.B, s); });
-        launch(h, -1, s, [&] { sbat::col_dots(n, m, 1, K.R, 0, K.R, K.partial, K.beta, 1, 0, s); });
+        launch(h, -1, s, [&] { sbat::col_dots(n, m, 1, K.R, 0, K.R, K.partial, K.beta, 1, s); });
         CK(cudaMemcpyAsync(K.host, K.beta, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
         res.assign(K.host, K.host + m);
