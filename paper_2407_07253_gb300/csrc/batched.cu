@@ -136,7 +136,7 @@ __global__ void __launch_bounds__(512, 1) k_patch_gemm(int npatch, const int* __
                                                     const int* __restrict__ poff,
                                                     const int* __restrict__ pdofs, const long long* __restrict__ ioff,
                                                     const float* __restrict__ inv, const float* __restrict__ X,
-                                                    const float* __restrict__ wt, float* __restrict__ Yb) {
+                                                    float* __restrict__ Yb) {
     extern __shared__ __align__(128) float smem_pg[];
     constexpr int NT = M / 8, Q = M / 4;
     const int p = plist ? __ldg(plist + blockIdx.x) : (int)blockIdx.x;     // one CTA per listed patch
@@ -210,15 +210,12 @@ __global__ void __launch_bounds__(512, 1) k_patch_gemm(int npatch, const int* __
     }
     __syncthreads();
 
-    float d[NT][4], w0 = 0.f, w1 = 0.f;
+    float d[NT][4];
     int rb = warp, gi = 0;
     for (int it = 0; it < items; ++it) {
         if (gi == 0) {
 #pragma unroll
             for (int q = 0; q < NT; ++q) d[q][0] = d[q][1] = d[q][2] = d[q][3] = 0.f;
-            const int r0 = rb * 16 + g, r1 = r0 + 8;     // weights, needed at the end of the row block
-            w0 = r0 < n ? __ldg(wt + __ldg(pdofs + s + r0)) : 0.f;
-            w1 = r1 < n ? __ldg(wt + __ldg(pdofs + s + r1)) : 0.f;
         }
         issue();
         cp_async_wait<ST - 1>();
@@ -261,9 +258,9 @@ __global__ void __launch_bounds__(512, 1) k_patch_gemm(int npatch, const int* __
             for (int q = 0; q < NT; ++q) {
                 const int c = q * 8 + 2 * t;
                 if (r0 < n)
-                    *reinterpret_cast<float2*>(Yb + (long long)(s + r0) * M + c) = make_float2(w0 * d[q][0], w0 * d[q][1]);
+                    *reinterpret_cast<float2*>(Yb + (long long)(s + r0) * M + c) = make_float2(d[q][0], d[q][1]);
                 if (r1 < n)
-                    *reinterpret_cast<float2*>(Yb + (long long)(s + r1) * M + c) = make_float2(w1 * d[q][2], w1 * d[q][3]);
+                    *reinterpret_cast<float2*>(Yb + (long long)(s + r1) * M + c) = make_float2(d[q][2], d[q][3]);
             }
             gi = 0;
             rb += nw;
@@ -286,13 +283,13 @@ __global__ void __launch_bounds__(512, 1) k_patch_gemm(int npatch, const int* __
 //                    core matrices, no swizzle), then fenced to the async
 //                    proxy; each warp takes every G-th stage, so up to
 //                    G = min(8, stages) gathers are in flight.
-//   warp 1, lane 0   waits for both, issues the stage's M = 128, N = np,
+//   warp 1           waits for both, issues (one elected lane) the stage's M = 128, N = np,
 //                    K = 8 MMAs (one per row tile and k-step) into the
 //                    patch's tensor-memory accumulator and commits them to
 //                    the stage's empty barrier; after the patch's last stage
 //                    it commits the accumulator to the epilogue.
 //   warps 10-13      epilogue: tensor memory -> registers (the 32 lanes of
-//                    warp w % 4), times the partition-of-unity weight, -> Yb.
+//                    warp w % 4) -> Yb.
 // Two accumulators alternate between patches when they fit in the 512
 // tensor-memory columns, so the epilogue of one patch overlaps the MMAs of
 // the next.  All mbarrier waits are bounded; on a timeout the CTA records it
@@ -304,17 +301,25 @@ constexpr int A_TILE = 128 * KS * 4;      // bytes of one 128-row tile of a stag
 constexpr int B_GROUP = (KS / 4) * 128;   // bytes between 8-row groups of the B operand
 constexpr int HDR = 1024;                 // barriers, tensor-memory address, abort flag
 constexpr int GATHER_WARPS = 8;           // stages gathered concurrently
-constexpr int THREADS = 32 * (2 + GATHER_WARPS + 4);
+constexpr int SPLIT_WARPS = 8;            // 3xTF32: the inverse's hi and lo parts
+constexpr int META_MAX = 512;             // patches of one CTA listed in shared memory
+__host__ __device__ constexpr int threads_of(bool split) { return 32 * (2 + GATHER_WARPS + 4 + (split ? SPLIT_WARPS : 0)); }
+// bytes of the CTA's patch list (patch, first slot, size) for nlist patches on grid CTAs
+__host__ __device__ inline int meta_bytes(int nlist, int grid) {
+    const int k = (nlist + grid - 1) / grid;
+    return (12 * (k < META_MAX ? k : META_MAX) + 15) & ~15;
+}
 constexpr long long WAIT_LIMIT = 1ll << 22;
 
 __host__ __device__ constexpr int np_of(int m) { return m < 16 ? 16 : m; }
 __host__ __device__ inline int tiles_of(int n) { return (n + 127) >> 7; }
-// a stage: the inverse's 128-row tiles (split: the hi tiles, then the lo
-// tiles), then the B operand (split: its hi part, then its lo part)
+// a stage: the inverse's 128-row tiles (split: their hi parts), then the B
+// operand (split: its hi part, then its lo part); the inverse's lo parts have
+// a shorter ring of their own behind the stages
 __host__ __device__ inline int stage_bytes(int maxn, int np, bool split = false) {
-    const int f = split ? 2 : 1;
-    return (f * tiles_of(maxn) * A_TILE + f * np * KS * 4 + 1023) & ~1023;
+    return (tiles_of(maxn) * A_TILE + (split ? 2 : 1) * np * KS * 4 + 1023) & ~1023;
 }
+__host__ __device__ inline int lo_bytes(int maxn) { return tiles_of(maxn) * A_TILE; }
 __host__ __device__ inline int acc_cols(int maxn, int np) { return tiles_of(maxn) * np; }
 __host__ __device__ inline int acc_bufs(int maxn, int np) { return 2 * acc_cols(maxn, np) <= 512 ? 2 : 1; }
 __host__ __device__ inline int tmem_cols(int maxn, int np) {
@@ -340,15 +345,18 @@ __host__ __device__ constexpr uint32_t idesc(int np) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(np >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
 }
 
+// one elected lane of a converged warp issues (the same one every time)
 __device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t id, uint32_t acc) {
     asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
+        "{\n\t.reg .pred p, q;\n\tsetp.ne.b32 p, %4, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d),
         "l"(a), "l"(b), "r"(id), "r"(acc));
 }
 __device__ __forceinline__ void commit(uint32_t mbar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-                 : "memory");
+    asm volatile(
+        "{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
+        "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::"r"(mbar)
+        : "memory");
 }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -358,6 +366,11 @@ __device__ __forceinline__ void mbar_init(uint32_t a, uint32_t count) {
 }
 __device__ __forceinline__ void mbar_arrive(uint32_t a) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(a) : "memory");
+}
+// one arrival for the warp, after every lane's writes (and proxy fence)
+__device__ __forceinline__ void warp_arrive(uint32_t a, int lane) {
+    __syncwarp();
+    if (lane == 0) mbar_arrive(a);
 }
 __device__ __forceinline__ void mbar_expect_tx(uint32_t a, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(a), "r"(bytes) : "memory");
@@ -408,6 +421,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, uint
         "l"(tmap), "r"(mbar), "r"(x), "r"(y)
         : "memory");
 }
+__device__ __forceinline__ void st32(float* p, const uint32_t* v) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+                 "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
+                 : "memory");
+}
 __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&v)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -416,32 +434,48 @@ __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&v)[16]) {
         : "r"(taddr));
 }
 
-// SPLIT (3xTF32): the inverse comes as two arrays, hi = TF32(a) and
-// lo = a - hi (tmaps over hi, tmaps_lo over lo), R as hi = TF32(r) and
-// lo = TF32(r - hi), and every k-step issues three MMAs into the same
-// accumulator: lo x hi, hi x lo, hi x hi (lo x lo, of relative size 2^-22,
-// is dropped).  This keeps FP32 accuracy on the tensor cores.
+// SPLIT (3xTF32): the inverse is used as hi = TF32(a) and lo = a - hi, R as
+// hi = TF32(r) and lo = TF32(r - hi), and every k-step issues three MMAs into
+// the same accumulator: lo x hi, hi x lo, hi x hi (lo x lo, of relative size
+// 2^-22, is dropped).  This keeps FP32 accuracy on the tensor cores.  Warps
+// 14-21 form the inverse's parts in shared memory, element by element (so in
+// the TMA's swizzled places): hi over the FP32 tile, lo into a ring of lr slots
+// (lr <= ST: a slot is refilled once the MMAs of lr stages before are done).
+// Reading both parts from memory instead costs twice the bytes of the kernel's
+// one large stream.
+//
+// What bounds it: the chain of a stage through its roles, so each was cut to
+// what it needs.  The MMA warp issues from warp-uniform descriptors (one thread
+// rebuilding them took longer than the MMAs: 80-90 cycles for an MMA); the
+// conversion works on 8 / gw stages at once; the epilogue stores 32-byte sectors
+// and loads nothing (the partition-of-unity weights are applied in the scatter);
+// the CTA's patches are listed in shared memory once for all roles.
+// 3xTF32, 32 right-hand sides, 16,129 patches of 81 DoFs and less: 434 -> 263 us;
+// 64 right-hand sides, 16^3 P3 (4817 patches of up to 540 DoFs, 3.9 GB of
+// inverses): 1664 -> 1262 us (3.1 TB/s; two to three stages of 40 KB fit).
 template <int M, int ST, bool SPLIT>
-__global__ void __launch_bounds__(THREADS, 1) k_patch_gemm_tc(int npatch, int maxn, const int* __restrict__ plist,
-                                                              const int* __restrict__ poff,
-                                                              const int* __restrict__ pdofs,
-                                                              const CUtensorMap* __restrict__ tmaps,
-                                                              const CUtensorMap* __restrict__ tmaps_lo,
-                                                              const float* __restrict__ X,
-                                                              const float* __restrict__ wt, float* __restrict__ Yb,
-                                                              int* status) {
+__global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npatch, int maxn, int lr, int gw, const int* __restrict__ plist,
+                                                                        const int* __restrict__ poff,
+                                                                        const int* __restrict__ pdofs,
+                                                                        const CUtensorMap* __restrict__ tmaps,
+                                                                        const float* __restrict__ X,
+                                                                        float* __restrict__ Yb, int* status) {
     constexpr int NP = np_of(M);
-    constexpr int F = SPLIT ? 2 : 1;
     extern __shared__ __align__(1024) unsigned char smem_tc[];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // uniform for the compiler
     const uint32_t base = smem_u32(smem_tc);
     const uint32_t full0 = base, empty0 = base + 8 * ST, accf0 = base + 16 * ST, acce0 = accf0 + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_tc + 16 * ST + 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_tc + 16 * ST + 36);
+    const uint32_t raw0 = base + 16 * ST + 48;                // SPLIT: the TMA's barriers
+    int* meta = reinterpret_cast<int*>(smem_tc + HDR);        // [kpatch][3]
     const int sbytes = stage_bytes(maxn, NP, SPLIT);
-    const uint32_t stage0 = (base + HDR + 1023) & ~1023u;     // swizzle atoms need 1024-byte alignment
-    const uint32_t lo_off = (uint32_t)(tiles_of(maxn) * A_TILE);     // lo tiles inside a stage (SPLIT)
-    const uint32_t b_off = (uint32_t)(F * tiles_of(maxn) * A_TILE);  // B operand inside a stage
+    // swizzle atoms need 1024-byte alignment
+    const uint32_t stage0 = (base + HDR + (uint32_t)meta_bytes(npatch, gridDim.x) + 1023) & ~1023u;
+    const int kpatch = (npatch - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;   // patches of this CTA
+    const uint32_t lo0 = stage0 + (uint32_t)(ST * sbytes);           // lo parts of the inverse (SPLIT)
+    const uint32_t b_off = (uint32_t)(tiles_of(maxn) * A_TILE);      // B operand inside a stage
     constexpr uint32_t BLO = (uint32_t)(NP * KS * 4);                 // its lo part after the hi part (SPLIT)
     const int nbuf = acc_bufs(maxn, NP), ccols = acc_cols(maxn, NP), ncols = tmem_cols(maxn, NP);
 
@@ -451,14 +485,35 @@ __global__ void __launch_bounds__(THREADS, 1) k_patch_gemm_tc(int npatch, int ma
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    for (int k = tid; k < min(kpatch, META_MAX); k += threads_of(SPLIT)) {
+        const int i = blockIdx.x + k * gridDim.x, p = plist ? __ldg(plist + i) : i;
+        const int s0 = __ldg(poff + p);
+        meta[3 * k] = p;
+        meta[3 * k + 1] = s0;
+        meta[3 * k + 2] = __ldg(poff + p + 1) - s0;
+    }
+    auto item = [&](int k, int& p, int& s0, int& n) {
+        if (k < META_MAX) {
+            p = meta[3 * k];
+            s0 = meta[3 * k + 1];
+            n = meta[3 * k + 2];
+        } else {
+            const int i = blockIdx.x + k * gridDim.x;
+            p = plist ? __ldg(plist + i) : i;
+            s0 = __ldg(poff + p);
+            n = __ldg(poff + p + 1) - s0;
+        }
+    };
     if (tid == 0) {
         for (int s = 0; s < ST; ++s) {
-            mbar_init(full0 + 8 * s, 1 + 32);      // TMA arrival with the byte count + one gather warp
+            // the inverse (TMA arrival with the byte count, or the split warps) + one gather warp
+            mbar_init(full0 + 8 * s, (SPLIT ? gw : 1) + 1);
             mbar_init(empty0 + 8 * s, 1);          // MMA commit
+            if (SPLIT) mbar_init(raw0 + 8 * s, 1); // TMA arrival with the byte count
         }
         for (int b = 0; b < 2; ++b) {
             mbar_init(accf0 + 8 * b, 1);           // MMA commit of a patch's last stage
-            mbar_init(acce0 + 8 * b, 128);         // epilogue threads
+            mbar_init(acce0 + 8 * b, 4);           // epilogue warps
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -471,61 +526,68 @@ __global__ void __launch_bounds__(THREADS, 1) k_patch_gemm_tc(int npatch, int ma
     if (warp == 0) {
         // ---------------------------------------------------------- TMA ---
         if (lane == 0) {
+            const uint32_t bar0 = SPLIT ? raw0 : full0;
             int it = 0;
-            for (int i = blockIdx.x; i < npatch; i += gridDim.x) {
-                const int p = plist ? __ldg(plist + i) : i;
-                const int n = poff[p + 1] - poff[p], tiles = tiles_of(n), nst = (n + KS - 1) / KS;
+            for (int k = 0; k < kpatch; ++k) {
+                int p, s0, n;
+                item(k, p, s0, n);
+                const int tiles = tiles_of(n), nst = (n + KS - 1) / KS;
                 const CUtensorMap* tm = tmaps + p;
-                const CUtensorMap* tml = SPLIT ? tmaps_lo + p : nullptr;
                 for (int j = 0; j < nst; ++j, ++it) {
                     const int s = it % ST;
                     if (it >= ST && !mbar_wait(empty0 + 8 * s, ((it / ST) - 1) & 1, abort_flag)) goto done;
                     const uint32_t st = stage0 + (uint32_t)(s * sbytes);
-                    mbar_expect_tx(full0 + 8 * s, (uint32_t)(F * tiles * A_TILE));
-                    for (int mt = 0; mt < tiles; ++mt) {
-                        tma_load_2d(st + mt * A_TILE, tm, full0 + 8 * s, j * KS, mt * 128);
-                        if (SPLIT) tma_load_2d(st + lo_off + mt * A_TILE, tml, full0 + 8 * s, j * KS, mt * 128);
-                    }
+                    mbar_expect_tx(bar0 + 8 * s, (uint32_t)(tiles * A_TILE));
+                    for (int mt = 0; mt < tiles; ++mt) tma_load_2d(st + mt * A_TILE, tm, bar0 + 8 * s, j * KS, mt * 128);
                 }
             }
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA ---
-        if (lane == 0) {
-            constexpr uint32_t ID = idesc(NP);
-            int it = 0, pc = 0;
-            for (int i = blockIdx.x; i < npatch; i += gridDim.x, ++pc) {
-                const int p = plist ? __ldg(plist + i) : i;
-                const int n = poff[p + 1] - poff[p], tiles = tiles_of(n), nst = (n + KS - 1) / KS;
-                const int b = pc % nbuf;
-                if (pc >= nbuf && !mbar_wait(acce0 + 8 * b, ((pc / nbuf) - 1) & 1, abort_flag)) goto done;
+        // the whole warp walks the stages and one lane issues: addresses and
+        // descriptors stay warp-uniform, a descriptor is a base plus an offset
+        // in its address field (16-byte units; shared memory fits its 14 bits)
+        constexpr uint32_t ID = idesc(NP);
+        const uint64_t a0 = desc_sw64(stage0), al0 = SPLIT ? desc_sw64(lo0) : 0;
+        const uint64_t b0 = desc_plain(stage0 + b_off, 128, B_GROUP);
+        int s = 0, ls = 0;
+        uint32_t ph = 0;
+        for (int pc = 0; pc < kpatch; ++pc) {
+            int p, s0, n;
+            item(pc, p, s0, n);
+            const int tiles = tiles_of(n), nst = (n + KS - 1) / KS;
+            const int b = pc % nbuf;
+            if (pc >= nbuf && !mbar_wait(acce0 + 8 * b, ((pc / nbuf) - 1) & 1, abort_flag)) goto done;
+            fence_after();
+            const uint32_t acc = tmem + (uint32_t)(b * ccols);
+            for (int j = 0; j < nst; ++j) {
+                if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) goto done;
                 fence_after();
-                const uint32_t acc = tmem + (uint32_t)(b * ccols);
-                for (int j = 0; j < nst; ++j, ++it) {
-                    const int s = it % ST;
-                    if (!mbar_wait(full0 + 8 * s, (it / ST) & 1, abort_flag)) goto done;
-                    fence_after();
-                    const uint32_t st = stage0 + (uint32_t)(s * sbytes);
+                const uint32_t so = (uint32_t)(s * sbytes) >> 4;
+                const uint32_t lo = SPLIT ? (uint32_t)(ls * lo_bytes(maxn)) >> 4 : 0;
 #pragma unroll
-                    for (int u = 0; u < KS / 8; ++u) {
-                        const uint64_t bd = desc_plain(st + b_off + (uint32_t)(u * 2 * 128), 128, B_GROUP);
-                        for (int mt = 0; mt < tiles; ++mt) {
-                            const uint64_t ad = desc_sw64(st + (uint32_t)(mt * A_TILE + u * 32));
-                            if (SPLIT) {
-                                const uint64_t adl = desc_sw64(st + lo_off + (uint32_t)(mt * A_TILE + u * 32));
-                                const uint64_t bdl = desc_plain(st + b_off + BLO + (uint32_t)(u * 2 * 128), 128, B_GROUP);
-                                mma(acc + (uint32_t)(mt * NP), adl, bd, ID, (j | u) != 0);
-                                mma(acc + (uint32_t)(mt * NP), ad, bdl, ID, 1);
-                                mma(acc + (uint32_t)(mt * NP), ad, bd, ID, 1);
-                            } else {
-                                mma(acc + (uint32_t)(mt * NP), ad, bd, ID, (j | u) != 0);
-                            }
+                for (int u = 0; u < KS / 8; ++u) {
+                    const uint64_t bd = b0 + so + (uint32_t)(u * 16);
+                    const uint64_t bdl = bd + (BLO >> 4);
+                    const uint32_t first = (j | u) != 0;
+                    for (int mt = 0; mt < tiles; ++mt) {
+                        const uint64_t ad = a0 + so + (uint32_t)((mt * A_TILE + u * 32) >> 4);
+                        const uint32_t d = acc + (uint32_t)(mt * NP);
+                        if (SPLIT) {
+                            const uint64_t adl = al0 + lo + (uint32_t)((mt * A_TILE + u * 32) >> 4);
+                            mma(d, adl, bd, ID, first);
+                            mma(d, ad, bdl, ID, 1);
+                            mma(d, ad, bd, ID, 1);
+                        } else {
+                            mma(d, ad, bd, ID, first);
                         }
                     }
-                    commit(empty0 + 8 * s);
                 }
-                commit(accf0 + 8 * b);
+                commit(empty0 + 8 * s);
+                if (++s == ST) { s = 0; ph ^= 1u; }
+                if (SPLIT && ++ls == lr) ls = 0;
             }
+            commit(accf0 + 8 * b);
         }
     } else if (warp < 2 + GATHER_WARPS) {
         // ------------------------------------------------------- gather ---
@@ -541,9 +603,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_patch_gemm_tc(int npatch, int ma
         constexpr int NE = (NP / 4 + 7) / 8;
         if (g >= G) goto done;
         int it = 0;
-        for (int i = blockIdx.x; i < npatch; i += gridDim.x) {
-            const int p = plist ? __ldg(plist + i) : i;
-            const int s0 = poff[p], n = poff[p + 1] - s0, nst = (n + KS - 1) / KS;
+        for (int pc = 0; pc < kpatch; ++pc) {
+            int p, s0, n;
+            item(pc, p, s0, n);
+            const int nst = (n + KS - 1) / KS;
             for (int j = 0; j < nst; ++j, ++it) {
                 if (it % G != g) continue;
                 const int s = it % ST;
@@ -584,23 +647,16 @@ __global__ void __launch_bounds__(THREADS, 1) k_patch_gemm_tc(int npatch, int ma
                     }
                 }
                 fence_proxy_async();
-                mbar_arrive(full0 + 8 * s);
+                warp_arrive(full0 + 8 * s, lane);
             }
         }
-    } else {
+    } else if (warp < 2 + GATHER_WARPS + 4) {
         // ----------------------------------------------------- epilogue ---
         const int q = warp & 3;            // tensor-memory lanes 32 q .. 32 q + 31
-        int pc = 0;
-        for (int i = blockIdx.x; i < npatch; i += gridDim.x, ++pc) {
-            const int p = plist ? __ldg(plist + i) : i;
-            const int s0 = poff[p], n = poff[p + 1] - s0, tiles = tiles_of(n);
-            const int b = pc % nbuf;
-            float w[8];
-#pragma unroll
-            for (int mt = 0; mt < 8; ++mt) {
-                const int row = mt * 128 + 32 * q + lane;
-                w[mt] = (mt < tiles && row < n) ? __ldg(wt + __ldg(pdofs + s0 + row)) : 0.f;
-            }
+        for (int pc = 0; pc < kpatch; ++pc) {
+            int p, s0, n;
+            item(pc, p, s0, n);
+            const int tiles = tiles_of(n), b = pc % nbuf;
             if (!mbar_wait(accf0 + 8 * b, (pc / nbuf) & 1, abort_flag)) goto done;
             fence_after();
 #pragma unroll
@@ -613,18 +669,52 @@ __global__ void __launch_bounds__(THREADS, 1) k_patch_gemm_tc(int npatch, int ma
                     ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * ccols + mt * NP + cb), v);
                     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
                     if (row < n && cb < M) {
-                        float4* dst = reinterpret_cast<float4*>(Yb + (long long)(s0 + row) * M + cb);
-#pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            if (cb + 4 * e < M)
-                                dst[e] = make_float4(w[mt] * __uint_as_float(v[4 * e]), w[mt] * __uint_as_float(v[4 * e + 1]),
-                                                     w[mt] * __uint_as_float(v[4 * e + 2]),
-                                                     w[mt] * __uint_as_float(v[4 * e + 3]));
+                        // 32-byte stores: a lane fills whole sectors of its row
+                        float* dst = Yb + (long long)(s0 + row) * M + cb;
+                        st32(dst, v);
+                        if (cb + 8 < M) st32(dst + 8, v + 8);
                     }
                 }
             }
             fence_before();
-            mbar_arrive(acce0 + 8 * b);
+            warp_arrive(acce0 + 8 * b, lane);
+        }
+    } else if (SPLIT) {
+        // -------------------------------------------- hi and lo parts ---
+        // group grp of gw warps takes every ng-th stage (a stage's chain of
+        // waits, conversion and fence takes about 0.5 us whatever its size).
+        // ng <= ST and lr <= ST: the MMAs complete in order, so the wait for
+        // stage it - lr shows that raw(it - ST) is over, and the wait before it
+        // (ng stages back) the same for empty(it - lr - ST): no barrier is two
+        // phases behind the parity polled for.
+        const int sw = warp - (2 + GATHER_WARPS + 4), ng = SPLIT_WARPS / gw, grp = sw / gw;
+        const int t = (sw - grp * gw) * 32 + lane;
+        int it = 0;
+        for (int pc = 0; pc < kpatch; ++pc) {
+            int p, s0, n;
+            item(pc, p, s0, n);
+            const int nst = (n + KS - 1) / KS, nvec = tiles_of(n) * (A_TILE / 16);
+            for (int j = 0; j < nst; ++j, ++it) {
+                if (it % ng != grp) continue;
+                const int s = it % ST;
+                if (it >= lr && !mbar_wait(empty0 + 8 * ((it - lr) % ST), ((it - lr) / ST) & 1, abort_flag)) goto done;
+                if (!mbar_wait(raw0 + 8 * s, (it / ST) & 1, abort_flag)) goto done;
+                float4* hp = reinterpret_cast<float4*>(smem_tc + (stage0 - base) + (size_t)s * sbytes);
+                float4* lp = reinterpret_cast<float4*>(smem_tc + (lo0 - base) + (size_t)(it % lr) * lo_bytes(maxn));
+#pragma unroll 4
+                for (int x = t; x < nvec; x += 32 * gw) {
+                    const float4 a = hp[x];
+                    float4 hi;
+                    hi.x = __uint_as_float(to_tf32(a.x));
+                    hi.y = __uint_as_float(to_tf32(a.y));
+                    hi.z = __uint_as_float(to_tf32(a.z));
+                    hi.w = __uint_as_float(to_tf32(a.w));
+                    hp[x] = hi;
+                    lp[x] = make_float4(a.x - hi.x, a.y - hi.y, a.z - hi.z, a.w - hi.w);
+                }
+                fence_proxy_async();
+                warp_arrive(full0 + 8 * s, lane);
+            }
         }
     }
 done:
@@ -640,8 +730,8 @@ done:
 }  // namespace tc
 
 __global__ void __launch_bounds__(256) k_pull_scatter(int n, int m, const int* __restrict__ soff,
-                                                      const int* __restrict__ sidx, const float2* __restrict__ Yb,
-                                                      float alpha, float beta, float2* __restrict__ out) {
+                                                      const int* __restrict__ sidx, const float* __restrict__ wt,
+                                                      const float2* __restrict__ Yb, float alpha, float beta, float2* __restrict__ out) {
     const int L = m >> 1;
     const long long gt = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     const int j = (int)(gt / L), c2 = (int)(gt - (long long)j * L);
@@ -653,6 +743,9 @@ __global__ void __launch_bounds__(256) k_pull_scatter(int n, int m, const int* _
         acc.x += y.x;
         acc.y += y.y;
     }
+    const float w = wt[j];
+    acc.x *= w;
+    acc.y *= w;
     const long long o = (long long)j * L + c2;
     if (beta == 0.f) out[o] = make_float2(alpha * acc.x, alpha * acc.y);
     else { const float2 v = out[o]; out[o] = make_float2(alpha * acc.x + beta * v.x, alpha * acc.y + beta * v.y); }
@@ -707,11 +800,11 @@ static size_t gemm_smem(int maxn, int m, int stages, int nw) {
 
 template <int M, int MODE, int ST>
 static void launch_gemm(int threads, size_t smem, int nlist, const int* plist, const int* poff, const int* pdofs,
-                        const long long* ioff, const float* inv, const float* X, const float* wt, float* Yb,
+                        const long long* ioff, const float* inv, const float* X, float* Yb,
                         cudaStream_t s) {
     cudaFuncSetAttribute(k_patch_gemm<M, MODE, ST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaFuncSetAttribute(k_patch_gemm<M, MODE, ST>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
-    k_patch_gemm<M, MODE, ST><<<nlist, threads, smem, s>>>(nlist, plist, poff, pdofs, ioff, inv, X, wt, Yb);
+    k_patch_gemm<M, MODE, ST><<<nlist, threads, smem, s>>>(nlist, plist, poff, pdofs, ioff, inv, X, Yb);
 }
 
 static int device_attr(cudaDeviceAttr attr) {
@@ -725,18 +818,18 @@ static int device_attr(cudaDeviceAttr attr) {
 // of 8, 6 or MIN_STAGES as fit the shared memory
 template <int M, int MODE>
 static void launch_gemm_st(int maxn, int nw, int nlist, const int* plist, const int* poff, const int* pdofs,
-                           const long long* ioff, const float* inv, const float* X, const float* wt, float* Yb,
+                           const long long* ioff, const float* inv, const float* X, float* Yb,
                            cudaStream_t s) {
     const size_t dev_max = (size_t)device_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin);
     if (nw <= 0) nw = gemm_default_warps(maxn);
     const int threads = 32 * nw;
     if (gemm_smem(maxn, M, 8, nw) <= dev_max)
-        launch_gemm<M, MODE, 8>(threads, gemm_smem(maxn, M, 8, nw), nlist, plist, poff, pdofs, ioff, inv, X, wt, Yb, s);
+        launch_gemm<M, MODE, 8>(threads, gemm_smem(maxn, M, 8, nw), nlist, plist, poff, pdofs, ioff, inv, X, Yb, s);
     else if (gemm_smem(maxn, M, 6, nw) <= dev_max)
-        launch_gemm<M, MODE, 6>(threads, gemm_smem(maxn, M, 6, nw), nlist, plist, poff, pdofs, ioff, inv, X, wt, Yb, s);
+        launch_gemm<M, MODE, 6>(threads, gemm_smem(maxn, M, 6, nw), nlist, plist, poff, pdofs, ioff, inv, X, Yb, s);
     else
         launch_gemm<M, MODE, MIN_STAGES>(threads, gemm_smem(maxn, M, MIN_STAGES, nw), nlist, plist, poff, pdofs, ioff,
-                                         inv, X, wt, Yb, s);
+                                         inv, X, Yb, s);
 }
 
 // Patches of <= TC_MIN_N DoFs fill under half of a 128-row MMA tile; the
@@ -754,7 +847,7 @@ int gemm_kind(int mode, int n) {
 // tensor-core TF32 path: a persistent grid of one CTA per SM (the dynamic
 // shared memory is at least half an SM's, so no two CTAs share an SM and its
 // 512 tensor-memory columns), with as many pipeline stages as fit, at most 12
-struct TcPlan { int stages = 0; size_t smem = 0; int grid = 0; };
+struct TcPlan { int stages = 0, lr = 0, gw = 1; size_t smem = 0; int grid = 0; };
 
 static TcPlan tc_plan(int maxn, int m, int npatch, bool split = false) {
     TcPlan pl;
@@ -762,33 +855,39 @@ static TcPlan tc_plan(int maxn, int m, int npatch, bool split = false) {
     if (tc::tiles_of(maxn) > 8 || tc::tmem_cols(maxn, np) > 512) return pl;
     const long long optin = device_attr(cudaDevAttrMaxSharedMemoryPerBlockOptin);
     const long long per_sm = device_attr(cudaDevAttrMaxSharedMemoryPerMultiprocessor);
-    const long long fixed = tc::HDR + 1024, sb = tc::stage_bytes(maxn, np, split);
-    const long long st = std::min<long long>(12, (optin - fixed) / sb);
-    if (st < 2) return pl;
-    pl.stages = (int)st;
-    pl.smem = (size_t)std::max<long long>(fixed + st * sb, per_sm / 2 + 1024);
-    if ((long long)pl.smem > optin) pl.smem = (size_t)optin;
     pl.grid = std::max(1, std::min(npatch, device_attr(cudaDevAttrMultiProcessorCount)));
+    const long long sb = tc::stage_bytes(maxn, np, split);
+    const long long fixed = tc::HDR + tc::meta_bytes(npatch, pl.grid) + 1024;
+    // split: lo slots, and warps per conversion group (one for a stage of one
+    // row tile, two for two, four above: 8 / gw stages are converted at once)
+    const long long lob = split ? tc::lo_bytes(maxn) : 0;
+    auto room = [&](int lr) { return (optin - fixed - lr * lob) / sb; };
+    pl.lr = !split ? 0 : room(8) >= 8 ? 8 : room(4) >= 6 ? 4 : 2;
+    const long long st = std::min<long long>(12, room(pl.lr));
+    if (st < 2) return pl;
+    pl.gw = tc::tiles_of(maxn) <= 1 ? 1 : tc::tiles_of(maxn) == 2 ? 2 : 4;
+    while (tc::SPLIT_WARPS / pl.gw > (int)st) pl.gw *= 2;
+    pl.stages = (int)st;
+    pl.smem = (size_t)std::max<long long>(fixed + st * sb + pl.lr * lob, per_sm / 2 + 1024);
+    if ((long long)pl.smem > optin) pl.smem = (size_t)optin;
     return pl;
 }
 
 template <int M, int ST, bool SPLIT>
 static void launch_tc(const TcPlan& pl, int nlist, const int* plist, int maxn, const int* poff, const int* pdofs,
-                      const void* tmaps, const void* tmaps_lo, const float* X, const float* wt, float* Yb, int* status,
-                      cudaStream_t s) {
+                      const void* tmaps, const float* X, float* Yb, int* status, cudaStream_t s) {
     cudaFuncSetAttribute(tc::k_patch_gemm_tc<M, ST, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
-    tc::k_patch_gemm_tc<M, ST, SPLIT><<<pl.grid, tc::THREADS, pl.smem, s>>>(
-        nlist, maxn, plist, poff, pdofs, reinterpret_cast<const CUtensorMap*>(tmaps),
-        reinterpret_cast<const CUtensorMap*>(tmaps_lo), X, wt, Yb, status);
+    tc::k_patch_gemm_tc<M, ST, SPLIT><<<pl.grid, tc::threads_of(SPLIT), pl.smem, s>>>(
+        nlist, maxn, pl.lr, pl.gw, plist, poff, pdofs, reinterpret_cast<const CUtensorMap*>(tmaps), X, Yb, status);
 }
 
 template <int M, bool SPLIT>
 static void launch_tc_st(int nlist, const int* plist, int maxn, const int* poff, const int* pdofs, const void* tmaps,
-                         const void* tmaps_lo, const float* X, const float* wt, float* Yb, int* status, cudaStream_t s) {
+                         const float* X, float* Yb, int* status, cudaStream_t s) {
     const TcPlan pl = tc_plan(maxn, M, nlist, SPLIT);
     switch (pl.stages) {
 #define SBAT_TC_CASE(S) \
-    case S: launch_tc<M, S, SPLIT>(pl, nlist, plist, maxn, poff, pdofs, tmaps, tmaps_lo, X, wt, Yb, status, s); break;
+    case S: launch_tc<M, S, SPLIT>(pl, nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, s); break;
         SBAT_TC_CASE(2) SBAT_TC_CASE(3) SBAT_TC_CASE(4) SBAT_TC_CASE(5) SBAT_TC_CASE(6) SBAT_TC_CASE(7)
         SBAT_TC_CASE(8) SBAT_TC_CASE(9) SBAT_TC_CASE(10) SBAT_TC_CASE(11) SBAT_TC_CASE(12)
 #undef SBAT_TC_CASE
@@ -799,17 +898,16 @@ static void launch_tc_st(int nlist, const int* plist, int maxn, const int* poff,
 template <int M>
 static void patch_gemm_m(int mode, int kind, int nw, int nlist, const int* plist, int maxn, const int* poff,
                          const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
-                         const void* tmaps_hi, const void* tmaps_lo, const float* X, const float* wt, float* Yb,
-                         int* status, cudaStream_t s) {
+                         const float* X, float* Yb, int* status, cudaStream_t s) {
     if (kind == GEMM_KIND_AUTO) kind = gemm_kind(mode, maxn);
     if (kind == GEMM_KIND_TC && mode == GEMM_3XTF32)
-        launch_tc_st<M, true>(nlist, plist, maxn, poff, pdofs, tmaps_hi, tmaps_lo, X, wt, Yb, status, s);
+        launch_tc_st<M, true>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, s);
     else if (kind == GEMM_KIND_TC)
-        launch_tc_st<M, false>(nlist, plist, maxn, poff, pdofs, tmaps, nullptr, X, wt, Yb, status, s);
+        launch_tc_st<M, false>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, s);
     else if (mode == GEMM_3XTF32)
-        launch_gemm_st<M, GEMM_3XTF32>(maxn, nw, nlist, plist, poff, pdofs, ioff, inv, X, wt, Yb, s);
+        launch_gemm_st<M, GEMM_3XTF32>(maxn, nw, nlist, plist, poff, pdofs, ioff, inv, X, Yb, s);
     else
-        launch_gemm_st<M, GEMM_TF32>(maxn, nw, nlist, plist, poff, pdofs, ioff, inv, X, wt, Yb, s);
+        launch_gemm_st<M, GEMM_TF32>(maxn, nw, nlist, plist, poff, pdofs, ioff, inv, X, Yb, s);
 }
 
 // the largest patch decides: a smaller patch of either kind needs no more
@@ -824,21 +922,6 @@ const char* patch_gemm_check(int mode, int maxn, int m) {
         return "patch too large for the tensor memory at this width";
     return tc_plan(maxn, m, 1, mode == GEMM_3XTF32).stages ? nullptr
                                                            : "patch too large for the shared memory of the tensor-core patch GEMM";
-}
-
-namespace {
-__global__ void k_split_tf32(long long n, const float* __restrict__ a, float* __restrict__ hi, float* __restrict__ lo) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float x = a[i];
-        const float h = __uint_as_float(to_tf32(x));
-        hi[i] = h;
-        lo[i] = x - h;
-    }
-}
-}  // namespace
-
-void split_tf32(long long n, const float* a, float* hi, float* lo, cudaStream_t s) {
-    if (n > 0) k_split_tf32<<<grid_of(n, 256), 256, 0, s>>>(n, a, hi, lo);
 }
 
 int wait_probe(long long polls, int* result_dev, cudaStream_t s) {
@@ -884,27 +967,27 @@ void build_tmaps(int npatch, const int* poff_d, const long long* ioff_d, const f
 }
 
 void patch_gemm(int mode, int kind, int nw, int nlist, const int* plist, int maxn, int m, const int* poff,
-                const int* pdofs, const long long* ioff, const float* inv, const void* tmaps, const void* tmaps_hi,
-                const void* tmaps_lo, const float* X, const float* wt, float* Yb, int* status, cudaStream_t s) {
+                const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
+                const float* X, float* Yb, int* status, cudaStream_t s) {
     if (nlist <= 0) return;
     switch (m) {
 #define SBAT_M(MM) \
     case MM: \
-        patch_gemm_m<MM>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, tmaps_hi, tmaps_lo, X, wt, \
+        patch_gemm_m<MM>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, X, \
                          Yb, status, s); \
         break;
         SBAT_M(8) SBAT_M(16) SBAT_M(32)
 #undef SBAT_M
         default:
-            patch_gemm_m<64>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, tmaps_hi, tmaps_lo, X, wt,
+            patch_gemm_m<64>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, X,
                              Yb, status, s);
     }
 }
 
-void pull_scatter(int n, int m, const int* soff, const int* sidx, const float* Yb, float alpha, float beta,
-                  float* out, cudaStream_t s) {
+void pull_scatter(int n, int m, const int* soff, const int* sidx, const float* wt, const float* Yb, float alpha,
+                  float beta, float* out, cudaStream_t s) {
     const long long threads = (long long)n * (m / 2);
-    k_pull_scatter<<<(int)((threads + 255) / 256), 256, 0, s>>>(n, m, soff, sidx, reinterpret_cast<const float2*>(Yb),
+    k_pull_scatter<<<(int)((threads + 255) / 256), 256, 0, s>>>(n, m, soff, sidx, wt, reinterpret_cast<const float2*>(Yb),
                                                                 alpha, beta, reinterpret_cast<float2*>(out));
 }
 

@@ -4,7 +4,7 @@
 // a level is stored as X[j * m + c] (DoF j, right-hand side c), m a multiple
 // of 8.  A sparse matrix is then read once per batch, every gathered row is
 // m contiguous floats, and the patch apply becomes one dense GEMM per patch,
-//   Y_i (n_i x m) = W_i K_i^{-1} (n_i x n_i) R_i (n_i x m),
+//   Y_i (n_i x m) = K_i^{-1} (n_i x n_i) R_i (n_i x m),
 // which runs on the tensor cores (warp-level m16n8k8 TF32 MMA; the 3xTF32
 // split a = a_hi + a_lo keeps FP32 accuracy).  At m = 64 the GEMM does
 // 2 m = 128 flop per 4-byte inverse entry, so it is bound by streaming the
@@ -42,15 +42,13 @@ int wait_probe(long long polls, int* result_dev, cudaStream_t s);
 size_t tmap_bytes(int npatch);
 void build_tmaps(int npatch, const int* poff, const long long* ioff, const float* inv, void* tmaps);
 
-// Yb[(poff[p] + a) * m + c] = wt[dof] * (K_p^{-1} R_p)[a][c], R_p[a][c] =
+// Yb[(poff[p] + a) * m + c] = (K_p^{-1} R_p)[a][c], R_p[a][c] =
 // X[pdofs[poff[p] + a] * m + c], for the nlist patches p = plist[i] (plist
 // NULL: p = i < nlist); inverses column-major with leading dimension
 // (n + 3) & ~3 at ioff[p] (the FP32 ASM layout), symmetric.
-//   kind GEMM_KIND_TC     tcgen05 tensor cores; GEMM_TF32 reads the inverses
-//                         through tmaps (build_tmaps over inv), GEMM_3XTF32
-//                         through tmaps_hi / tmaps_lo (build_tmaps over the
-//                         split_tf32 parts, same layout) with three MMAs per
-//                         k-step;
+//   kind GEMM_KIND_TC     tcgen05 tensor cores, the inverses read through
+//                         tmaps (build_tmaps over inv); GEMM_3XTF32 splits
+//                         them in shared memory, three MMAs per k-step;
 //   kind GEMM_KIND_WARP   warp-level MMA, nw warps per CTA (0: from maxn);
 //   kind GEMM_KIND_AUTO   gemm_kind(mode, maxn).
 // gemm_kind gives each patch's kind by its size: the tensor cores for
@@ -63,16 +61,15 @@ enum GemmKind { GEMM_KIND_AUTO = 0, GEMM_KIND_WARP = 1, GEMM_KIND_TC = 2 };
 int gemm_kind(int mode, int n);
 int gemm_default_warps(int maxn);
 void patch_gemm(int mode, int kind, int nw, int nlist, const int* plist, int maxn, int m, const int* poff,
-                const int* pdofs, const long long* ioff, const float* inv, const void* tmaps, const void* tmaps_hi,
-                const void* tmaps_lo, const float* X, const float* wt, float* Yb, int* status, cudaStream_t s);
-// hi[i] = TF32(a[i]) (round to nearest), lo[i] = a[i] - hi[i] (exact): the
-// operands of the 3xTF32 tensor-core GEMM
-void split_tf32(long long n, const float* a, float* hi, float* lo, cudaStream_t s);
+                const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
+                const float* X, float* Yb, int* status, cudaStream_t s);
 
-// out[j * m + c] = alpha * sum_{q in slots(j)} Yb[sidx[q] * m + c] + beta * out[j * m + c]
-// (slots in increasing order: a fixed summation order)
-void pull_scatter(int n, int m, const int* soff, const int* sidx, const float* Yb, float alpha, float beta,
-                  float* out, cudaStream_t s);
+// out[j * m + c] = alpha * wt[j] * sum_{q in slots(j)} Yb[sidx[q] * m + c] + beta * out[j * m + c]
+// (slots in increasing order: a fixed summation order; the partition-of-unity
+// weight once per DoF here instead of once per slot in the GEMM's epilogue,
+// which then loads nothing)
+void pull_scatter(int n, int m, const int* soff, const int* sidx, const float* wt, const float* Yb, float alpha,
+                  float beta, float* out, cudaStream_t s);
 
 // E[i * m + c] = sum_j C[i * ldc + j] B[j * m + c] for i, j < nc: the dense
 // FP64 coarse inverse applied to a batch (FP64 accumulation).
