@@ -1148,25 +1148,27 @@ __device__ __forceinline__ void patch_apply_body(int p, const int* __restrict__ 
 __global__ void __launch_bounds__(128) patch_apply_f32(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                                        const long long* __restrict__ ioff, const float* __restrict__ inv,
                                                        const float* __restrict__ r, const float* __restrict__ wt,
-                                                       float* __restrict__ Y) {
+                                                       float* __restrict__ Y, int n, long long nslot) {
     extern __shared__ __align__(16) unsigned char smem_pa[];
     float4* red = reinterpret_cast<float4*>(smem_pa);
     float* xs = reinterpret_cast<float*>(smem_pa + sizeof(float4) * (blockDim.x + 4));
     pdl_wait();
     pdl_release();
-    patch_apply_body<float, float4, 4>(blockIdx.x, poff, pdofs, ioff, inv, r, wt, Y, xs, red);
+    patch_apply_body<float, float4, 4>(blockIdx.x, poff, pdofs, ioff, inv, r + (long long)blockIdx.y * n, wt,
+                                            Y + blockIdx.y * nslot, xs, red);
 }
 
 __global__ void __launch_bounds__(128) patch_apply_f64(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                                        const long long* __restrict__ ioff, const double* __restrict__ inv,
                                                        const double* __restrict__ r, const double* __restrict__ wt,
-                                                       double* __restrict__ Y) {
+                                                       double* __restrict__ Y, int n, long long nslot) {
     extern __shared__ __align__(16) unsigned char smem_pa[];
     double2* red = reinterpret_cast<double2*>(smem_pa);
     double* xs = reinterpret_cast<double*>(smem_pa + sizeof(double2) * (blockDim.x + 4));
     pdl_wait();
     pdl_release();
-    patch_apply_body<double, double2, 2>(blockIdx.x, poff, pdofs, ioff, inv, r, wt, Y, xs, red);
+    patch_apply_body<double, double2, 2>(blockIdx.x, poff, pdofs, ioff, inv, r + (long long)blockIdx.y * n, wt,
+                                            Y + blockIdx.y * nslot, xs, red);
 }
 
 // One ASM sweep with factored saddle inverses (saddle_core's factored form):

@@ -41,10 +41,19 @@ enum SpmvMode { SPMV_SET = 0, SPMV_ADD = 1, SPMV_RESID = 2 };
 
 // One LANES-wide group of threads per row; values of type T accumulate in T.
 // mode SET:   y = A x        ADD: y += A x        RESID: y = b - A x
-template <typename T, int LANES, int MODE>
-__global__ void __launch_bounds__(256) spmv_csr(int nrows, const int* __restrict__ rp, const int* __restrict__ ci,
-                                                const T* __restrict__ av, const T* __restrict__ x,
-                                                T* __restrict__ y, const T* __restrict__ b) {
+// MV: blockIdx.y selects the vector; the V-cycle's kernels then work on
+// gridDim.y vectors stored one after another (the velocity components of FBF),
+// each with the arithmetic of a single one.  (Templates: the offsets cost a
+// single vector's small kernels 1-4%.)
+template <typename T, int LANES, int MODE, bool MV>
+__global__ void __launch_bounds__(256) spmv_csr(int nrows, int ncols, const int* __restrict__ rp,
+                                                const int* __restrict__ ci, const T* __restrict__ av,
+                                                const T* __restrict__ x, T* __restrict__ y, const T* __restrict__ b) {
+    if (MV) {
+        x += (long long)blockIdx.y * ncols;
+        y += (long long)blockIdx.y * nrows;
+        if (MODE == SPMV_RESID) b += (long long)blockIdx.y * nrows;
+    }
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
     const int row = gtid / LANES;
     const int lane = threadIdx.x % LANES;
@@ -286,24 +295,36 @@ __global__ void saddle_apply_bulk_f64(int d, const int* __restrict__ poff, const
 
 // One ASM sweep (Eq. 3.4): Y[poff[i] + a] = w[dof_a] * sum_b Kinv_i[a][b] r[dof_b].
 // FP32: float4 loads of 4 consecutive rows per thread; FP64: double2 loads
-// of 2 rows.  One CTA per patch; blockDim = round_up(ld / VEC, 32).
+// of 2 rows.  One CTA per patch and vector (blockIdx.y; vectors of n DoFs and
+// nslot slots); blockDim = round_up(ld / VEC, 32).
 __global__ void patch_apply_f32(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                 const long long* __restrict__ ioff, const float* __restrict__ inv,
-                                const float* __restrict__ r, const float* __restrict__ wt, float* __restrict__ Y);
+                                const float* __restrict__ r, const float* __restrict__ wt, float* __restrict__ Y, int n,
+                                long long nslot);
 __global__ void patch_apply_f64(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                 const long long* __restrict__ ioff, const double* __restrict__ inv,
-                                const double* __restrict__ r, const double* __restrict__ wt, double* __restrict__ Y);
+                                const double* __restrict__ r, const double* __restrict__ wt, double* __restrict__ Y, int n,
+                                long long nslot);
 
 // out[j] = alpha * sum_{s in slots(j)} Y[s] + beta * out[j]  (slots in a
 // fixed order, so the sum is bitwise reproducible).  Fused Chebyshev
 // bookkeeping: xmode PULL_X_SET also sets x[j] = out[j], PULL_X_ADD adds
 // x[j] += out[j]; with rdst != NULL, rdst[j] = bsrc[j].
 enum PullX { PULL_X_NONE = 0, PULL_X_SET = 1, PULL_X_ADD = 2 };
-template <typename T>
+template <typename T, bool MV>
 __global__ void __launch_bounds__(256) pull_scatter(int n, const int* __restrict__ soff, const int* __restrict__ sidx,
                                                     const T* __restrict__ Y, T alpha, T beta, T* __restrict__ out,
                                                     T* __restrict__ x, int xmode, const T* __restrict__ bsrc,
-                                                    T* __restrict__ rdst) {
+                                                    T* __restrict__ rdst, long long nslot) {
+    if (MV) {                                     // vectors of n DoFs and nslot slots, one after another
+        Y += blockIdx.y * nslot;
+        out += (long long)blockIdx.y * n;
+        if (x) x += (long long)blockIdx.y * n;
+        if (rdst) {
+            bsrc += (long long)blockIdx.y * n;
+            rdst += (long long)blockIdx.y * n;
+        }
+    }
     pdl_wait();
     pdl_release();
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
@@ -352,9 +373,13 @@ __global__ void gj_cluster_panel(int n, int k0, int B, double* __restrict__ A, i
 // y[i] = sum_j A[i][j] x[j] for i < nout (row-major, leading dimension lda),
 // one warp per row, accumulated in FP64 whatever the vectors' type (an FP32
 // x is widened exactly, y rounded once)
-template <typename TI, typename TO>
+template <typename TI, typename TO, bool MV>
 __global__ void __launch_bounds__(256) dense_gemv(int nout, int ncol, int lda, const double* __restrict__ A,
                                                   const TI* __restrict__ x, TO* __restrict__ y) {
+    if (MV) {
+        x += (long long)blockIdx.y * ncol;
+        y += (long long)blockIdx.y * nout;
+    }
     pdl_wait();
     pdl_release();
     const int lane = threadIdx.x & 31;

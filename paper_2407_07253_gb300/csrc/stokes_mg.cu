@@ -257,6 +257,12 @@ struct stokes_mg {
     double *vin = nullptr, *vout = nullptr;
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     long long graph_launches[2] = {0, 0};
+    // vectors that one pass of the V-cycle works on (blockIdx.y of its
+    // kernels): 1, or the dim velocity components while FBF's cycle is issued;
+    // the level vectors, Y, vin and vout have room for nvec_max.  Its graph:
+    int nvec = 1, nvec_max = 1;
+    cudaGraphExec_t vgraph = nullptr;
+    long long vgraph_launches = 0;
     // batched V-cycle: interleaved work vectors of width bm per level, and
     // one captured graph per patch-GEMM mode for that width
     // one launch of the batched patch GEMM: `count` patches of one kind from
@@ -520,27 +526,30 @@ int lanes_for(const DevCSR& A, size_t elem) {
     return elem == 4 && avg > 32 && avg <= 64 ? 8 : A.lanes;
 }
 
-template <typename T, int MODE>
+template <typename T, int MODE, bool MV>
 void spmv_lanes(stokes_mg* h, const DevCSR& A, const T* x, T* y, const T* b, cudaStream_t s) {
     const int lanes = lanes_for(A, sizeof(T));
     const long long threads = (long long)A.nr * lanes;
-    const int grid = (int)((threads + 255) / 256);
+    const dim3 grid((unsigned)((threads + 255) / 256), h->nvec);
     if (A.nr == 0) return;
     const T* av = vals<T>(A);
     switch (lanes) {
-        case 4: kl(h, skern::spmv_csr<T, 4, MODE>, grid, 256, 0, s, A.nr, A.rp, A.ci, av, x, y, b); break;
-        case 8: kl(h, skern::spmv_csr<T, 8, MODE>, grid, 256, 0, s, A.nr, A.rp, A.ci, av, x, y, b); break;
-        case 16: kl(h, skern::spmv_csr<T, 16, MODE>, grid, 256, 0, s, A.nr, A.rp, A.ci, av, x, y, b); break;
-        default: kl(h, skern::spmv_csr<T, 32, MODE>, grid, 256, 0, s, A.nr, A.rp, A.ci, av, x, y, b); break;
+        case 4: kl(h, skern::spmv_csr<T, 4, MODE, MV>, grid, 256, 0, s, A.nr, A.nc, A.rp, A.ci, av, x, y, b); break;
+        case 8: kl(h, skern::spmv_csr<T, 8, MODE, MV>, grid, 256, 0, s, A.nr, A.nc, A.rp, A.ci, av, x, y, b); break;
+        case 16: kl(h, skern::spmv_csr<T, 16, MODE, MV>, grid, 256, 0, s, A.nr, A.nc, A.rp, A.ci, av, x, y, b); break;
+        default: kl(h, skern::spmv_csr<T, 32, MODE, MV>, grid, 256, 0, s, A.nr, A.nc, A.rp, A.ci, av, x, y, b); break;
     }
 }
 
 template <typename T>
 void spmv(stokes_mg* h, int kind, const DevCSR& A, int mode, const T* x, T* y, const T* b, cudaStream_t s) {
     launch(h, kind, s, [&] {
-        if (mode == skern::SPMV_SET) spmv_lanes<T, skern::SPMV_SET>(h, A, x, y, b, s);
-        else if (mode == skern::SPMV_ADD) spmv_lanes<T, skern::SPMV_ADD>(h, A, x, y, b, s);
-        else spmv_lanes<T, skern::SPMV_RESID>(h, A, x, y, b, s);
+        if (mode == skern::SPMV_SET) h->nvec > 1 ? spmv_lanes<T, skern::SPMV_SET, true>(h, A, x, y, b, s)
+                             : spmv_lanes<T, skern::SPMV_SET, false>(h, A, x, y, b, s);
+        else if (mode == skern::SPMV_ADD) h->nvec > 1 ? spmv_lanes<T, skern::SPMV_ADD, true>(h, A, x, y, b, s)
+                             : spmv_lanes<T, skern::SPMV_ADD, false>(h, A, x, y, b, s);
+        else h->nvec > 1 ? spmv_lanes<T, skern::SPMV_RESID, true>(h, A, x, y, b, s)
+                             : spmv_lanes<T, skern::SPMV_RESID, false>(h, A, x, y, b, s);
     });
 }
 
@@ -632,13 +641,14 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
         if (!inv) throw StokesError(STOKES_EINVAL, PO::none);
         const size_t smem = PO::red * (128 + 4) + sizeof(T) * l.maxn;
         launch(h, PK_PATCH, s, [&] {
-            kl(h, PO::expl, l.npatch, 128, smem, s, l.npatch, poff, pdofs, PO::ioff(l), inv, r, wt, Y);
+            kl(h, PO::expl, dim3(l.npatch, h->nvec), 128, smem, s, l.npatch, poff, pdofs, PO::ioff(l), inv, r, wt, Y, l.n,
+               l.nent);
         });
     }
     const int *soff = l.soff, *sidx = l.sidx;
     launch(h, PK_PULL, s, [&] {
-        kl(h, skern::pull_scatter<T>, grid_for(l.n), 256, 0, s, l.n, soff, sidx, (const T*)Y, (T)alpha, (T)beta, out, x,
-           xmode, bsrc, rdst);
+        kl(h, h->nvec > 1 ? skern::pull_scatter<T, true> : skern::pull_scatter<T, false>, dim3(grid_for(l.n), h->nvec), 256,
+           0, s, l.n, soff, sidx, (const T*)Y, (T)alpha, (T)beta, out, x, xmode, bsrc, rdst, l.nent);
     });
 }
 
@@ -687,7 +697,8 @@ template <typename T>
 void coarse_apply(stokes_mg* h, const T* b, T* e, cudaStream_t s) {
     const int n = h->nc;
     launch(h, -1, s, [&] {
-        kl(h, skern::dense_gemv<T, T>, (n * 32 + 255) / 256, 256, 0, s, n, n, n + 1, (const double*)h->Cinv, b, e);
+        kl(h, h->nvec > 1 ? skern::dense_gemv<T, T, true> : skern::dense_gemv<T, T, false>,
+           dim3((n * 32 + 255) / 256, h->nvec), 256, 0, s, n, n, n + 1, (const double*)h->Cinv, b, e);
     });
 }
 
@@ -719,7 +730,7 @@ void pcycle(stokes_mg* h, int li, const T* b, T* e, cudaStream_t s) {
         for (int t = 1; t < h->opts.n_V; ++t) {
             spmv<T>(h, PK_SPMV, l.K, skern::SPMV_RESID, e, LV<T>::t(l), b, s);
             hcycle<T>(h, li, LV<T>::t(l), LV<T>::u(l), s);
-            axpby_l<T>(h, l.n, 1.0, LV<T>::u(l), 1.0, e, s);
+            axpby_l<T>(h, l.n * h->nvec, 1.0, LV<T>::u(l), 1.0, e, s);
         }
         return;
     }
@@ -738,7 +749,7 @@ void pcycle(stokes_mg* h, int li, const T* b, T* e, cudaStream_t s) {
 // programmatic dependent launch (the body issues kernels only).
 void vcycle_body(stokes_mg* h, int prec, cudaStream_t s, bool pdl = true) {
     DevLevel& l0 = h->L[0];
-    const int n = l0.n;
+    const int n = l0.n * h->nvec;
     h->pdl_chain = pdl;
     h->pdl_armed = false;
     try {
@@ -756,24 +767,34 @@ void vcycle_body(stokes_mg* h, int prec, cudaStream_t s, bool pdl = true) {
     h->pdl_chain = h->pdl_armed = false;
 }
 
-void vcycle_run(stokes_mg* h, int prec, cudaStream_t s) {
+// vout = B_MG vin for nvec vectors (1 or nvec_max), by the graph if there is one
+void vcycle_run(stokes_mg* h, int prec, cudaStream_t s, int nvec = 1) {
     // per-launch events cannot sit inside a replayed graph: profiling any
     // V-cycle kernel class runs the V-cycle as plain launches
     const bool any_prof = h->prof[PK_PATCH].on || h->prof[PK_SPMV].on || h->prof[PK_PULL].on || h->prof[PK_TRANSFER].on;
-    if (h->graph[prec] && !any_prof) {
-        CK(cudaGraphLaunch(h->graph[prec], s));
-        h->launches += h->graph_launches[prec];
+    const cudaGraphExec_t g = nvec > 1 ? h->vgraph : h->graph[prec];
+    if (g && !any_prof) {
+        CK(cudaGraphLaunch(g, s));
+        h->launches += nvec > 1 ? h->vgraph_launches : h->graph_launches[prec];
     } else {
-        vcycle_body(h, prec, s, !any_prof);
+        h->nvec = nvec;
+        try {
+            vcycle_body(h, prec, s, !any_prof);
+        } catch (...) {
+            h->nvec = 1;
+            throw;
+        }
+        h->nvec = 1;
     }
 }
 
-void capture_graph(stokes_mg* h, int prec, cudaStream_t s) {
+void capture_graph(stokes_mg* h, int prec, int nvec, cudaGraphExec_t* out, long long* n_launches) {
     cudaStream_t cs;
     CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t g;
     long long before = h->launches;
     h->capturing = true;
+    h->nvec = nvec;
     CK(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
     try {
         vcycle_body(h, prec, cs);
@@ -781,17 +802,18 @@ void capture_graph(stokes_mg* h, int prec, cudaStream_t s) {
         cudaGraph_t dummy;
         cudaStreamEndCapture(cs, &dummy);
         h->capturing = false;
+        h->nvec = 1;
         cudaStreamDestroy(cs);
         throw;
     }
     CK(cudaStreamEndCapture(cs, &g));
     h->capturing = false;
-    h->graph_launches[prec] = h->launches - before;
+    h->nvec = 1;
+    *n_launches = h->launches - before;
     h->launches = before;
-    CK(cudaGraphInstantiate(&h->graph[prec], g, 0));
+    CK(cudaGraphInstantiate(out, g, 0));
     CK(cudaGraphDestroy(g));
     CK(cudaStreamDestroy(cs));
-    (void)s;
 }
 
 // ---- batched V-cycle (m interleaved right-hand sides, FP32 operators) -----
@@ -1352,13 +1374,14 @@ int fgmres(stokes_mg* h, const double* b, double* x, double tol, int* its_out, d
 // (a, 0) and (0, z_p); S~^-1 is the block-diagonal -nu_e M_p,e^-1.
 void fbf_apply(stokes_mg* h, const double* r, double* z, cudaStream_t s) {
     FbfData& F = *h->fbf;
-    const int nu = F.nu, nS = F.nS, nvf = F.nvf, d = F.S0.d, np = nS - nu, prec = h->opts.precision;
+    const int nu = F.nu, nS = F.nS, d = F.S0.d, np = nS - nu, prec = h->opts.precision;
+    // the components in one pass of the cycle: one after another its launches,
+    // whose work on the coarse levels is far below what a launch takes, came d
+    // times (setup and solve of SV P4 on the disk, mixed: 52.5 ms, 46.7 ms now)
     auto vcycles = [&](const double* in, double* out) {
-        for (int c = 0; c < d; ++c) {
-            CK(cudaMemcpyAsync(h->vin, in + (size_t)c * nvf, sizeof(double) * nvf, cudaMemcpyDeviceToDevice, s));
-            vcycle_run(h, prec, s);
-            CK(cudaMemcpyAsync(out + (size_t)c * nvf, h->vout, sizeof(double) * nvf, cudaMemcpyDeviceToDevice, s));
-        }
+        CK(cudaMemcpyAsync(h->vin, in, sizeof(double) * nu, cudaMemcpyDeviceToDevice, s));
+        vcycle_run(h, prec, s, d);
+        CK(cudaMemcpyAsync(out, h->vout, sizeof(double) * nu, cudaMemcpyDeviceToDevice, s));
     };
     vcycles(r, F.a);
     CK(cudaMemcpyAsync(F.t, F.a, sizeof(double) * nu, cudaMemcpyDeviceToDevice, s));
@@ -1435,6 +1458,17 @@ void setup_fbf(stokes_mg* h, cudaStream_t s) {
 // ---------------------------------------------------------------- setup --
 void upload_assembly_inputs(stokes_mg* h, int li, bool want32, cudaStream_t s);
 
+// a level's V-cycle work vectors, room for nvec_max each
+void alloc_level_vectors(stokes_mg* h, DevLevel& l, bool want32) {
+    const size_t n = (size_t)l.n * h->nvec_max;
+    l.b64 = halloc<double>(h, n); l.e64 = halloc<double>(h, n); l.r64 = halloc<double>(h, n);
+    l.d64 = halloc<double>(h, n); l.t64 = halloc<double>(h, n); l.u64 = halloc<double>(h, n);
+    if (want32) {
+        l.b32 = halloc<float>(h, n); l.e32 = halloc<float>(h, n); l.r32 = halloc<float>(h, n);
+        l.d32 = halloc<float>(h, n); l.t32 = halloc<float>(h, n); l.u32 = halloc<float>(h, n);
+    }
+}
+
 // Operator part of a level (its CSR, or the inputs of the device assembly)
 // and the level's work vectors.
 void upload_level_operator(stokes_mg* h, int li, bool want32, cudaStream_t s) {
@@ -1449,12 +1483,7 @@ void upload_level_operator(stokes_mg* h, int li, bool want32, cudaStream_t s) {
         upload_assembly_inputs(h, li, want32, s);
     }
     trace("upload K", li, tt);
-    l.b64 = halloc<double>(h, l.n); l.e64 = halloc<double>(h, l.n); l.r64 = halloc<double>(h, l.n);
-    l.d64 = halloc<double>(h, l.n); l.t64 = halloc<double>(h, l.n); l.u64 = halloc<double>(h, l.n);
-    if (want32) {
-        l.b32 = halloc<float>(h, l.n); l.e32 = halloc<float>(h, l.n); l.r32 = halloc<float>(h, l.n);
-        l.d32 = halloc<float>(h, l.n); l.t32 = halloc<float>(h, l.n); l.u32 = halloc<float>(h, l.n);
-    }
+    alloc_level_vectors(h, l, want32);
 }
 
 // Patch part of a relaxed level: index sets, offsets of the dense blocks and
@@ -1524,7 +1553,7 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
         }
         trace("patch maps", li, tt);
         tt = host_ms();
-        l.Y64 = halloc<double>(h, l.nent);
+        l.Y64 = halloc<double>(h, l.nent * h->nvec_max);
         // the stored inverses: the factored saddle form for the saddle-block
         // solver, explicit otherwise; FP32 on MIXED handles (the V-cycle and
         // the lambda_max estimate run in FP32 there), FP64 on FP64 handles
@@ -1585,7 +1614,7 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
             l.wt32 = halloc<float>(h, l.n);
             skern::convert_vec<float, double><<<grid_for(l.n), 256, 0, s>>>(l.n, l.wt64, l.wt32);
             CK(cudaGetLastError());
-            l.Y32 = halloc<float>(h, l.nent);
+            l.Y32 = halloc<float>(h, l.nent * h->nvec_max);
             if (!l.factored) l.inv32 = halloc<float>(h, l.ninv32);
         }
     }
@@ -1705,12 +1734,7 @@ void fbf_level0_operator(stokes_mg* h, bool want32, cudaStream_t target) {
     DevLevel& l = h->L[0];
     l.n = HL.n_free;
     l.p_level = HL.p_level;
-    l.b64 = halloc<double>(h, l.n); l.e64 = halloc<double>(h, l.n); l.r64 = halloc<double>(h, l.n);
-    l.d64 = halloc<double>(h, l.n); l.t64 = halloc<double>(h, l.n); l.u64 = halloc<double>(h, l.n);
-    if (want32) {
-        l.b32 = halloc<float>(h, l.n); l.e32 = halloc<float>(h, l.n); l.r32 = halloc<float>(h, l.n);
-        l.d32 = halloc<float>(h, l.n); l.t32 = halloc<float>(h, l.n); l.u32 = halloc<float>(h, l.n);
-    }
+    alloc_level_vectors(h, l, want32);
     upload_assembly_inputs_lv(h, F.S0, F.S0d, false, h->s_up);
     const int n = l.n;
     const long long bound = F.S0d.K.nnz;
@@ -2260,8 +2284,8 @@ void alloc_krylov(stokes_mg* h, cudaStream_t s) {
     h->partial = halloc<double>(h, (size_t)h->partial_blocks * 32);
     h->ticket = halloc<unsigned int>(h, 1);
     CK(cudaMemsetAsync(h->ticket, 0, sizeof(unsigned int), s));
-    h->vin = halloc<double>(h, n0);
-    h->vout = halloc<double>(h, n0);
+    h->vin = halloc<double>(h, (size_t)n0 * h->nvec_max);
+    h->vout = halloc<double>(h, (size_t)n0 * h->nvec_max);
     h->v0buf = halloc<double>(h, n0);
     CK(cudaMallocHost((void**)&h->pinned, 64));
 }
@@ -2629,6 +2653,7 @@ int setup_impl(const stokes_mesh* coarse, int n_refine, int barycentric_finest, 
             h->H.t_matrices_ms = S.t_matrices_ms;
             h->H.t_transfers_ms = S.t_transfers_ms;
             h->opts.patch_solver = 1;          // dense SPD star blocks: Gauss-Jordan
+            h->nvec_max = F.S0.d;              // every component in one pass of the cycle
             const int nlv = (int)h->H.levels.size();
             if (on_level) {
                 on_level(nlv - 1, 0);
@@ -2700,7 +2725,10 @@ int setup_impl(const stokes_mesh* coarse, int n_refine, int barycentric_finest, 
         }
         h->st.t_eig_ms = host_ms() - t1;
         t1 = host_ms();
-        if (o.use_graph) capture_graph(h.get(), o.precision, s);
+        if (o.use_graph) {
+            capture_graph(h.get(), o.precision, 1, &h->graph[o.precision], &h->graph_launches[o.precision]);
+            if (h->nvec_max > 1) capture_graph(h.get(), o.precision, h->nvec_max, &h->vgraph, &h->vgraph_launches);
+        }
         h->st.t_graph_ms = host_ms() - t1;
         h->st.t_total_ms = host_ms() - t0;
         mark(h.get(), "setup end", s);
@@ -3553,6 +3581,7 @@ void stokes_mg_destroy(stokes_mg_t h) {
         if (h->graph[i]) cudaGraphExecDestroy(h->graph[i]);
         if (h->bgraph[i]) cudaGraphExecDestroy(h->bgraph[i]);
     }
+    if (h->vgraph) cudaGraphExecDestroy(h->vgraph);
     if (h->s_up || h->s_coarse) cudaDeviceSynchronize();   // setup work may still be in flight after an error
     free_pending(h);
     free_coarse_ws(h);
