@@ -1072,6 +1072,286 @@ __global__ void __launch_bounds__(256) saddle_inverse_global(int npatch, int d, 
     if (threadIdx.x == 0) status[p] = st;
 }
 
+// ---- large patches: the symmetric sweep on 4 x 4 tiles ------------------
+// Factored form of patches beyond saddle_inverse_smem's shared memory (stars of
+// TH P6 and up, SV P4, 3D P3).  One pivot at a time in a global scratch costs a
+// read and a write of the whole block per pivot, from L2; here the upper
+// triangle's 4 x 4 tiles stay in shared memory and a step sweeps four pivots:
+//   U = A[K, :] (4 x n, published), P = A[K, K]^-1 (one warp), V = P U,
+//   A -= U^T V on every tile (64 FMAs between 128 bytes read and written), and
+//   row K becomes V, A[K, K] becomes -P; after the last step A holds -A^-1.
+// The FP64 pipe (2 FMA lanes per SM and clock) bounds it: 1089 patches of the
+// P8 stars on 32 x 32 took 38.2 ms, NEW_P8 now; the padding to tiles adds 4% to the
+// FMAs at 217 nodes, the 4 x 4 inverses and V another 8%.
+// A tile's entry (r, c) is double c & 1 of 16-byte group 2 r + c / 2, groups
+// [8][ntile], so that the threads of a warp, on consecutive tiles, read and
+// write them without bank conflicts.
+__device__ __forceinline__ int tile_row(int n4, int I) { return I * n4 - I * (I - 1) / 2 - I; }   // + J: tile (I, J)
+__device__ __forceinline__ double& tile_at(double2* T, int ntile, int t, int r, int c) {
+    return reinterpret_cast<double*>(T)[((size_t)(2 * r + (c >> 1)) * ntile + t) * 2 + (c & 1)];
+}
+
+// the tiles' places: map[t] = (I, J)
+__device__ __forceinline__ void tile_map(int n4, ushort2* map) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int I = warp; I < n4; I += nw)
+        for (int J = I + lane; J < n4; J += 32) map[tile_row(n4, I) + J] = make_ushort2(I, J);
+}
+
+// All threads of the CTA; T, U [4][4 n4], V [4][4 n4], P [16] in shared memory.
+// status <- 1 + step of the first non-positive pivot.
+__device__ void sweep_tiles(double2* T, int n4, const ushort2* map, double* U, double* V, double* P, int* status) {
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
+    const int ntile = n4 * (n4 + 1) / 2, ldu = 4 * n4;
+    for (int K = 0; K < n4; ++K) {
+        for (int x = tid; x < 16 * n4; x += nt) {
+            const int J = x >> 4, k = (x >> 2) & 3, c = x & 3;
+            U[k * ldu + 4 * J + c] = J >= K ? tile_at(T, ntile, tile_row(n4, K) + J, k, c)
+                                            : tile_at(T, ntile, tile_row(n4, J) + K, c, k);
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // the 4 x 4 sweep, one entry per lane (the upper half-warp repeats the lower)
+            const int r = (lane >> 2) & 3, c = lane & 3;
+            double v = U[r * ldu + 4 * K + c];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const double piv = __shfl_sync(0xffffffffu, v, 5 * k);
+                const double vrk = __shfl_sync(0xffffffffu, v, 4 * r + k), vkc = __shfl_sync(0xffffffffu, v, 4 * k + c);
+                const double inv = piv > 0.0 ? 1.0 / piv : 0.0;
+                if (lane == 0 && !(piv > 0.0) && *status == 0) *status = 4 * K + k + 1;
+                const double w = vrk * inv;
+                v = r == k ? (c == k ? flip(inv) : vkc * inv) : (c == k ? w : fma(-w, vkc, v));
+            }
+            if (lane < 16) P[lane] = flip(v);
+        }
+        __syncthreads();
+        for (int j = tid; j < ldu; j += nt) {
+            double u[4];
+#pragma unroll
+            for (int l = 0; l < 4; ++l) u[l] = U[l * ldu + j];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                double v = P[4 * k] * u[0];
+#pragma unroll
+                for (int l = 1; l < 4; ++l) v = fma(P[4 * k + l], u[l], v);
+                V[k * ldu + j] = v;
+            }
+        }
+        __syncthreads();
+        for (int t = tid; t < ntile; t += nt) {
+            const int I = map[t].x, J = map[t].y;
+            double a[4][4];
+            if (I == K || J == K) {
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        a[r][c] = I == J ? flip(P[4 * r + c]) : I == K ? V[r * ldu + 4 * J + c] : V[c * ldu + 4 * I + r];
+            } else {
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const double2 x = T[(size_t)(2 * r + h) * ntile + t];
+                        a[r][2 * h] = x.x;
+                        a[r][2 * h + 1] = x.y;
+                    }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const double2 u0 = *reinterpret_cast<const double2*>(U + k * ldu + 4 * I);
+                    const double2 u1 = *reinterpret_cast<const double2*>(U + k * ldu + 4 * I + 2);
+                    const double2 v0 = *reinterpret_cast<const double2*>(V + k * ldu + 4 * J);
+                    const double2 v1 = *reinterpret_cast<const double2*>(V + k * ldu + 4 * J + 2);
+                    const double u[4] = {u0.x, u0.y, u1.x, u1.y}, v[4] = {v0.x, v0.y, v1.x, v1.y};
+#pragma unroll
+                    for (int r = 0; r < 4; ++r)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) a[r][c] = fma(-u[r], v[c], a[r][c]);
+                }
+            }
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+#pragma unroll
+                for (int h = 0; h < 2; ++h) T[(size_t)(2 * r + h) * ntile + t] = make_double2(a[r][2 * h], a[r][2 * h + 1]);
+        }
+        __syncthreads();
+    }
+}
+
+// zero tiles with a unit diagonal behind row n
+__device__ __forceinline__ void tiles_clear(double2* T, int n, int n4) {
+    const int ntile = n4 * (n4 + 1) / 2;
+    for (int t = threadIdx.x; t < 8 * ntile; t += blockDim.x) T[t] = make_double2(0.0, 0.0);
+    __syncthreads();
+    for (int i = n + threadIdx.x; i < 4 * n4; i += blockDim.x)
+        tile_at(T, ntile, tile_row(n4, i >> 2) + (i >> 2), i & 3, i & 3) = 1.0;
+}
+
+// One CTA per listed patch; its part of the global scratch (saddle_tiles_scratch)
+// holds W row by row, and per pressure column the entries of B_c^T (position,
+// value), component after component.
+template <int NT>
+__device__ __forceinline__ void saddle_tiles_body(
+    int d, const int* __restrict__ list, const int* __restrict__ poff, const int* __restrict__ pnv,
+    const long long* __restrict__ foff64, double* __restrict__ fac64, const long long* __restrict__ foff32,
+    float* __restrict__ fac32, int packed, const int* __restrict__ pdofs, const int* __restrict__ rp,
+    const int* __restrict__ ci, const double* __restrict__ av, int max4, int max_np, const long long* __restrict__ soff,
+    double* scratch, int* __restrict__ status, unsigned char* smem) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int maxt = max4 * (max4 + 1) / 2;
+    double2* T = reinterpret_cast<double2*>(smem);                                     // [8][ntile]
+    double* U = reinterpret_cast<double*>(T + 8 * (size_t)maxt);                       // [4][4 max4]
+    double* V = U + 16 * max4;                                                         // [4][4 max4]
+    double* P = V + 16 * max4;                                                         // [16]
+    ushort2* map = reinterpret_cast<ushort2*>(P + 16);                                 // [maxt]
+    int* coff = reinterpret_cast<int*>(map + maxt);                                    // [np][d + 1]
+    int* sd = coff + max_np * (d + 1);                                                 // [n]
+    __shared__ int st;
+    const int p = list[blockIdx.x], s0 = poff[p], n = poff[p + 1] - s0, nv = pnv[p];
+    const int dnv = d * nv, np = n - dnv, npl = (np + 3) & ~3;
+    double* Wr = scratch + soff[blockIdx.x];                                           // [d nv][npl]
+    double* lv = Wr + (long long)dnv * npl;                                            // [np][d nv]
+    int* lp = reinterpret_cast<int*>(lv + (long long)dnv * np);                        // [np][d nv]
+    const int n4 = (nv + 3) >> 2, q4 = (np + 3) >> 2;
+    const int vec = fac64 ? 2 : 4;
+    const int ldl = (nv + vec - 1) / vec * vec, ldw = (dnv + vec - 1) / vec * vec, lds = (np + vec - 1) / vec * vec;
+    const long long lenL = packed ? ((long long)nv * (nv + 1) / 2 + vec - 1) / vec * vec : (long long)ldl * nv;
+    const long long oW = lenL, oS = oW + (long long)ldw * np;
+    double* f64 = fac64 ? fac64 + foff64[p] : nullptr;
+    float* f32 = fac32 ? fac32 + foff32[p] : nullptr;
+    auto put = [&](long long o, double v) {
+        if (f64) f64[o] = v;
+        if (f32) f32[o] = (float)v;
+    };
+    if (tid == 0) st = 0;
+    for (int a = tid; a < n; a += NT) sd[a] = pdofs[s0 + a];
+    tile_map(n4, map);
+    tiles_clear(T, nv, n4);
+    __syncthreads();
+    int ntile = n4 * (n4 + 1) / 2;
+    // the velocity block, from the rows of component 0
+    for (int i = warp; i < nv; i += NW) {
+        const int g = sd[i], e = rp[g + 1];
+        for (int q = rp[g] + lane; q < e; q += 32) {
+            const int pos = patch_pos(sd, n, ci[q]);
+            if (pos < nv && pos >= 0 && (pos >> 2) >= (i >> 2))
+                tile_at(T, ntile, tile_row(n4, i >> 2) + (pos >> 2), i & 3, pos & 3) = av[q];
+        }
+    }
+    // B's columns, from the pressure rows (a warp per row, an order that
+    // depends on the row alone)
+    for (int q = warp; q < np; q += NW) {
+        const int g = sd[dnv + q], b0 = rp[g], e = rp[g + 1];
+        int k = 0;
+        for (int c = 0; c < d; ++c) {
+            if (lane == 0) coff[q * (d + 1) + c] = k;
+            for (int x0 = b0; x0 < e; x0 += 32) {
+                const int x = x0 + lane;
+                const int pos = x < e ? patch_pos(sd, n, ci[x]) : -1;
+                const bool in = pos >= c * nv && pos < (c + 1) * nv;
+                const unsigned m = __ballot_sync(0xffffffffu, in);
+                if (in) {
+                    const int at = k + __popc(m & ((1u << lane) - 1u));
+                    lp[(long long)q * dnv + at] = pos - c * nv;
+                    lv[(long long)q * dnv + at] = av[x];
+                }
+                k += __popc(m);
+            }
+        }
+        if (lane == 0) coff[q * (d + 1) + d] = k;
+    }
+    __syncthreads();
+    sweep_tiles(T, n4, map, U, V, P, &st);
+    // Li = -tiles
+    auto li = [&](int a, int b) {
+        return a <= b ? tile_at(T, ntile, tile_row(n4, a >> 2) + (b >> 2), a & 3, b & 3)
+                      : tile_at(T, ntile, tile_row(n4, b >> 2) + (a >> 2), b & 3, a & 3);
+    };
+    if (packed) {
+        for (int a = warp; a < nv; a += NW) {
+            const long long o = (long long)a * nv - (long long)a * (a - 1) / 2 - a;
+            for (int b = a + lane; b < nv; b += 32) put(o + b, flip(li(a, b)));
+        }
+        for (long long t = (long long)nv * (nv + 1) / 2 + tid; t < lenL; t += NT) put(t, 0.0);
+    } else {
+        for (int b = warp; b < nv; b += NW)
+            for (int a = lane; a < ldl; a += 32) put((long long)b * ldl + a, a < nv ? flip(li(a, b)) : 0.0);
+    }
+    for (int t = tid; t < np * (ldw - dnv); t += NT) {
+        const int q = t / (ldw - dnv);
+        put(oW + (long long)q * ldw + dnv + (t - q * (ldw - dnv)), 0.0);
+    }
+    // W_c = Li B_c^T: a warp takes column q for 32 rows
+    const int nh = (nv + 31) >> 5;
+    for (int it = warp; it < np * nh; it += NW) {
+        const int q = it / nh, a = (it - q * nh) * 32 + lane, aa = min(a, nv - 1);
+        for (int c = 0; c < d; ++c) {
+            const int k0 = coff[q * (d + 1) + c], k1 = coff[q * (d + 1) + c + 1];
+            double acc = 0.0;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k) acc = fma(li(aa, lp[(long long)q * dnv + k]), lv[(long long)q * dnv + k], acc);
+            if (a < nv) {
+                const double w = flip(acc);
+                put(oW + (long long)q * ldw + c * nv + a, w);
+                Wr[(long long)(c * nv + a) * npl + q] = w;
+            }
+        }
+    }
+    __syncthreads();
+    // S = sum_c B_c W_c: a warp takes row q for 32 columns r >= q
+    tile_map(q4, map);
+    tiles_clear(T, np, q4);
+    __syncthreads();
+    ntile = q4 * (q4 + 1) / 2;
+    const int nc = (np + 31) >> 5;
+    for (int it = warp; it < np * nc; it += NW) {
+        const int q = it / nc, ch = it - q * nc, r = ch * 32 + lane;
+        if (32 * ch + 31 < q) continue;
+        const double* w = Wr + min(r, np - 1);
+        double acc = 0.0;
+        for (int c = 0; c < d; ++c) {
+            const int k0 = coff[q * (d + 1) + c], k1 = coff[q * (d + 1) + c + 1];
+            const double* wc = w + (long long)c * nv * npl;
+#pragma unroll 4
+            for (int k = k0; k < k1; ++k)
+                acc = fma(lv[(long long)q * dnv + k], wc[(long long)lp[(long long)q * dnv + k] * npl], acc);
+        }
+        if (r < np && r >= q) {
+            tile_at(T, ntile, tile_row(q4, q >> 2) + (r >> 2), q & 3, r & 3) = acc;
+            if ((q >> 2) == (r >> 2)) tile_at(T, ntile, tile_row(q4, q >> 2) + (r >> 2), r & 3, q & 3) = acc;
+        }
+    }
+    __syncthreads();
+    sweep_tiles(T, q4, map, U, V, P, &st);
+    for (int r = warp; r < np; r += NW)
+        for (int q = lane; q < lds; q += 32) {
+            double v = 0.0;
+            if (q < np) {
+                const int x = min(q, r), y = max(q, r);
+                v = flip(tile_at(T, ntile, tile_row(q4, x >> 2) + (y >> 2), x & 3, y & 3));
+            }
+            put(oS + (long long)r * lds + q, v);
+        }
+    if (tid == 0) status[p] = st;
+}
+
+#define SADDLE_TILES_KERNEL(NAME, NT)                                                                                  \
+    __global__ void __launch_bounds__(NT, 512 / NT) NAME(                                                              \
+        int d, const int* __restrict__ list, const int* __restrict__ poff, const int* __restrict__ pnv,                \
+        const long long* __restrict__ foff64, double* __restrict__ fac64, const long long* __restrict__ foff32,        \
+        float* __restrict__ fac32, int packed, const int* __restrict__ pdofs, const int* __restrict__ rp,              \
+        const int* __restrict__ ci, const double* __restrict__ av, int max4, int max_np,                               \
+        const long long* __restrict__ soff, double* scratch, int* __restrict__ status) {                               \
+        extern __shared__ __align__(16) unsigned char smem_st[];                                                       \
+        saddle_tiles_body<NT>(d, list, poff, pnv, foff64, fac64, foff32, fac32, packed, pdofs, rp, ci, av, max4,       \
+                              max_np, soff, scratch, status, smem_st);                                                 \
+    }
+SADDLE_TILES_KERNEL(saddle_inverse_tiles_512, 512)
+SADDLE_TILES_KERNEL(saddle_inverse_tiles_256, 256)
+#undef SADDLE_TILES_KERNEL
+
 // One ASM sweep.  The patch inverse is column-major with its leading
 // dimension padded to VEC rows; a thread owns VEC consecutive rows (one
 // 16-byte vector per column) and the columns are split among G groups of

@@ -233,6 +233,28 @@ __global__ void saddle_inverse_global(int npatch, int d, const int* __restrict__
                                       const long long* __restrict__ foff32, float* __restrict__ fac32, int back,
                                       int packed, long long max_scratch, const long long* __restrict__ soff,
                                       double* __restrict__ scratch, int* __restrict__ status);
+// The factored form of the listed patches from the CSR operator, on 4 x 4 tiles
+// in shared memory, one CTA of 512 or 256 threads per patch.  max4: the largest
+// of nv and np in tiles of four; max_np, max_n: the largest np and n; soff: each
+// listed patch's place in the scratch (saddle_tiles_scratch doubles).
+constexpr size_t SADDLE_TILES_SMEM_MAX = 226 * 1024;
+__host__ __device__ inline size_t saddle_tiles_smem(int d, int max4, int max_np, int max_n) {
+    const size_t nt = (size_t)max4 * (max4 + 1) / 2;
+    return nt * (128 + 4) + sizeof(double) * (32 * (size_t)max4 + 16) + sizeof(int) * ((size_t)max_np * (d + 1) + max_n);
+}
+__host__ __device__ inline long long saddle_tiles_scratch(int d, int n, int nv) {
+    const long long dnv = (long long)d * nv, np = n - dnv;
+    return dnv * ((np + 3) & ~3LL) + dnv * np + (dnv * np + 1) / 2;
+}
+#define SADDLE_TILES_ARGS                                                                                              \
+    int d, const int *__restrict__ list, const int *__restrict__ poff, const int *__restrict__ pnv,                    \
+        const long long *__restrict__ foff64, double *__restrict__ fac64, const long long *__restrict__ foff32,        \
+        float *__restrict__ fac32, int packed, const int *__restrict__ pdofs, const int *__restrict__ rp,              \
+        const int *__restrict__ ci, const double *__restrict__ av, int max4, int max_np,                               \
+        const long long *__restrict__ soff, double *scratch, int *__restrict__ status
+__global__ void saddle_inverse_tiles_512(SADDLE_TILES_ARGS);
+__global__ void saddle_inverse_tiles_256(SADDLE_TILES_ARGS);
+#undef SADDLE_TILES_ARGS
 // Elements of one patch's factored inverse (Li, W, Si with leading
 // dimensions rounded up to vec = 2 (FP64) or 4 (FP32)); packed: Li as its
 // upper triangle row by row (nv (nv + 1) / 2 entries, rounded up to vec),

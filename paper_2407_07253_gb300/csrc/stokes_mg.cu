@@ -160,6 +160,11 @@ struct DevLevel {
     long long saddle_smem_fac = 0;  // the same for the factored-only inversion
     long long saddle_global = 0;    // total scratch (doubles) of the others
     long long* scoff = nullptr;     // their offsets into the global scratch
+    // the tiled inversion of those patches (tl_count 0: none, or one too large for it)
+    int tl_count = 0, tl_max4 = 0, tl_np = 0, tl_n = 0;
+    int* tl_list = nullptr;
+    long long* tl_soff = nullptr;   // places in its scratch of tl_scratch doubles
+    long long tl_scratch = 0;
     long long ninv64 = 0, ninv32 = 0;
     double* inv64 = nullptr;            // explicit inverses (Gauss-Jordan patches; FP32 also for the batched path)
     float* inv32 = nullptr;
@@ -1513,7 +1518,8 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
         l.pdofs = hupload(h, HL.patch_dofs, s);
         l.pnv = hupload(h, HL.patch_nv, s);
         trace("patch lists uploaded", li, tt);
-        std::vector<long long> scoff(l.npatch + 1, 0);
+        std::vector<long long> scoff(l.npatch + 1, 0), tl_soff;
+        std::vector<int> tl_list;
         for (int p = 0; p < l.npatch; ++p) {
             const long long sc = skern::saddle_scratch(HL.d, HL.patch_off[p + 1] - HL.patch_off[p], HL.patch_nv[p]);
             if (sc <= skern::SADDLE_SMEM_MAX_DOUBLES) {
@@ -1523,10 +1529,24 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
                                                                     HL.patch_nv[p]));
                 scoff[p + 1] = scoff[p];
             }
-            else
+            else {
+                const int n = HL.patch_off[p + 1] - HL.patch_off[p], nv = HL.patch_nv[p], np = n - HL.d * nv;
+                l.tl_max4 = std::max(l.tl_max4, (std::max(nv, np) + 3) / 4);
+                l.tl_np = std::max(l.tl_np, np);
+                l.tl_n = std::max(l.tl_n, n);
+                tl_list.push_back(p);
+                tl_soff.push_back(l.tl_scratch);
+                l.tl_scratch += skern::saddle_tiles_scratch(HL.d, n, nv);
                 scoff[p + 1] = scoff[p] + std::max(sc, skern::saddle_scratch_factored(
                                                            HL.d, HL.patch_off[p + 1] - HL.patch_off[p], HL.patch_nv[p],
                                                            false));
+            }
+        }
+        if (!tl_list.empty() &&
+            skern::saddle_tiles_smem(HL.d, l.tl_max4, l.tl_np, l.tl_n) <= skern::SADDLE_TILES_SMEM_MAX) {
+            l.tl_count = (int)tl_list.size();
+            l.tl_list = hupload(h, tl_list, s);
+            l.tl_soff = hupload(h, tl_soff, s);
         }
         l.saddle_global = scoff[l.npatch];
         l.scoff = hupload(h, scoff, s);
@@ -1903,10 +1923,28 @@ void build_transfer_dev(stokes_mg* h, int li, bool want32, const std::function<v
 // gather K_i and invert every patch of level li; work receives the
 // row-major inverses (sum n_i^2 doubles) when keep != nullptr.
 // whether level li's factored inverses are computed straight from its CSR
-// operator (every patch inverted in shared memory, with room for its DoF list)
+// operator: every patch inverted in shared memory, the small ones with room
+// for their DoF list, the others (if any) by the tiled kernel
 bool fused_factor(const stokes_mg* h, const DevLevel& l) {
-    return h->opts.patch_solver == 0 && !l.inv64 && !l.inv32 && l.saddle_global == 0 && l.saddle_smem > 0 &&
+    return h->opts.patch_solver == 0 && !l.inv64 && !l.inv32 && (l.saddle_global == 0 || l.tl_count > 0) &&
+           (l.saddle_smem > 0 || l.saddle_global > 0) &&
            l.saddle_smem_fac + (l.maxn + 1) / 2 <= skern::SADDLE_SMEM_MAX_DOUBLES;
+}
+
+// the tiled inversion of a level's large patches (512 threads a CTA where the
+// tiles fill an SM's shared memory, 256 where two CTAs fit)
+void launch_tiles(stokes_mg* h, DevLevel& l, double* f64, float* f32, int* status, cudaStream_t s) {
+    const size_t smem = skern::saddle_tiles_smem(h->dim, l.tl_max4, l.tl_np, l.tl_n);
+    const bool two = 2 * (smem + 2048) <= 227 * 1024;
+    auto kern = two ? skern::saddle_inverse_tiles_256 : skern::saddle_inverse_tiles_512;
+    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)skern::SADDLE_TILES_SMEM_MAX));
+    double* scr = palloc<double>(h->device, l.tl_scratch, s);
+    launch(h, PK_GJ, s, [&] {
+        kern<<<l.tl_count, two ? 256 : 512, smem, s>>>(h->dim, l.tl_list, l.poff, l.pnv, l.foff64, f64, l.foff32, f32,
+                                                       l.fac_packed ? 1 : 0, l.pdofs, l.K.rp, l.K.ci, l.K.v64, l.tl_max4,
+                                                       l.tl_np, l.tl_soff, scr, status);
+    });
+    CK(cudaFreeAsync(scr, s));
 }
 
 void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status, cudaStream_t s) {
@@ -1944,7 +1982,9 @@ void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status,
                     l.K.v64, (int)sd_off, status);
             });
         }
-        if (l.saddle_global > 0) {
+        if (l.saddle_global > 0 && fused) {
+            launch_tiles(h, l, f64, f32, status, s);
+        } else if (l.saddle_global > 0) {
             // scratch of the patches too large for shared memory, from the
             // stream-ordered pool (freed on the same stream, no host wait)
             double* scr = palloc<double>(h->device, l.saddle_global, s);
