@@ -1017,14 +1017,14 @@ __global__ void __launch_bounds__(256) saddle_inverse_smem(int npatch, int d, co
                                                            float* __restrict__ inv32, const long long* __restrict__ foff64,
                                                            double* __restrict__ fac64, const long long* __restrict__ foff32,
                                                            float* __restrict__ fac32, int back, int packed,
-                                                           long long max_scratch, const int* __restrict__ pdofs,
+                                                           long long max_scratch, int skip_from, const int* __restrict__ pdofs,
                                                            const int* __restrict__ rp, const int* __restrict__ ci,
                                                            const double* __restrict__ av, int sd_off,
                                                            int* __restrict__ status) {
     extern __shared__ double sscr[];
     const int p = blockIdx.x;
     const int n = poff[p + 1] - poff[p], nv = pnv[p];
-    if (n == 0 || saddle_scratch(d, n, nv) > max_scratch) return;
+    if (n == 0 || saddle_scratch(d, n, nv) > max_scratch || max(nv, n - d * nv) >= skip_from) return;
     __shared__ int st;
     int* sd = reinterpret_cast<int*>(sscr + sd_off);
     if (!work && (inv64 || inv32 || back)) {      // the explicit forms need the dense block
@@ -1350,6 +1350,7 @@ __device__ __forceinline__ void saddle_tiles_body(
     }
 SADDLE_TILES_KERNEL(saddle_inverse_tiles_512, 512)
 SADDLE_TILES_KERNEL(saddle_inverse_tiles_256, 256)
+SADDLE_TILES_KERNEL(saddle_inverse_tiles_128, 128)
 #undef SADDLE_TILES_KERNEL
 
 // One ASM sweep.  The patch inverse is column-major with its leading

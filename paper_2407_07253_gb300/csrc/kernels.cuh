@@ -209,6 +209,7 @@ __host__ __device__ inline long long saddle_scratch_factored(int d, int n, int n
     const int mx = nv > np ? nv : np;
     return (pp ? pp_size(nv) : (long long)nv * nv) + 2LL * nv * npp + (long long)np * np + 7LL * mx + 2 + (long long)np * ((nv + 63) / 64);
 }
+// (saddle_inverse_smem leaves patches with max(nv, np) >= skip_from alone.)
 // Outputs (each may be NULL): explicit inverses inv64 / inv32 (column-major,
 // leading dimension n rounded up to 2 / 4), the factored form fac64 / fac32
 // at foff64[p] / foff32[p] (saddle_factor_len), and, if back, the explicit
@@ -222,7 +223,7 @@ __global__ void saddle_inverse_smem(int npatch, int d, const int* __restrict__ p
                                     const long long* __restrict__ off32, float* __restrict__ inv32,
                                     const long long* __restrict__ foff64, double* __restrict__ fac64,
                                     const long long* __restrict__ foff32, float* __restrict__ fac32, int back,
-                                    int packed, long long max_scratch, const int* __restrict__ pdofs,
+                                    int packed, long long max_scratch, int skip_from, const int* __restrict__ pdofs,
                                     const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ av,
                                     int sd_off, int* __restrict__ status);
 __global__ void saddle_inverse_global(int npatch, int d, const int* __restrict__ poff, const int* __restrict__ pnv,
@@ -238,6 +239,11 @@ __global__ void saddle_inverse_global(int npatch, int d, const int* __restrict__
 // of nv and np in tiles of four; max_np, max_n: the largest np and n; soff: each
 // listed patch's place in the scratch (saddle_tiles_scratch doubles).
 constexpr size_t SADDLE_TILES_SMEM_MAX = 226 * 1024;
+// Patches of max(nv, np) from here on are tiled even where the pivot-pair
+// kernel's shared memory would hold them: the P5 level (91 nodes) of the P8
+// hierarchy takes setup and solve from 50.2 to 48.4 ms; at 61 nodes (P4, where
+// the 4 x 4 inverses and the padding weigh more) it is 2.42 ms against 2.81.
+constexpr int SADDLE_TILES_MIN_N = 80;
 __host__ __device__ inline size_t saddle_tiles_smem(int d, int max4, int max_np, int max_n) {
     const size_t nt = (size_t)max4 * (max4 + 1) / 2;
     return nt * (128 + 4) + sizeof(double) * (32 * (size_t)max4 + 16) + sizeof(int) * ((size_t)max_np * (d + 1) + max_n);
@@ -254,6 +260,7 @@ __host__ __device__ inline long long saddle_tiles_scratch(int d, int n, int nv) 
         const long long *__restrict__ soff, double *scratch, int *__restrict__ status
 __global__ void saddle_inverse_tiles_512(SADDLE_TILES_ARGS);
 __global__ void saddle_inverse_tiles_256(SADDLE_TILES_ARGS);
+__global__ void saddle_inverse_tiles_128(SADDLE_TILES_ARGS);
 #undef SADDLE_TILES_ARGS
 // Elements of one patch's factored inverse (Li, W, Si with leading
 // dimensions rounded up to vec = 2 (FP64) or 4 (FP32)); packed: Li as its

@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <numeric>
 #include <chrono>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -162,6 +163,8 @@ struct DevLevel {
     long long* scoff = nullptr;     // their offsets into the global scratch
     // the tiled inversion of those patches (tl_count 0: none, or one too large for it)
     int tl_count = 0, tl_max4 = 0, tl_np = 0, tl_n = 0;
+    int tl_min = INT_MAX;           // smaller ones too, from this max(nv, np)
+    int sm_n = 0;                   // the largest patch left to the shared-memory kernel
     int* tl_list = nullptr;
     long long* tl_soff = nullptr;   // places in its scratch of tl_scratch doubles
     long long tl_scratch = 0;
@@ -1518,35 +1521,43 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
         l.pdofs = hupload(h, HL.patch_dofs, s);
         l.pnv = hupload(h, HL.patch_nv, s);
         trace("patch lists uploaded", li, tt);
-        std::vector<long long> scoff(l.npatch + 1, 0), tl_soff;
-        std::vector<int> tl_list;
-        for (int p = 0; p < l.npatch; ++p) {
-            const long long sc = skern::saddle_scratch(HL.d, HL.patch_off[p + 1] - HL.patch_off[p], HL.patch_nv[p]);
-            if (sc <= skern::SADDLE_SMEM_MAX_DOUBLES) {
-                l.saddle_smem = std::max(l.saddle_smem, sc);
-                l.saddle_smem_fac = std::max(l.saddle_smem_fac, skern::saddle_scratch_factored(
-                                                                    HL.d, HL.patch_off[p + 1] - HL.patch_off[p],
-                                                                    HL.patch_nv[p]));
-                scoff[p + 1] = scoff[p];
-            }
-            else {
+        // patches of the tiled inversion (factored form, all of a level's large ones or none)
+        {
+            std::vector<long long> soff;
+            std::vector<int> list;
+            for (int p = 0; p < l.npatch; ++p) {
                 const int n = HL.patch_off[p + 1] - HL.patch_off[p], nv = HL.patch_nv[p], np = n - HL.d * nv;
+                if (skern::saddle_scratch(HL.d, n, nv) <= skern::SADDLE_SMEM_MAX_DOUBLES && std::max(nv, np) < skern::SADDLE_TILES_MIN_N)
+                    continue;
                 l.tl_max4 = std::max(l.tl_max4, (std::max(nv, np) + 3) / 4);
                 l.tl_np = std::max(l.tl_np, np);
                 l.tl_n = std::max(l.tl_n, n);
-                tl_list.push_back(p);
-                tl_soff.push_back(l.tl_scratch);
+                list.push_back(p);
+                soff.push_back(l.tl_scratch);
                 l.tl_scratch += skern::saddle_tiles_scratch(HL.d, n, nv);
-                scoff[p + 1] = scoff[p] + std::max(sc, skern::saddle_scratch_factored(
-                                                           HL.d, HL.patch_off[p + 1] - HL.patch_off[p], HL.patch_nv[p],
-                                                           false));
+            }
+            if (!list.empty() &&
+                skern::saddle_tiles_smem(HL.d, l.tl_max4, l.tl_np, l.tl_n) <= skern::SADDLE_TILES_SMEM_MAX) {
+                l.tl_count = (int)list.size();
+                l.tl_min = skern::SADDLE_TILES_MIN_N;
+                l.tl_list = hupload(h, list, s);
+                l.tl_soff = hupload(h, soff, s);
             }
         }
-        if (!tl_list.empty() &&
-            skern::saddle_tiles_smem(HL.d, l.tl_max4, l.tl_np, l.tl_n) <= skern::SADDLE_TILES_SMEM_MAX) {
-            l.tl_count = (int)tl_list.size();
-            l.tl_list = hupload(h, tl_list, s);
-            l.tl_soff = hupload(h, tl_soff, s);
+        std::vector<long long> scoff(l.npatch + 1, 0);
+        for (int p = 0; p < l.npatch; ++p) {
+            const int n = HL.patch_off[p + 1] - HL.patch_off[p], nv = HL.patch_nv[p];
+            const long long sc = skern::saddle_scratch(HL.d, n, nv);
+            if (sc <= skern::SADDLE_SMEM_MAX_DOUBLES) {
+                l.saddle_smem = std::max(l.saddle_smem, sc);
+                if (std::max(nv, n - HL.d * nv) < l.tl_min) {
+                    l.saddle_smem_fac = std::max(l.saddle_smem_fac, skern::saddle_scratch_factored(HL.d, n, nv));
+                    l.sm_n = std::max(l.sm_n, n);
+                }
+                scoff[p + 1] = scoff[p];
+            }
+            else
+                scoff[p + 1] = scoff[p] + std::max(sc, skern::saddle_scratch_factored(HL.d, n, nv, false));
         }
         l.saddle_global = scoff[l.npatch];
         l.scoff = hupload(h, scoff, s);
@@ -1927,20 +1938,20 @@ void build_transfer_dev(stokes_mg* h, int li, bool want32, const std::function<v
 // for their DoF list, the others (if any) by the tiled kernel
 bool fused_factor(const stokes_mg* h, const DevLevel& l) {
     return h->opts.patch_solver == 0 && !l.inv64 && !l.inv32 && (l.saddle_global == 0 || l.tl_count > 0) &&
-           (l.saddle_smem > 0 || l.saddle_global > 0) &&
-           l.saddle_smem_fac + (l.maxn + 1) / 2 <= skern::SADDLE_SMEM_MAX_DOUBLES;
+           (l.sm_n > 0 || l.tl_count > 0) &&
+           l.saddle_smem_fac + (l.sm_n + 1) / 2 <= skern::SADDLE_SMEM_MAX_DOUBLES;
 }
 
 // the tiled inversion of a level's large patches (512 threads a CTA where the
 // tiles fill an SM's shared memory, 256 where two CTAs fit)
 void launch_tiles(stokes_mg* h, DevLevel& l, double* f64, float* f32, int* status, cudaStream_t s) {
     const size_t smem = skern::saddle_tiles_smem(h->dim, l.tl_max4, l.tl_np, l.tl_n);
-    const bool two = 2 * (smem + 2048) <= 227 * 1024;
-    auto kern = two ? skern::saddle_inverse_tiles_256 : skern::saddle_inverse_tiles_512;
+    const int nt = 2 * (smem + 2048) > 227 * 1024 ? 512 : 4 * (smem + 2048) > 227 * 1024 ? 256 : 128;
+    auto kern = nt == 512 ? skern::saddle_inverse_tiles_512 : nt == 256 ? skern::saddle_inverse_tiles_256 : skern::saddle_inverse_tiles_128;
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)skern::SADDLE_TILES_SMEM_MAX));
     double* scr = palloc<double>(h->device, l.tl_scratch, s);
     launch(h, PK_GJ, s, [&] {
-        kern<<<l.tl_count, two ? 256 : 512, smem, s>>>(h->dim, l.tl_list, l.poff, l.pnv, l.foff64, f64, l.foff32, f32,
+        kern<<<l.tl_count, nt, smem, s>>>(h->dim, l.tl_list, l.poff, l.pnv, l.foff64, f64, l.foff32, f32,
                                                        l.fac_packed ? 1 : 0, l.pdofs, l.K.rp, l.K.ci, l.K.v64, l.tl_max4,
                                                        l.tl_np, l.tl_soff, scr, status);
     });
@@ -1967,10 +1978,10 @@ void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status,
         const int d = h->dim;
         double* f64 = store ? l.fac64 : nullptr;
         float* f32 = store ? l.fac32 : nullptr;
-        if (l.saddle_smem > 0) {
+        if (l.saddle_smem > 0 && (!fused || l.sm_n > 0)) {
             const bool fac_only = !i64 && !i32 && !back;
             const long long sd_off = fac_only ? l.saddle_smem_fac : l.saddle_smem;
-            const size_t smem = (size_t)(sd_off + (fused ? (l.maxn + 1) / 2 : 0)) * sizeof(double);
+            const size_t smem = (size_t)(sd_off + (fused ? (l.sm_n + 1) / 2 : 0)) * sizeof(double);
             // one upper bound for every level (levels launch from one thread
             // onto different streams)
             CK(cudaFuncSetAttribute(skern::saddle_inverse_smem, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1978,11 +1989,11 @@ void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status,
             launch(h, PK_GJ, s, [&] {
                 skern::saddle_inverse_smem<<<l.npatch, 256, smem, s>>>(
                     l.npatch, d, l.poff, l.pnv, l.moff, fused ? nullptr : work, l.ioff64, i64, l.ioff32, i32, l.foff64, f64,
-                    l.foff32, f32, back, l.fac_packed ? 1 : 0, skern::SADDLE_SMEM_MAX_DOUBLES, l.pdofs, l.K.rp, l.K.ci,
-                    l.K.v64, (int)sd_off, status);
+                    l.foff32, f32, back, l.fac_packed ? 1 : 0, skern::SADDLE_SMEM_MAX_DOUBLES,
+                    fused ? l.tl_min : INT_MAX, l.pdofs, l.K.rp, l.K.ci, l.K.v64, (int)sd_off, status);
             });
         }
-        if (l.saddle_global > 0 && fused) {
+        if (l.tl_count > 0 && fused) {
             launch_tiles(h, l, f64, f32, status, s);
         } else if (l.saddle_global > 0) {
             // scratch of the patches too large for shared memory, from the
