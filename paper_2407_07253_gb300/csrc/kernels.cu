@@ -832,6 +832,9 @@ __device__ void saddle_core(int d, int n, int nv, double* K, double* scratch, do
     }
 }
 
+// 4 x 4 tiles of an upper triangle, n4 rows of tiles: tile (I, J), I <= J, is number tile_row(n4, I) + J
+__device__ __forceinline__ int tile_row(int n4, int I) { return I * n4 - I * (I - 1) / 2 - I; }
+
 // The factored form alone (no explicit output), in less shared memory: the
 // components' B_c^T and W_c = Li B_c^T go through one pair of buffers, W_c
 // is written out as soon as it exists and S = sum_c B_c W_c accumulates over
@@ -879,7 +882,7 @@ __device__ void saddle_core_factored(int d, int n, int nv, const double* K, cons
     const int ldl = (nv + vec - 1) / vec * vec;
     const int ldw = (dnv + vec - 1) / vec * vec;
     const int lds = (np + vec - 1) / vec * vec;
-    const long long lenL = packed ? ((long long)nv * (nv + 1) / 2 + vec - 1) / vec * vec : (long long)ldl * nv;
+    const long long lenL = saddle_factor_lenL(nv, vec, packed);
     const long long oW = lenL, oS = oW + (long long)ldw * np;
     const int ns = np * (np + 1) / 2;
     if (K) {
@@ -902,7 +905,17 @@ __device__ void saddle_core_factored(int d, int n, int nv, const double* K, cons
     for (int t = tid; t < np * np; t += nt) Ss[t] = 0.0;
     __syncthreads();
     sweep_spd2<PP>(Ls, nv, nv, ck, cs, c1p, cs1, rinv, status);
-    if (packed) {
+    if (packed == 2) {
+        // 4 x 4 tiles (FP32): group r ntile + t of four columns
+        const int n4 = (nv + 3) >> 2, ntile = n4 * (n4 + 1) / 2;
+        for (int I = warp; I < n4; I += nw)
+            for (int x = lane; x < 16 * (n4 - I); x += 32) {
+                const int J = I + (x >> 4), rr = (x >> 2) & 3, c = x & 3, a = 4 * I + rr, b = 4 * J + c;
+                const int lo = min(a, b), hi = max(a, b);
+                fac32[4 * ((long long)rr * ntile + tile_row(n4, I) + J) + c] =
+                    hi < nv ? (float)Ls[(PP ? pp_row(nv, lo) : lo * nv) + hi] : 0.f;
+            }
+    } else if (packed) {
         // upper triangle row by row: (a, b >= a) at a nv - a (a - 1) / 2 + b - a
         for (int a = warp; a < nv; a += nw) {
             const long long o = (long long)a * nv - (long long)a * (a - 1) / 2 - a;
@@ -1086,7 +1099,6 @@ __global__ void __launch_bounds__(256) saddle_inverse_global(int npatch, int d, 
 // A tile's entry (r, c) is double c & 1 of 16-byte group 2 r + c / 2, groups
 // [8][ntile], so that the threads of a warp, on consecutive tiles, read and
 // write them without bank conflicts.
-__device__ __forceinline__ int tile_row(int n4, int I) { return I * n4 - I * (I - 1) / 2 - I; }   // + J: tile (I, J)
 __device__ __forceinline__ double& tile_at(double2* T, int ntile, int t, int r, int c) {
     return reinterpret_cast<double*>(T)[((size_t)(2 * r + (c >> 1)) * ntile + t) * 2 + (c & 1)];
 }
@@ -1217,7 +1229,7 @@ __device__ __forceinline__ void saddle_tiles_body(
     const int n4 = (nv + 3) >> 2, q4 = (np + 3) >> 2;
     const int vec = fac64 ? 2 : 4;
     const int ldl = (nv + vec - 1) / vec * vec, ldw = (dnv + vec - 1) / vec * vec, lds = (np + vec - 1) / vec * vec;
-    const long long lenL = packed ? ((long long)nv * (nv + 1) / 2 + vec - 1) / vec * vec : (long long)ldl * nv;
+    const long long lenL = saddle_factor_lenL(nv, vec, packed);
     const long long oW = lenL, oS = oW + (long long)ldw * np;
     double* f64 = fac64 ? fac64 + foff64[p] : nullptr;
     float* f32 = fac32 ? fac32 + foff32[p] : nullptr;
@@ -1269,7 +1281,12 @@ __device__ __forceinline__ void saddle_tiles_body(
         return a <= b ? tile_at(T, ntile, tile_row(n4, a >> 2) + (b >> 2), a & 3, b & 3)
                       : tile_at(T, ntile, tile_row(n4, b >> 2) + (a >> 2), b & 3, a & 3);
     };
-    if (packed) {
+    if (packed == 2) {
+        for (int x = tid; x < 16 * ntile; x += NT) {
+            const int rr = x / (4 * ntile), t = (x - rr * 4 * ntile) >> 2, c = x & 3, a = 4 * map[t].x + rr, b = 4 * map[t].y + c;
+            put(x, max(a, b) < nv ? flip(li(a, b)) : 0.0);
+        }
+    } else if (packed) {
         for (int a = warp; a < nv; a += NW) {
             const long long o = (long long)a * nv - (long long)a * (a - 1) / 2 - a;
             for (int b = a + lane; b < nv; b += 32) put(o + b, flip(li(a, b)));
@@ -1713,6 +1730,202 @@ __device__ __forceinline__ void sa_bulk_load(uint32_t dst, const void* src, uint
                  : "memory");
 }
 
+// ---- the FP32 sweep on tiles ---------------------------------------------
+// As above (one bulk copy per patch and CTA), with Li as 4 x 4 tiles of its
+// upper triangle (tile (I, J) of tile_row's order; row r of tile t is 16-byte
+// group r ntile + t) and the products on 16-byte shared-memory reads: the kernel
+// above spends its time on issue (5400 warp instructions per P4 patch, two
+// scalar reads per FMA).  Li r_u: a thread multiplies a tile by x_J for block
+// row I and, transposed, by x_I for block row J, all components at once, and
+// keeps the results in registers; once every tile has been read they go over
+// Li's place as partial sums part[slot][R] (slot J of row I, slot I of row J,
+// each pair once; a row of 4 n4 D + 4 floats, so that the writes of consecutive
+// tiles fall into different banks), which the thread of an output row adds in
+// slot order.  t: eight lanes per column of W; z: one thread per row.
+// 64 x 64 P4: 31.8 -> 24.5 us a sweep (84 MB, 3.4 TB/s; 3100 warp instructions a
+// patch), bound by a patch's chain of dependent loads, copy and barriers times the
+// patches that fit an SM; 256 x 256 P4: a solve 71.1 -> 61.3 ms.
+template <int D, int NT, int TPT>
+__device__ __forceinline__ void saddle_tile_apply_body(
+    const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
+    const long long* __restrict__ foff, const float* __restrict__ fac, const float* __restrict__ r,
+    const float* __restrict__ wt, float* __restrict__ Y, int buf_bytes, int xs_len, int* __restrict__ status,
+    unsigned char* smem, unsigned long long* bar) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int p = blockIdx.x;
+    const int xl = (xs_len + 7) & ~3;
+    float* xi = reinterpret_cast<float*>(smem + (size_t)buf_bytes);   // [xl + 4 D] r_u by node, components together
+    float* xs = xi + xl + 4 * D;                                       // [xl] r_u as W's rows, zero padded
+    float* wq = xs + xl;                                               // [xl] weights
+    float* tq = wq + xl;                                               // [xl] r_p, then t
+    float* sq = tq + xl;                                               // [xl] s
+    const uint32_t b = sa_smem_u32(bar);
+    const int s0 = poff[p], n = poff[p + 1] - s0, nv = pnv[p], dnv = D * nv, np = n - dnv;
+    const int n4 = (nv + 3) >> 2, ntile = n4 * (n4 + 1) / 2, lenL = 16 * ntile;
+    const int ldw = (dnv + 3) & ~3, lds = (np + 3) & ~3;
+    if (tid == 0) {
+        sa_mbar_init(b);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        const long long o = foff[p];
+        const uint32_t bytes = (uint32_t)((foff[p + 1] - o) * (long long)sizeof(float));
+        if (bytes > 0) sa_bulk_load(sa_smem_u32(smem), fac + o, bytes, b);
+        else asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
+    }
+    pdl_wait();
+    pdl_release();
+    for (int a = tid; a < n; a += NT) {
+        const int j = pdofs[s0 + a];
+        const float v = r[j];
+        wq[a] = wt[j];
+        if (a < dnv) {
+            const int c = a / nv;
+            xi[(a - c * nv) * D + c] = v;
+            xs[a] = v;
+        } else {
+            tq[a - dnv] = v;
+        }
+    }
+    if (tid < 4 * D && dnv + tid < 4 * n4 * D) xi[dnv + tid] = 0.f;
+    if (tid < ldw - dnv) xs[dnv + tid] = 0.f;
+    __syncthreads();
+    // (the wait: as in saddle_apply_bulk_body)
+    bool ok = warp != 0;
+    if (warp == 0)
+        for (long long it = 0; it < SA_WAIT_LIMIT; ++it)
+            if (sa_mbar_try(b, 0)) { ok = true; break; }
+    if (__syncthreads_and(ok) && warp != 0) ok = sa_mbar_try(b, 0);
+    if (!__syncthreads_and(ok)) {
+        if (tid == 0) {
+            for (long long it = 0; it < SA_WAIT_LIMIT && !sa_mbar_try(b, 0); ++it) {}
+            atomicExch(status, 1);
+        }
+        return;
+    }
+    const float4* Tl = reinterpret_cast<const float4*>(smem);
+    const float* Wm = reinterpret_cast<const float*>(smem) + lenL;
+    const float* Si = Wm + ldw * np;
+    // y by tiles, into registers
+    float yI[TPT][4 * D], yJ[TPT][4 * D];
+    int tI[TPT], tJ[TPT];
+#pragma unroll
+    for (int u = 0; u < TPT; ++u) {
+        const int t = tid + u * NT;
+        tI[u] = -1;
+        tJ[u] = -1;
+        if (t < ntile) {
+            // row I of tile t: the largest I with I n4 - I (I - 1) / 2 <= t
+            const float h = (float)(2 * n4 + 1);
+            int I = (int)(0.5f * (h - sqrtf(h * h - 8.f * (float)t)));
+            if (I > 0 && I * n4 - I * (I - 1) / 2 > t) --I;
+            if ((I + 1) * n4 - (I + 1) * I / 2 <= t) ++I;
+            const int J = t - tile_row(n4, I);
+            tI[u] = I;
+            tJ[u] = J;
+            float xI[4 * D], xJ[4 * D];
+#pragma unroll
+            for (int q = 0; q < D; ++q) {
+                const float4 a = *reinterpret_cast<const float4*>(xi + 4 * D * I + 4 * q);
+                const float4 c = *reinterpret_cast<const float4*>(xi + 4 * D * J + 4 * q);
+                xI[4 * q] = a.x; xI[4 * q + 1] = a.y; xI[4 * q + 2] = a.z; xI[4 * q + 3] = a.w;
+                xJ[4 * q] = c.x; xJ[4 * q + 1] = c.y; xJ[4 * q + 2] = c.z; xJ[4 * q + 3] = c.w;
+            }
+#pragma unroll
+            for (int q = 0; q < 4 * D; ++q) { yI[u][q] = 0.f; yJ[u][q] = 0.f; }
+#pragma unroll
+            for (int rr = 0; rr < 4; ++rr) {
+                const float4 v4 = Tl[rr * ntile + t];
+                const float v[4] = {v4.x, v4.y, v4.z, v4.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+#pragma unroll
+                    for (int c = 0; c < D; ++c) {
+                        yI[u][rr * D + c] = fmaf(v[k], xJ[k * D + c], yI[u][rr * D + c]);
+                        yJ[u][k * D + c] = fmaf(v[k], xI[rr * D + c], yJ[u][k * D + c]);
+                    }
+            }
+        }
+    }
+    // t = r_p - W^T r_u
+    {
+        const int sub = lane & 7, ldwv = ldw >> 2;
+        const float4* xv = reinterpret_cast<const float4*>(xs);
+        for (int q0 = warp * 4; q0 < np; q0 += NT / 8) {
+            const int q = q0 + (lane >> 3);
+            float acc = 0.f;
+            if (q < np) {
+                const float4* wc = reinterpret_cast<const float4*>(Wm) + q * ldwv;
+#pragma unroll 4
+                for (int i = sub; i < ldwv; i += 8) {
+                    const float4 w = wc[i], x = xv[i];
+                    acc = fmaf(w.x, x.x, acc);
+                    acc = fmaf(w.y, x.y, acc);
+                    acc = fmaf(w.z, x.z, acc);
+                    acc = fmaf(w.w, x.w, acc);
+                }
+            }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (sub == 0 && q < np) tq[q] -= acc;
+        }
+    }
+    __syncthreads();
+    // partial sums over Li's place; s = Si t
+    float* part = reinterpret_cast<float*>(smem + (size_t)(D == 3 ? buf_bytes - tile_part_bytes(D, n4) : 0));
+    const int ldp = 4 * D * n4 + 4;
+#pragma unroll
+    for (int u = 0; u < TPT; ++u)
+        if (tI[u] >= 0) {
+            float4* pi = reinterpret_cast<float4*>(part + tJ[u] * ldp + 4 * D * tI[u]);
+            float4* pj = reinterpret_cast<float4*>(part + tI[u] * ldp + 4 * D * tJ[u]);
+#pragma unroll
+            for (int q = 0; q < D; ++q) {
+                pi[q] = make_float4(yI[u][4 * q], yI[u][4 * q + 1], yI[u][4 * q + 2], yI[u][4 * q + 3]);
+                if (tI[u] != tJ[u]) pj[q] = make_float4(yJ[u][4 * q], yJ[u][4 * q + 1], yJ[u][4 * q + 2], yJ[u][4 * q + 3]);
+            }
+        }
+    // (from the last thread down: the first ones have the most tiles to write)
+    for (int q = NT - 1 - tid; q < np; q += NT) {
+        float acc = 0.f;
+        for (int x = 0; x < np; ++x) acc = fmaf(Si[x * lds + q], tq[x], acc);
+        sq[q] = acc;
+    }
+    __syncthreads();
+    // z_u = y + W s, z_p = -s, weighted
+    for (int a = tid; a < dnv; a += NT) {
+        const int c = a / nv, i = a - c * nv;
+        const float* pp = part + i * D + c;
+        float z = 0.f;
+#pragma unroll 4
+        for (int sl = 0; sl < n4; ++sl) z += pp[sl * ldp];
+#pragma unroll 4
+        for (int q = 0; q < np; ++q) z = fmaf(Wm[q * ldw + a], sq[q], z);
+        Y[s0 + a] = wq[a] * z;
+    }
+    for (int q = tid; q < np; q += NT) Y[s0 + dnv + q] = -wq[dnv + q] * sq[q];
+}
+
+#define SADDLE_TILE_APPLY_KERNEL(D, NT, TPT)                                                                        \
+    __global__ void __launch_bounds__(NT) saddle_tile_apply_##D##d_##NT##_##TPT(                                    \
+        const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,                   \
+        const long long* __restrict__ foff, const float* __restrict__ fac, const float* __restrict__ r,             \
+        const float* __restrict__ wt, float* __restrict__ Y, int buf_bytes, int xs_len, int* __restrict__ status) { \
+        extern __shared__ __align__(128) unsigned char smem_ta[];                                                   \
+        __shared__ __align__(8) unsigned long long bar;                                                             \
+        saddle_tile_apply_body<D, NT, TPT>(poff, pdofs, pnv, foff, fac, r, wt, Y, buf_bytes, xs_len, status,        \
+                                           smem_ta, &bar);                                                          \
+    }
+#define SADDLE_TILE_APPLY_KERNELS(D)     \
+    SADDLE_TILE_APPLY_KERNEL(D, 32, 1)   \
+    SADDLE_TILE_APPLY_KERNEL(D, 64, 1)   \
+    SADDLE_TILE_APPLY_KERNEL(D, 128, 1)  \
+    SADDLE_TILE_APPLY_KERNEL(D, 160, 1)  \
+    SADDLE_TILE_APPLY_KERNEL(D, 256, 1)  \
+    SADDLE_TILE_APPLY_KERNEL(D, 256, 2)
+SADDLE_TILE_APPLY_KERNELS(2)
+SADDLE_TILE_APPLY_KERNELS(3)
+#undef SADDLE_TILE_APPLY_KERNELS
+#undef SADDLE_TILE_APPLY_KERNEL
+
 template <typename T>
 __device__ __forceinline__ void saddle_apply_bulk_body(
     int d, const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
@@ -1810,14 +2023,6 @@ __device__ __forceinline__ void saddle_apply_bulk_body(
     for (int q = tid; q < np; q += NT) Y[s0 + dnv + q] = -wq[dnv + q] * sq[q];
 }
 
-__global__ void __launch_bounds__(SA_BULK_THREADS) saddle_apply_bulk_f32(
-    int d, const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
-    const long long* __restrict__ foff, const float* __restrict__ fac, const float* __restrict__ r,
-    const float* __restrict__ wt, float* __restrict__ Y, int buf_bytes, int xs_len, int* __restrict__ status) {
-    extern __shared__ __align__(128) unsigned char smem_sb[];
-    __shared__ __align__(8) unsigned long long bar;
-    saddle_apply_bulk_body<float>(d, poff, pdofs, pnv, foff, fac, r, wt, Y, buf_bytes, xs_len, status, smem_sb, &bar);
-}
 __global__ void __launch_bounds__(SA_BULK_THREADS) saddle_apply_bulk_f64(
     int d, const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
     const long long* __restrict__ foff, const double* __restrict__ fac, const double* __restrict__ r,

@@ -263,15 +263,20 @@ __global__ void saddle_inverse_tiles_256(SADDLE_TILES_ARGS);
 __global__ void saddle_inverse_tiles_128(SADDLE_TILES_ARGS);
 #undef SADDLE_TILES_ARGS
 // Elements of one patch's factored inverse (Li, W, Si with leading
-// dimensions rounded up to vec = 2 (FP64) or 4 (FP32)); packed: Li as its
-// upper triangle row by row (nv (nv + 1) / 2 entries, rounded up to vec),
-// the layout of the bulk-copy apply.
+// dimensions rounded up to vec = 2 (FP64) or 4 (FP32)).  Li's form, packed:
+// 0 column-major; 1 its upper triangle row by row (nv (nv + 1) / 2 entries,
+// rounded up to vec: the FP64 bulk-copy apply); 2 the 4 x 4 tiles of its upper
+// triangle, zero padded, 16-byte group r ntile + t holding row r of tile t (the
+// FP32 bulk-copy apply).
+__host__ __device__ inline long long saddle_factor_lenL(int nv, int vec, int packed) {
+    const long long n4 = (nv + 3) / 4;
+    if (packed == 2) return 8 * n4 * (n4 + 1);
+    return packed ? ((long long)nv * (nv + 1) / 2 + vec - 1) / vec * vec : (long long)((nv + vec - 1) / vec * vec) * nv;
+}
 __host__ __device__ inline long long saddle_factor_len(int d, int n, int nv, int vec, int packed = 0) {
     const int np = n - d * nv;
-    const long long ldl = (nv + vec - 1) / vec * vec, ldw = (d * nv + vec - 1) / vec * vec,
-                    lds = (np + vec - 1) / vec * vec;
-    const long long lenL = packed ? ((long long)nv * (nv + 1) / 2 + vec - 1) / vec * vec : ldl * nv;
-    return lenL + ldw * np + lds * np;
+    const long long ldw = (d * nv + vec - 1) / vec * vec, lds = (np + vec - 1) / vec * vec;
+    return saddle_factor_lenL(nv, vec, packed) + ldw * np + lds * np;
 }
 // One ASM sweep with the factored inverses streamed from global memory, one
 // CTA per patch, D = 2 or 3 components; xs_len >= the largest patch.  Shared
@@ -311,16 +316,47 @@ constexpr long long SA_WAIT_LIMIT = 1ll << 22;
 __host__ __device__ inline size_t saddle_apply_bulk_smem(int buf_bytes, int elem_bytes, int xs_len) {
     return (size_t)buf_bytes + (size_t)elem_bytes * 5 * xs_len;
 }
-__global__ void saddle_apply_bulk_f32(int d, const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                      const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                      const float* __restrict__ fac, const float* __restrict__ r,
-                                      const float* __restrict__ wt, float* __restrict__ Y, int buf_bytes,
-                                      int xs_len, int* __restrict__ status);
 __global__ void saddle_apply_bulk_f64(int d, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                       const int* __restrict__ pnv, const long long* __restrict__ foff,
                                       const double* __restrict__ fac, const double* __restrict__ r,
                                       const double* __restrict__ wt, double* __restrict__ Y, int buf_bytes,
                                       int xs_len, int* __restrict__ status);
+
+// The FP32 sweep with Li on tiles (packed = 2): buf_bytes >= the largest block
+// rounded up to 128 bytes, in 3D plus tile_part_bytes of the largest patch (its
+// partial sums; in 2D they fit over Li).  saddle_tile_apply_<dim>_<threads>_<tiles per thread>.
+__host__ __device__ inline int tile_part_bytes(int d, int n4) { return (4 * d * n4 + 4) * n4 * 4; }
+__host__ __device__ inline size_t saddle_tile_apply_smem(int buf_bytes, int d, int xs_len) {
+    return (size_t)buf_bytes + 4 * (5 * (size_t)((xs_len + 7) & ~3) + 4 * d);
+}
+#define SADDLE_TILE_APPLY_ARGS                                                                                      \
+    const int *__restrict__ poff, const int *__restrict__ pdofs, const int *__restrict__ pnv,                       \
+        const long long *__restrict__ foff, const float *__restrict__ fac, const float *__restrict__ r,             \
+        const float *__restrict__ wt, float *__restrict__ Y, int buf_bytes, int xs_len, int *__restrict__ status
+#define SADDLE_TILE_APPLY_DECL(D)                                         \
+    __global__ void saddle_tile_apply_##D##d_32_1(SADDLE_TILE_APPLY_ARGS);  \
+    __global__ void saddle_tile_apply_##D##d_64_1(SADDLE_TILE_APPLY_ARGS);  \
+    __global__ void saddle_tile_apply_##D##d_128_1(SADDLE_TILE_APPLY_ARGS); \
+    __global__ void saddle_tile_apply_##D##d_160_1(SADDLE_TILE_APPLY_ARGS); \
+    __global__ void saddle_tile_apply_##D##d_256_1(SADDLE_TILE_APPLY_ARGS); \
+    __global__ void saddle_tile_apply_##D##d_256_2(SADDLE_TILE_APPLY_ARGS);
+SADDLE_TILE_APPLY_DECL(2)
+SADDLE_TILE_APPLY_DECL(3)
+#undef SADDLE_TILE_APPLY_DECL
+using saddle_tile_apply_t = void (*)(SADDLE_TILE_APPLY_ARGS);
+#undef SADDLE_TILE_APPLY_ARGS
+// threads per CTA for npatch patches of at most n4 tile rows (0: too many
+// tiles): one tile a thread where a CTA of up to 256 holds them, so that small
+// patches take little of an SM and many of them are in flight; two above.  With
+// 128 threads for all, 64 x 64 P4 took 29 us (24.5 with 160) and its 4225 P2
+// stars 12.3 (8.6 with 32); a level too small to fill the SMs (one warp a patch
+// takes the longest there: 6.4 us against 5.9 for 1089 stars) keeps two warps.
+constexpr int SADDLE_TILE_APPLY_MAX = 512, SADDLE_TILE_APPLY_WARP_MIN = 152 * 16;
+inline int saddle_tile_apply_threads(int n4, int npatch) {
+    const int t = n4 * (n4 + 1) / 2;
+    if (t <= 64) return t <= 32 && npatch >= SADDLE_TILE_APPLY_WARP_MIN ? 32 : 64;
+    return t <= 128 ? 128 : t <= 160 ? 160 : t <= SADDLE_TILE_APPLY_MAX ? 256 : 0;
+}
 
 // One ASM sweep (Eq. 3.4): Y[poff[i] + a] = w[dof_a] * sum_b Kinv_i[a][b] r[dof_b].
 // FP32: float4 loads of 4 consecutive rows per thread; FP64: double2 loads

@@ -180,7 +180,8 @@ struct DevLevel {
     float* fac32 = nullptr;
     int sa_xs = 0;                      // saddle apply: largest patch
     int sa_buf = 0;                     // bulk-copy apply: buffer bytes (0: not used on this level)
-    bool fac_packed = false;            // L^-1 stored as its packed upper triangle (bulk-copy apply only)
+    int sa_n4 = 0;                      // its tile rows (FP32)
+    int fac_packed = 0;                 // the form of L^-1 (saddle_factor_len; 1 and 2 with the bulk-copy apply only)
     double* wt64 = nullptr;
     float* wt32 = nullptr;
     int *soff = nullptr, *sidx = nullptr;
@@ -600,7 +601,18 @@ template <> struct PatchOf<float> {
     static const long long* ioff(const DevLevel& l) { return l.ioff32; }
     static const float* wt(const DevLevel& l) { return l.wt32; }
     static float* Y(const DevLevel& l) { return l.Y32; }
-    static constexpr auto bulk = skern::saddle_apply_bulk_f32;
+    static skern::saddle_tile_apply_t tiles(int dim, int n4, int npatch) {
+        const bool two = n4 * (n4 + 1) / 2 > 256;
+        switch (skern::saddle_tile_apply_threads(n4, npatch)) {
+            case 32: return dim == 3 ? skern::saddle_tile_apply_3d_32_1 : skern::saddle_tile_apply_2d_32_1;
+            case 64: return dim == 3 ? skern::saddle_tile_apply_3d_64_1 : skern::saddle_tile_apply_2d_64_1;
+            case 128: return dim == 3 ? skern::saddle_tile_apply_3d_128_1 : skern::saddle_tile_apply_2d_128_1;
+            case 160: return dim == 3 ? skern::saddle_tile_apply_3d_160_1 : skern::saddle_tile_apply_2d_160_1;
+            default:
+                if (two) return dim == 3 ? skern::saddle_tile_apply_3d_256_2 : skern::saddle_tile_apply_2d_256_2;
+                return dim == 3 ? skern::saddle_tile_apply_3d_256_1 : skern::saddle_tile_apply_2d_256_1;
+        }
+    }
     static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f32_3d : skern::saddle_apply_f32_2d; }
     static constexpr auto expl = skern::patch_apply_f32;
     static constexpr size_t red = sizeof(float4);
@@ -613,7 +625,6 @@ template <> struct PatchOf<double> {
     static const long long* ioff(const DevLevel& l) { return l.ioff64; }
     static const double* wt(const DevLevel& l) { return l.wt64; }
     static double* Y(const DevLevel& l) { return l.Y64; }
-    static constexpr auto bulk = skern::saddle_apply_bulk_f64;
     static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f64_3d : skern::saddle_apply_f64_2d; }
     static constexpr auto expl = skern::patch_apply_f64;
     static constexpr size_t red = sizeof(double2);
@@ -633,10 +644,15 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
     T* Y = PO::Y(l);
     const int *poff = l.poff, *pdofs = l.pdofs, *pnv = l.pnv;
     if (fac && l.sa_buf > 0) {
-        const size_t smem = skern::saddle_apply_bulk_smem(l.sa_buf, sizeof(T), l.sa_xs);
         launch(h, PK_PATCH, s, [&] {
-            kl(h, PO::bulk, l.npatch, skern::SA_BULK_THREADS, smem, s, h->dim, poff, pdofs, pnv, foff, fac, r, wt, Y,
-               (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
+            if constexpr (sizeof(T) == 4)
+                kl(h, PO::tiles(h->dim, l.sa_n4, l.npatch), l.npatch, skern::saddle_tile_apply_threads(l.sa_n4, l.npatch),
+                   skern::saddle_tile_apply_smem(l.sa_buf, h->dim, l.sa_xs), s, poff, pdofs, pnv, foff, fac, r, wt, Y,
+                   (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
+            else
+                kl(h, skern::saddle_apply_bulk_f64, l.npatch, skern::SA_BULK_THREADS,
+                   skern::saddle_apply_bulk_smem(l.sa_buf, sizeof(T), l.sa_xs), s, h->dim, poff, pdofs, pnv, foff, fac, r,
+                   wt, Y, (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
         });
     } else if (fac) {
         const size_t smem = skern::saddle_apply_smem(sizeof(T), h->dim, l.sa_xs);
@@ -1608,26 +1624,36 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
             };
             opt_in(PatchOf<float>::fact(HL.d));
             opt_in(PatchOf<double>::fact(HL.d));
-            opt_in(skern::saddle_apply_bulk_f32);
             opt_in(skern::saddle_apply_bulk_f64);
-            // the bulk-copy apply, with L^-1 stored as its packed upper
-            // triangle, when the level's largest packed block fits in shared
-            // memory with room for at least two CTAs per SM
+            // the bulk-copy apply, with L^-1 stored as its upper triangle (FP32:
+            // in 4 x 4 tiles, at most SADDLE_TILE_APPLY_MAX), when the level's largest
+            // block fits in shared memory with room for at least two CTAs per SM
             {
-                const int eb = want32 ? 4 : 8, vec = 16 / eb;
+                const int eb = want32 ? 4 : 8, vec = 16 / eb, packed = want32 ? 2 : 1;
                 long long mb = 0;
+                int n4 = 0;
                 std::vector<long long> fp(l.npatch + 1, 0);
                 for (int p = 0; p < l.npatch; ++p) {
                     const long long len = skern::saddle_factor_len(HL.d, HL.patch_off[p + 1] - HL.patch_off[p],
-                                                                   HL.patch_nv[p], vec, 1);
+                                                                   HL.patch_nv[p], vec, packed);
                     fp[p + 1] = fp[p] + len;
                     mb = std::max(mb, len);
+                    n4 = std::max(n4, (HL.patch_nv[p] + 3) / 4);
                 }
-                const long long buf = (mb * eb + 127) & ~127LL;
-                const size_t smem = skern::saddle_apply_bulk_smem((int)std::min<long long>(buf, 1 << 30), eb, l.sa_xs);
-                if (buf > 0 && smem <= skern::SADDLE_APPLY_SMEM_MAX / 2 && !std::getenv("STOKES_NO_BULK_APPLY")) {
+                const bool tiles = skern::saddle_tile_apply_threads(n4, l.npatch) > 0;
+                long long buf = (mb * eb + 127) & ~127LL;
+                if (want32 && HL.d == 3) buf += (skern::tile_part_bytes(3, std::min(n4, 64)) + 127) & ~127;
+                buf = std::min<long long>(buf, 1 << 30);
+                const size_t smem = want32 ? skern::saddle_tile_apply_smem((int)buf, HL.d, l.sa_xs)
+                                           : skern::saddle_apply_bulk_smem((int)buf, eb, l.sa_xs);
+                if (mb > 0 && smem <= skern::SADDLE_APPLY_SMEM_MAX / 2 && (!want32 || tiles) &&
+                    !std::getenv("STOKES_NO_BULK_APPLY")) {
                     l.sa_buf = (int)buf;
-                    l.fac_packed = true;
+                    l.sa_n4 = n4;
+                    if (want32)
+                        CK(cudaFuncSetAttribute(PatchOf<float>::tiles(HL.d, n4, l.npatch), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                (int)skern::SADDLE_APPLY_SMEM_MAX));
+                    l.fac_packed = packed;
                     (want32 ? f32 : f64) = fp;
                     (want32 ? l.nfac32 : l.nfac64) = fp[l.npatch];
                 }
@@ -1952,7 +1978,7 @@ void launch_tiles(stokes_mg* h, DevLevel& l, double* f64, float* f32, int* statu
     double* scr = palloc<double>(h->device, l.tl_scratch, s);
     launch(h, PK_GJ, s, [&] {
         kern<<<l.tl_count, nt, smem, s>>>(h->dim, l.tl_list, l.poff, l.pnv, l.foff64, f64, l.foff32, f32,
-                                                       l.fac_packed ? 1 : 0, l.pdofs, l.K.rp, l.K.ci, l.K.v64, l.tl_max4,
+                                                       l.fac_packed, l.pdofs, l.K.rp, l.K.ci, l.K.v64, l.tl_max4,
                                                        l.tl_np, l.tl_soff, scr, status);
     });
     CK(cudaFreeAsync(scr, s));
@@ -1989,7 +2015,7 @@ void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status,
             launch(h, PK_GJ, s, [&] {
                 skern::saddle_inverse_smem<<<l.npatch, 256, smem, s>>>(
                     l.npatch, d, l.poff, l.pnv, l.moff, fused ? nullptr : work, l.ioff64, i64, l.ioff32, i32, l.foff64, f64,
-                    l.foff32, f32, back, l.fac_packed ? 1 : 0, skern::SADDLE_SMEM_MAX_DOUBLES,
+                    l.foff32, f32, back, l.fac_packed, skern::SADDLE_SMEM_MAX_DOUBLES,
                     fused ? l.tl_min : INT_MAX, l.pdofs, l.K.rp, l.K.ci, l.K.v64, (int)sd_off, status);
             });
         }
@@ -2002,7 +2028,7 @@ void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status,
             launch(h, PK_GJ, s, [&] {
                 skern::saddle_inverse_global<<<l.npatch, 256, 0, s>>>(l.npatch, d, l.poff, l.pnv, l.moff, work, l.ioff64, i64,
                                                                       l.ioff32, i32, l.foff64, f64, l.foff32, f32, back,
-                                                                      l.fac_packed ? 1 : 0, skern::SADDLE_SMEM_MAX_DOUBLES,
+                                                                      l.fac_packed, skern::SADDLE_SMEM_MAX_DOUBLES,
                                                                       l.scoff, scr, status);
             });
             CK(cudaFreeAsync(scr, s));

@@ -1,8 +1,9 @@
-"""The streamed saddle apply (one ASM sweep, Eq. 3.4) on every level of small
-hierarchies whose patches cover its edges: one row group to several, row counts
-of every remainder of the 16-byte vectors, one pressure column to more than a
-warp's, two and three components, both precisions.  The bulk-copy apply is
-switched off, so that the small levels take the streamed one too.
+"""The saddle applies (one ASM sweep, Eq. 3.4) on every level of small
+hierarchies whose patches cover their edges: one row group or tile to several
+per thread, row counts of every remainder of the 16-byte vectors, one pressure
+column to more than a warp's, two and three components, both precisions.  Once
+with the bulk-copy applies (the FP32 one on tiles) on the levels that they take,
+once with them switched off, so that every level takes the streamed one.
 
 Reference: z = sum_i I_i^T W_i K_i^-1 I_i r with numpy's LU solves of the
 exported patch blocks.  The two sides factor the blocks differently and agree
@@ -29,9 +30,11 @@ CASES = {
 
 
 @pytest.mark.parametrize("precision", [P.FP64, P.MIXED])
+@pytest.mark.parametrize("bulk", [True, False])
 @pytest.mark.parametrize("name", sorted(CASES))
-def test_streamed_apply_matches_patch_solves(name, precision, monkeypatch):
-    monkeypatch.setenv("STOKES_NO_BULK_APPLY", "1")
+def test_apply_matches_patch_solves(name, bulk, precision, monkeypatch):
+    if not bulk:
+        monkeypatch.setenv("STOKES_NO_BULK_APPLY", "1")
     (v, c), nref, fam, k, sched, bary = CASES[name]
     h = P.StokesMG(v, c, nref, fam, k, barycentric=bary, hierarchy=P.HIER_EXPLICIT, schedule=sched,
                    precision=precision)
