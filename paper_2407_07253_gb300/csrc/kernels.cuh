@@ -100,6 +100,96 @@ __global__ void __launch_bounds__(256) spmv_csr(int nrows, int ncols, const int*
     }
 }
 
+// y = A x (SET) or y = b - A x (RESID) in FP32 for a Stokes operator as the device
+// assembly writes it: the rows of a velocity node's D components have their
+// entries in the same places (the velocity block, with the same values and the
+// columns of the component, then the pressures, with the same columns), and a
+// pressure row holds the components' blocks one after another, node by node
+// alike.  A group of LANES threads takes a node's D rows, or a pressure row, so
+// that one column index serves D entries, a velocity value D rows and a gathered
+// pressure D rows: 4 instead of 6 (2D) or 5 instead of 9 (3D) loads for D
+// entries, and D times as many gathers in flight per thread.  The gathers' latency
+// bounds it (cold caches, against spmv_csr): 64 x 64 P4 26.2 -> 23.6 us, 3D P3
+// 16^3 70 -> 56, 256 x 256 P4 231 -> 199 us (0.7 GB less the shared entries).  In FP64,
+// bound by the FP64 pipe, it measured no faster and is not used.
+template <int LANES, int MODE, int D>
+__global__ void __launch_bounds__(256) spmv_stokes(int nvf, int nq, const int* __restrict__ rp,
+                                                   const int* __restrict__ ci, const float* __restrict__ av,
+                                                   const float* __restrict__ x, float* __restrict__ y, const float* __restrict__ b) {
+    constexpr int U = 4;
+    const int g = (blockIdx.x * blockDim.x + threadIdx.x) / LANES;
+    const int lane = threadIdx.x % LANES;
+    const bool live = g < nvf + nq, vel = g < nvf;
+    const int row = vel ? g : g - nvf + D * nvf;
+    int s[D];
+    s[0] = live ? __ldg(rp + row) : 0;
+    int len = live ? __ldg(rp + row + 1) - s[0] : 0;
+#pragma unroll
+    for (int c = 1; c < D; ++c) s[c] = live && vel ? __ldg(rp + row + c * nvf) : 0;
+    if (!vel) {
+        len /= D;
+#pragma unroll
+        for (int c = 1; c < D; ++c) s[c] = s[0] + c * len;
+    }
+    int col[U];
+    float a[D][U];
+    auto load = [&](int p0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = p0 + u * LANES;
+            const bool ok = p < len;
+            col[u] = ok ? __ldg(ci + s[0] + p) : 0;
+            a[0][u] = ok ? __ldg(av + s[0] + p) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int p = p0 + u * LANES;
+            const bool own = p < len && !(vel && col[u] < nvf);      // B's entries; the velocity block's are shared
+#pragma unroll
+            for (int c = 1; c < D; ++c) a[c][u] = own ? __ldg(av + s[c] + p) : a[0][u];
+        }
+    };
+    int p = lane;
+    load(p);
+    pdl_wait();
+    pdl_release();
+    if (!live) return;   // whole LANES-group exits together (LANES divides 32)
+    float acc[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) acc[c] = 0;
+    for (;;) {
+        float xv[D][U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const bool one = vel && col[u] >= nvf;                   // a pressure: the same for every component
+            xv[0][u] = x[col[u]];
+#pragma unroll
+            for (int c = 1; c < D; ++c) xv[c][u] = one ? xv[0][u] : x[col[u] + c * nvf];
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int c = 0; c < D; ++c) acc[c] += a[c][u] * xv[c][u];
+        p += U * LANES;
+        if (p >= len) break;
+        load(p);
+    }
+    if (!vel) {
+#pragma unroll
+        for (int c = 1; c < D; ++c) acc[0] += acc[c];
+    }
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+        if (c > 0 && !vel) break;
+#pragma unroll
+        for (int o = LANES / 2; o > 0; o >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o, LANES);
+        if (lane == 0) {
+            const int i = row + c * nvf;
+            y[i] = MODE == SPMV_SET ? acc[c] : b[i] - acc[c];
+        }
+    }
+}
+
 // ------------------------------------------------------- vector kernels ---
 template <typename TO, typename TI>
 __global__ void convert_vec(int n, const TI* __restrict__ x, TO* __restrict__ y) {

@@ -141,6 +141,7 @@ inline int grid_for(long long n, int block = 256) {
 
 struct DevCSR {
     int nr = 0, nc = 0;
+    int dim = 0, nvf = 0;      // a Stokes operator in the device assembly's order (spmv_stokes): velocity nodes per component
     long long nnz = 0;
     int lanes = 16;
     int *rp = nullptr, *ci = nullptr;
@@ -550,8 +551,37 @@ void spmv_lanes(stokes_mg* h, const DevCSR& A, const T* x, T* y, const T* b, cud
     }
 }
 
+// Lanes per node of spmv_stokes: 8, which a small level's latency and long rows
+// want (64 x 64 P4 23.6 us against 25.5 with 4 and 30.8 with 2; 3D P3 16^3, 77
+// entries a row, 56 against 62), 4 where rows of up to 64 entries make so many
+// groups that issue counts (256 x 256 P4, 1.7 M groups: 199 us against 219).
+constexpr int kStokesFewLanesFrom = 1 << 20;
+
+template <int MODE, int D>
+void spmv_stokes_lanes(stokes_mg* h, const DevCSR& A, const float* x, float* y, const float* b, cudaStream_t s) {
+    const int nq = A.nr - D * A.nvf;
+    const bool few = A.nvf + nq >= kStokesFewLanesFrom && A.nnz <= 64LL * A.nr;
+    const int lanes = few ? 4 : 8, grid = (int)(((long long)(A.nvf + nq) * lanes + 255) / 256);
+    if (A.nr == 0) return;
+    if (few) kl(h, skern::spmv_stokes<4, MODE, D>, grid, 256, 0, s, A.nvf, nq, A.rp, A.ci, A.v32, x, y, b);
+    else kl(h, skern::spmv_stokes<8, MODE, D>, grid, 256, 0, s, A.nvf, nq, A.rp, A.ci, A.v32, x, y, b);
+}
+
 template <typename T>
 void spmv(stokes_mg* h, int kind, const DevCSR& A, int mode, const T* x, T* y, const T* b, cudaStream_t s) {
+    if constexpr (sizeof(T) == 4) {
+        if (A.nvf > 0 && mode != skern::SPMV_ADD && h->nvec == 1) {
+            launch(h, kind, s, [&] {
+                if (mode == skern::SPMV_SET)
+                    A.dim == 3 ? spmv_stokes_lanes<skern::SPMV_SET, 3>(h, A, x, y, b, s)
+                               : spmv_stokes_lanes<skern::SPMV_SET, 2>(h, A, x, y, b, s);
+                else
+                    A.dim == 3 ? spmv_stokes_lanes<skern::SPMV_RESID, 3>(h, A, x, y, b, s)
+                               : spmv_stokes_lanes<skern::SPMV_RESID, 2>(h, A, x, y, b, s);
+            });
+            return;
+        }
+    }
     launch(h, kind, s, [&] {
         if (mode == skern::SPMV_SET) h->nvec > 1 ? spmv_lanes<T, skern::SPMV_SET, true>(h, A, x, y, b, s)
                              : spmv_lanes<T, skern::SPMV_SET, false>(h, A, x, y, b, s);
@@ -1745,6 +1775,8 @@ void upload_assembly_inputs_lv(stokes_mg* h, const sfem::Level& HL, DevLevel& l,
     const int n = HL.n_free;
     DevCSR& K = l.K;
     K.nr = K.nc = n;
+    K.dim = a.d;
+    K.nvf = a.nVf;
     K.nnz = bound;                       // exact count read back once setup has synchronised
     K.rp = halloc<int>(h, n + 1);
     K.ci = halloc<int>(h, bound);
