@@ -1384,7 +1384,17 @@ __device__ __forceinline__ void patch_apply_body(int p, const int* __restrict__ 
                                                  T* xs, V* red) {
     const int s = poff[p], n = poff[p + 1] - s;
     const int ldv = (n + VEC - 1) / VEC;
-    for (int a = threadIdx.x; a < n; a += blockDim.x) xs[a] = r[pdofs[s + a]];
+    // the map is constant: fetched before the wait for the kernel that wrote r
+    constexpr int PRE = 2;
+    int jd[PRE];
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) jd[u] = (int)threadIdx.x + u * 128 < n ? __ldg(pdofs + s + threadIdx.x + u * 128) : -1;
+    pdl_wait();
+    pdl_release();
+#pragma unroll
+    for (int u = 0; u < PRE; ++u)
+        if (jd[u] >= 0) xs[threadIdx.x + u * 128] = r[jd[u]];
+    for (int a = threadIdx.x + PRE * 128; a < n; a += 128) xs[a] = r[pdofs[s + a]];
     __syncthreads();
     const int G = ldv >= (int)blockDim.x ? 1 : (int)blockDim.x / ldv;
     const V* base = reinterpret_cast<const V*>(inv + ioff[p]);
@@ -1450,8 +1460,6 @@ __global__ void __launch_bounds__(128) patch_apply_f32(int npatch, const int* __
     extern __shared__ __align__(16) unsigned char smem_pa[];
     float4* red = reinterpret_cast<float4*>(smem_pa);
     float* xs = reinterpret_cast<float*>(smem_pa + sizeof(float4) * (blockDim.x + 4));
-    pdl_wait();
-    pdl_release();
     patch_apply_body<float, float4, 4>(blockIdx.x, poff, pdofs, ioff, inv, r + (long long)blockIdx.y * n, wt,
                                             Y + blockIdx.y * nslot, xs, red);
 }
@@ -1463,8 +1471,6 @@ __global__ void __launch_bounds__(128) patch_apply_f64(int npatch, const int* __
     extern __shared__ __align__(16) unsigned char smem_pa[];
     double2* red = reinterpret_cast<double2*>(smem_pa);
     double* xs = reinterpret_cast<double*>(smem_pa + sizeof(double2) * (blockDim.x + 4));
-    pdl_wait();
-    pdl_release();
     patch_apply_body<double, double2, 2>(blockIdx.x, poff, pdofs, ioff, inv, r + (long long)blockIdx.y * n, wt,
                                             Y + blockIdx.y * nslot, xs, red);
 }
@@ -1601,10 +1607,14 @@ __device__ __forceinline__ void saddle_apply_body(int p, const int* __restrict__
     T* ys = xs;                                                             // then blockdiag(Li) r_u
     T* tq = xs + xl + 4;                                                    // [xl] r_p, then t
     T* sq = tq + xl;                                                        // [xl] s
+    // the map is constant: fetched before the wait
+    constexpr int PRE = 4;
+    int jd[PRE];
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) jd[u] = tid + u * NT < n ? __ldg(pdofs + s0 + tid + u * NT) : -1;
     pdl_wait();
     pdl_release();
-    for (int a = tid; a < n; a += NT) {
-        const T v = r[pdofs[s0 + a]];
+    auto place = [&](int a, T v) {
         if (a < dnv) {
             const int c = a / nv;
             xi[a - c * nv].v[c] = v;
@@ -1612,7 +1622,11 @@ __device__ __forceinline__ void saddle_apply_body(int p, const int* __restrict__
         } else {
             tq[a - dnv] = v;
         }
-    }
+    };
+#pragma unroll
+    for (int u = 0; u < PRE; ++u)
+        if (jd[u] >= 0) place(tid + u * NT, r[jd[u]]);
+    for (int a = tid + PRE * NT; a < n; a += NT) place(a, r[pdofs[s0 + a]]);
     for (int a = dnv + tid; a < ldw; a += NT) xs[a] = 0;
     __syncthreads();
     // t = r_p - W^T r_u: eight lanes per column (a 128-byte line per step),
@@ -1771,12 +1785,17 @@ __device__ __forceinline__ void saddle_tile_apply_body(
         if (bytes > 0) sa_bulk_load(sa_smem_u32(smem), fac + o, bytes, b);
         else asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
     }
+    // the map and the weights are constant: fetched before the wait
+    constexpr int PRE = 4;
+    int jd[PRE];
+    float w[PRE];
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) jd[u] = tid + u * NT < n ? __ldg(pdofs + s0 + tid + u * NT) : -1;
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) w[u] = jd[u] >= 0 ? __ldg(wt + jd[u]) : 0.f;
     pdl_wait();
     pdl_release();
-    for (int a = tid; a < n; a += NT) {
-        const int j = pdofs[s0 + a];
-        const float v = r[j];
-        wq[a] = wt[j];
+    auto place = [&](int a, float v) {
         if (a < dnv) {
             const int c = a / nv;
             xi[(a - c * nv) * D + c] = v;
@@ -1784,6 +1803,23 @@ __device__ __forceinline__ void saddle_tile_apply_body(
         } else {
             tq[a - dnv] = v;
         }
+    };
+    {
+        float v[PRE];
+#pragma unroll
+        for (int u = 0; u < PRE; ++u)
+            if (jd[u] >= 0) v[u] = r[jd[u]];
+#pragma unroll
+        for (int u = 0; u < PRE; ++u)
+            if (jd[u] >= 0) {
+                wq[tid + u * NT] = w[u];
+                place(tid + u * NT, v[u]);
+            }
+    }
+    for (int a = tid + PRE * NT; a < n; a += NT) {
+        const int j = pdofs[s0 + a];
+        wq[a] = wt[j];
+        place(a, r[j]);
     }
     if (tid < 4 * D && dnv + tid < 4 * n4 * D) xi[dnv + tid] = 0.f;
     if (tid < ldw - dnv) xs[dnv + tid] = 0.f;
@@ -1954,9 +1990,23 @@ __device__ __forceinline__ void saddle_apply_bulk_body(
         if (bytes > 0) sa_bulk_load(sa_smem_u32(smem), fac + o, bytes, b);
         else asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(b) : "memory");
     }
+    // (the map and the weights, constant too, before the wait)
+    constexpr int PRE = 4;
+    int jd[PRE];
+    T w[PRE];
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) jd[u] = tid + u * NT < n ? __ldg(pdofs + s0 + tid + u * NT) : -1;
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) w[u] = jd[u] >= 0 ? __ldg(wt + jd[u]) : T(0);
     pdl_wait();
     pdl_release();
-    for (int a = tid; a < n; a += NT) {
+#pragma unroll
+    for (int u = 0; u < PRE; ++u)
+        if (jd[u] >= 0) {
+            xs[tid + u * NT] = r[jd[u]];
+            wq[tid + u * NT] = w[u];
+        }
+    for (int a = tid + PRE * NT; a < n; a += NT) {
         const int j = pdofs[s0 + a];
         xs[a] = r[j];
         wq[a] = wt[j];

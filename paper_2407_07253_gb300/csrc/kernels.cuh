@@ -480,17 +480,40 @@ __global__ void __launch_bounds__(256) pull_scatter(int n, const int* __restrict
             rdst += (long long)blockIdx.y * n;
         }
     }
+    // the map is constant: the first DoF's slots (eight at most) and weight are
+    // fetched before the wait for the kernel that wrote Y
+    constexpr int PRE = 8;
+    int j = blockIdx.x * blockDim.x + threadIdx.x;
+    int q = 0, e = 0, idx[PRE];
+    if (j < n) {
+        q = __ldg(soff + j);
+        e = __ldg(soff + j + 1);
+#pragma unroll
+        for (int u = 0; u < PRE; ++u) idx[u] = q + u < e ? __ldg(sidx + q + u) : 0;
+    }
     pdl_wait();
     pdl_release();
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        T s = 0;
-        const int e = soff[j + 1];
-        for (int q = soff[j]; q < e; ++q) s += Y[sidx[q]];
+    for (; j < n;) {
+        T y[PRE], s = 0;
+#pragma unroll
+        for (int u = 0; u < PRE; ++u)
+            if (q + u < e) y[u] = Y[idx[u]];
+#pragma unroll
+        for (int u = 0; u < PRE; ++u)
+            if (q + u < e) s += y[u];
+        for (int k = q + PRE; k < e; ++k) s += Y[__ldg(sidx + k)];
         const T o = beta == T(0) ? alpha * s : alpha * s + beta * out[j];
         out[j] = o;
         if (xmode == PULL_X_SET) x[j] = o;
         else if (xmode == PULL_X_ADD) x[j] += o;
         if (rdst) rdst[j] = bsrc[j];
+        j += gridDim.x * blockDim.x;
+        if (j < n) {
+            q = __ldg(soff + j);
+            e = __ldg(soff + j + 1);
+#pragma unroll
+            for (int u = 0; u < PRE; ++u) idx[u] = q + u < e ? __ldg(sidx + q + u) : 0;
+        }
     }
 }
 
@@ -535,13 +558,26 @@ __global__ void __launch_bounds__(256) dense_gemv(int nout, int ncol, int lda, c
         x += (long long)blockIdx.y * ncol;
         y += (long long)blockIdx.y * nout;
     }
-    pdl_wait();
-    pdl_release();
     const int lane = threadIdx.x & 31;
     const int row = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    // A is constant: the row's first entries are fetched before the wait
+    constexpr int PRE = 8;
+    double a[PRE];
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) {
+        const int j = lane + 32 * u;
+        a[u] = row < nout && j < ncol ? __ldg(A + (long long)row * lda + j) : 0.0;
+    }
+    pdl_wait();
+    pdl_release();
     if (row >= nout) return;
     double s = 0;
-    for (int j = lane; j < ncol; j += 32) s += A[(long long)row * lda + j] * (double)x[j];
+#pragma unroll
+    for (int u = 0; u < PRE; ++u) {
+        const int j = lane + 32 * u;
+        if (j < ncol) s += a[u] * (double)x[j];
+    }
+    for (int j = lane + 32 * PRE; j < ncol; j += 32) s += __ldg(A + (long long)row * lda + j) * (double)x[j];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     if (lane == 0) y[row] = (TO)s;
 }
