@@ -455,9 +455,10 @@ __device__ void gj_store(const double* A, int n, double* inv64, long long o64, f
 __global__ void __launch_bounds__(256) gj_inverse_smem(int npatch, const int* __restrict__ poff, const long long* __restrict__ moff,
                                                        double* __restrict__ work, const long long* __restrict__ off64,
                                                        double* __restrict__ inv64, const long long* __restrict__ off32,
-                                                       float* __restrict__ inv32, int* __restrict__ status, int) {
+                                                       float* __restrict__ inv32, int* __restrict__ status, int retry) {
     extern __shared__ double smem[];
     const int p = blockIdx.x;
+    if (retry && status[p] == 0) return;
     const int n = poff[p + 1] - poff[p];
     if (n > GJ_SMEM_MAX_N || n == 0) return;
     double* A = smem;
@@ -480,8 +481,10 @@ __global__ void __launch_bounds__(512) gj_inverse_global(int npatch, const int* 
                                                          double* __restrict__ work, const long long* __restrict__ off64,
                                                          double* __restrict__ inv64, const long long* __restrict__ off32,
                                                          float* __restrict__ inv32, int* __restrict__ status,
-                                                         int* __restrict__ ipiv_ws, double* __restrict__ col_ws) {
+                                                         int* __restrict__ ipiv_ws, double* __restrict__ col_ws,
+                                                         int retry) {
     const int p = blockIdx.x;
+    if (retry && status[p] == 0) return;
     const int n = poff[p + 1] - poff[p];
     if (n <= GJ_SMEM_MAX_N) return;
     __shared__ int st;
@@ -1094,7 +1097,7 @@ __global__ void __launch_bounds__(256) saddle_inverse_global(int npatch, int d, 
 //   A -= U^T V on every tile (64 FMAs between 128 bytes read and written), and
 //   row K becomes V, A[K, K] becomes -P; after the last step A holds -A^-1.
 // The FP64 pipe (2 FMA lanes per SM and clock) bounds it: 1089 patches of the
-// P8 stars on 32 x 32 took 38.2 ms, NEW_P8 now; the padding to tiles adds 4% to the
+// P8 stars on 32 x 32 took 38.2 ms, 24.9 now (79% of the pipe); the padding to tiles adds 4% to the
 // FMAs at 217 nodes, the 4 x 4 inverses and V another 8%.
 // A tile's entry (r, c) is double c & 1 of 16-byte group 2 r + c / 2, groups
 // [8][ntile], so that the threads of a warp, on consecutive tiles, read and
@@ -1369,6 +1372,60 @@ SADDLE_TILES_KERNEL(saddle_inverse_tiles_512, 512)
 SADDLE_TILES_KERNEL(saddle_inverse_tiles_256, 256)
 SADDLE_TILES_KERNEL(saddle_inverse_tiles_128, 128)
 #undef SADDLE_TILES_KERNEL
+
+// Explicit inverses of SPD patch blocks (row-major in work) of lo < n <= hi, by
+// the same sweep: half the FMAs of Gauss-Jordan and no pivot search (FBF's star
+// blocks on the SV disk, 5671 of up to 161 nodes: 2.4-4.7 -> 0.9-1.1 ms).  work is left as
+// it is, for gj_inverse_* with retry on the patches whose status is not 0.
+template <int NT>
+__device__ __forceinline__ void spd_tiles_body(int lo, int hi, const int* __restrict__ poff, const long long* __restrict__ moff,
+                                               const double* __restrict__ work, const long long* __restrict__ off64,
+                                               double* __restrict__ inv64, const long long* __restrict__ off32,
+                                               float* __restrict__ inv32, int* __restrict__ status, unsigned char* smem) {
+    const int tid = threadIdx.x, p = blockIdx.x, n = poff[p + 1] - poff[p];
+    if (n <= lo || n > hi) return;
+    const int n4 = (n + 3) >> 2, ntile = n4 * (n4 + 1) / 2;
+    double2* T = reinterpret_cast<double2*>(smem);                      // [8][ntile]
+    double* U = reinterpret_cast<double*>(T + 8 * (size_t)ntile);       // [4][4 n4]
+    double* V = U + 16 * n4;                                            // [4][4 n4]
+    double* P = V + 16 * n4;                                            // [16]
+    ushort2* map = reinterpret_cast<ushort2*>(P + 16);                  // [ntile]
+    __shared__ int st;
+    if (tid == 0) st = 0;
+    tile_map(n4, map);
+    __syncthreads();
+    const double* A = work + moff[p];
+    for (int x = tid; x < 16 * ntile; x += NT) {
+        const int r = x / (4 * ntile), y = x - r * 4 * ntile, t = y >> 2, c = y & 3;
+        const int i = 4 * map[t].x + r, j = 4 * map[t].y + c;
+        tile_at(T, ntile, t, r, c) = i < n && j < n ? A[(long long)i * n + j] : i == j ? 1.0 : 0.0;
+    }
+    __syncthreads();
+    sweep_tiles(T, n4, map, U, V, P, &st);
+    const int ld64 = (n + 1) & ~1, ld32 = (n + 3) & ~3;
+    for (int x = tid; x < ld32 * n; x += NT) {
+        const int j = x / ld32, i = x - j * ld32;
+        double v = 0.0;
+        if (i < n) {
+            const int a = min(i, j), b = max(i, j);
+            v = flip(tile_at(T, ntile, tile_row(n4, a >> 2) + (b >> 2), a & 3, b & 3));
+        }
+        if (inv64 && i < ld64) inv64[off64[p] + (long long)j * ld64 + i] = v;
+        if (inv32) inv32[off32[p] + x] = (float)v;
+    }
+    if (tid == 0) status[p] = st;
+}
+#define SPD_TILES_KERNEL(NT)                                                                                           \
+    __global__ void __launch_bounds__(NT, 512 / NT) spd_inverse_tiles_##NT(                                            \
+        int lo, int hi, const int* __restrict__ poff, const long long* __restrict__ moff,                              \
+        const double* __restrict__ work, const long long* __restrict__ off64, double* __restrict__ inv64,              \
+        const long long* __restrict__ off32, float* __restrict__ inv32, int* __restrict__ status) {                    \
+        extern __shared__ __align__(16) unsigned char smem_pt[];                                                       \
+        spd_tiles_body<NT>(lo, hi, poff, moff, work, off64, inv64, off32, inv32, status, smem_pt);                     \
+    }
+SPD_TILES_KERNEL(128)
+SPD_TILES_KERNEL(512)
+#undef SPD_TILES_KERNEL
 
 // One ASM sweep.  The patch inverse is column-major with its leading
 // dimension padded to VEC rows; a thread owns VEC consecutive rows (one

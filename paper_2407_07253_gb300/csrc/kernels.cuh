@@ -260,16 +260,17 @@ __global__ void patch_gather(int npatch, const int* __restrict__ poff, const int
 // Writes K_i^{-1} column-major with leading dimension ld64 (FP64) and, if
 // inv32 != nullptr, ld32 (FP32); the row-major inverse is also written back
 // to `work` when keep_rowmajor.  status[patch] = 0, or 1 + pivot step of the
-// first zero pivot.
+// first zero pivot.  retry: only the patches whose status is not 0.
 __global__ void gj_inverse_smem(int npatch, const int* __restrict__ poff, const long long* __restrict__ moff,
                                 double* __restrict__ work, const long long* __restrict__ off64, double* __restrict__ inv64,
                                 const long long* __restrict__ off32, float* __restrict__ inv32,
-                                int* __restrict__ status, int only_large);
+                                int* __restrict__ status, int retry);
 // Same algorithm operating on the matrix in global memory (large patches).
 __global__ void gj_inverse_global(int npatch, const int* __restrict__ poff, const long long* __restrict__ moff,
                                   double* __restrict__ work, const long long* __restrict__ off64, double* __restrict__ inv64,
                                   const long long* __restrict__ off32, float* __restrict__ inv32,
-                                  int* __restrict__ status, int* __restrict__ ipiv_ws, double* __restrict__ col_ws);
+                                  int* __restrict__ status, int* __restrict__ ipiv_ws, double* __restrict__ col_ws,
+                                  int retry);
 
 // Block (Schur-complement) inverse of saddle-structured Vanka patches:
 // K_i = [L 0 B_0^T; 0 L B_1^T; B_0 B_1 0] with one SPD velocity block L per
@@ -352,6 +353,21 @@ __global__ void saddle_inverse_tiles_512(SADDLE_TILES_ARGS);
 __global__ void saddle_inverse_tiles_256(SADDLE_TILES_ARGS);
 __global__ void saddle_inverse_tiles_128(SADDLE_TILES_ARGS);
 #undef SADDLE_TILES_ARGS
+// Explicit inverses of SPD blocks of lo < n <= hi (work row-major, kept),
+// outputs and status as gj_inverse_*; spd_tiles_smem(min(hi, largest n)) bytes.
+// Up to SPD_TILES_SMALL_N six CTAs of 128 threads share an SM.
+constexpr int SPD_TILES_SMALL_N = 88, SPD_TILES_MAX_N = 220;
+__host__ __device__ inline size_t spd_tiles_smem(int n) {
+    const size_t n4 = (n + 3) / 4, nt = n4 * (n4 + 1) / 2;
+    return nt * (128 + 4) + sizeof(double) * (32 * n4 + 16);
+}
+#define SPD_TILES_ARGS                                                                                                 \
+    int lo, int hi, const int *__restrict__ poff, const long long *__restrict__ moff, const double *__restrict__ work, \
+        const long long *__restrict__ off64, double *__restrict__ inv64, const long long *__restrict__ off32,          \
+        float *__restrict__ inv32, int *__restrict__ status
+__global__ void spd_inverse_tiles_128(SPD_TILES_ARGS);
+__global__ void spd_inverse_tiles_512(SPD_TILES_ARGS);
+#undef SPD_TILES_ARGS
 // Elements of one patch's factored inverse (Li, W, Si with leading
 // dimensions rounded up to vec = 2 (FP64) or 4 (FP32)).  Li's form, packed:
 // 0 column-major; 1 its upper triangle row by row (nv (nv + 1) / 2 entries,

@@ -134,7 +134,7 @@ extern "C" int stokes_batched_inverse_noalloc(int npatch, const int* sizes, doub
     if ((e = cudaGetLastError()) != cudaSuccess) return fail(STOKES_ECUDA, cudaGetErrorString(e));
     if (nmax > skern::GJ_SMEM_MAX_N) {
         skern::gj_inverse_global<<<npatch, 512, 0, s>>>(npatch, poff, moff, mats, nullptr, nullptr, nullptr, nullptr,
-                                                        status, ipiv, col);
+                                                        status, ipiv, col, 0);
         if ((e = cudaGetLastError()) != cudaSuccess) return fail(STOKES_ECUDA, cudaGetErrorString(e));
     }
     if ((e = cudaMemcpyAsync(h_status, status, sizeof(int) * npatch, cudaMemcpyDeviceToHost, s)) != cudaSuccess ||

@@ -1440,7 +1440,11 @@ void fbf_apply(stokes_mg* h, const double* r, double* z, cudaStream_t s) {
     vcycles(r, F.a);
     CK(cudaMemcpyAsync(F.t, F.a, sizeof(double) * nu, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemsetAsync(F.t + nu, 0, sizeof(double) * np, s));
-    spmv<double>(h, PK_SPMV, F.S0d.K, skern::SPMV_SET, F.t, F.w, nullptr, s);      // w_p = B a
+    DevCSR Bp = F.S0d.K;                                                            // its pressure rows (a fifth of the entries)
+    Bp.rp += nu;
+    Bp.nr = np;
+    Bp.nvf = 0;
+    spmv<double>(h, PK_SPMV, Bp, skern::SPMV_SET, F.t, F.w + nu, nullptr, s);       // w_p = B a
     axpby_l<double>(h, np, 1.0, r + nu, -1.0, F.w + nu, s);                         // w_p = r_p - B a
     launch(h, -1, s, [&] {
         skern::block_mass_inverse<<<grid_for((long long)F.ncell * F.nbq), 256, 0, s>>>(F.ncell, F.nbq, F.qcell, F.minv,
@@ -2067,6 +2071,23 @@ void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status,
         }
         return;
     }
+    // FBF's scalar star blocks are SPD: swept on tiles first, the patches that
+    // fail there (an indefinite block) left to the pivoting below
+    const bool spd = h->fbf && store && l.maxn <= skern::SPD_TILES_MAX_N;
+    if (spd) {
+        auto sweep = [&](auto kern, int nt, int lo, int hi) {
+            const size_t sm = skern::spd_tiles_smem(std::min(hi, l.maxn));
+            CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)skern::spd_tiles_smem(std::min(hi, skern::SPD_TILES_MAX_N))));
+            launch(h, PK_GJ, s, [&] {
+                kern<<<l.npatch, nt, sm, s>>>(lo, hi, l.poff, l.moff, work, i64 ? l.ioff64 : nullptr, i64,
+                                              i32 ? l.ioff32 : nullptr, i32, status);
+            });
+        };
+        sweep(skern::spd_inverse_tiles_128, 128, 0, skern::SPD_TILES_SMALL_N);
+        if (l.maxn > skern::SPD_TILES_SMALL_N)
+            sweep(skern::spd_inverse_tiles_512, 512, skern::SPD_TILES_SMALL_N, skern::SPD_TILES_MAX_N);
+    }
     const int nsm = std::min(l.maxn, skern::GJ_SMEM_MAX_N);
     const size_t smem = (size_t)nsm * nsm * sizeof(double) + nsm * sizeof(double) + nsm * sizeof(int) + 64;
     {
@@ -2076,14 +2097,14 @@ void gather_and_invert(stokes_mg* h, int li, double* work, int out, int* status,
     }
     launch(h, PK_GJ, s, [&] {
         skern::gj_inverse_smem<<<l.npatch, 256, smem, s>>>(l.npatch, l.poff, l.moff, work, i64 ? l.ioff64 : nullptr, i64,
-                                                           i32 ? l.ioff32 : nullptr, i32, status, 0);
+                                                           i32 ? l.ioff32 : nullptr, i32, status, spd ? 1 : 0);
     });
     if (l.maxn > skern::GJ_SMEM_MAX_N) {
         int* ipiv = palloc<int>(h->device, l.nent, s);
         double* col = palloc<double>(h->device, l.nent, s);
         launch(h, PK_GJ, s, [&] {
             skern::gj_inverse_global<<<l.npatch, 512, 0, s>>>(l.npatch, l.poff, l.moff, work, i64 ? l.ioff64 : nullptr, i64,
-                                                              i32 ? l.ioff32 : nullptr, i32, status, ipiv, col);
+                                                              i32 ? l.ioff32 : nullptr, i32, status, ipiv, col, spd ? 1 : 0);
         });
         CK(cudaFreeAsync(ipiv, s));
         CK(cudaFreeAsync(col, s));
