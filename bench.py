@@ -400,14 +400,14 @@ def batched_section(a, P, W, dev, stream, flush, hbm):
     gemm_bytes = 4.0 * float((n_i * ld_i).sum()) + 4.0 * m * float(n_i.sum()) + 4.0 * m * n
     gemm_flop = 2.0 * m * float((n_i * n_i).sum())
     gemm_gbs = gemm_bytes / (gemm_ms * 1e-3) / 1e9
-    # DRAM traffic per launch: the last ncu capture of the tensor-core launch
-    # (level 0 of th_p3_cube8 at 64 right-hand sides, batch_tune 0:
-    # dram__bytes_read.sum + dram__bytes_write.sum = 440.98 + 43.14 MB
-    # against 471.24 MB of algorithmic bytes) predates the 3xTF32 split of the
-    # kernel, so no traffic is reported for the current kernel
+    # DRAM traffic per launch: the last ncu capture of the TF32 tensor-core
+    # launch (level 0 of th_p3_cube8 at 64 right-hand sides, batch_tune 0:
+    # dram__bytes_read.sum + dram__bytes_write.sum = 440.98 + 43.14 MB against
+    # 471.24 MB of algorithmic bytes) predates the kernel's present form, so no
+    # traffic is reported for it
     traffic = None
-    traffic_src = ("not re-captured since the kernel gained its 3xTF32 split; the TF32 launch measured "
-                   "484.1 MB for 471.2 MB algorithmic (1.03x) on th_p3_cube8 before that change")
+    traffic_src = ("not re-captured for the kernel's present form; an earlier TF32 launch measured 484.1 MB for "
+                   "471.2 MB algorithmic (1.03x) on th_p3_cube8")
     return {
         "workload": a.batched_workload, "nrhs": m, "n_free": n, "relaxed_levels": npatch_levels,
         "vcycle_ms": {"tf32": tf32_ms, "3xtf32": x3_ms, "single_rhs_mixed_per_rhs": single_ms},
@@ -979,8 +979,9 @@ def main():
                 zq = np.asarray((K[pd[c == cc]][:, pres] != 0).sum(axis=0)).ravel().astype(float)
                 f += 2 * nv * zq.sum() + 2 * float((zq * (npr - np.arange(len(zq)))).sum())
             nvi, npi = int(nv), int(npr)
-            # L^-1 as its packed upper triangle (the bulk-copy apply's layout)
-            by += 4.0 * (up4(nvi * (nvi + 1) // 2) + up4(d * nvi) * npi + up4(npi) * npi) + 12.0 * (d * nvi + npi)
+            # L^-1 as the 4 x 4 tiles of its upper triangle (the FP32 bulk-copy apply's layout)
+            n4 = (nvi + 3) // 4
+            by += 4.0 * (8 * n4 * (n4 + 1) + up4(d * nvi) * npi + up4(npi) * npi) + 12.0 * (d * nvi + npi)
         flops_levels.append(f)
         apply_bytes.append(by)
         sizes.append(np.diff(off))
@@ -1036,8 +1037,8 @@ def main():
                      "flop_per_launch": flops_levels[0], "ms_per_launch": gj0_ms,
                      "all_levels": {"launches_per_step": gj_launches_per_step, "ms_per_step": gj_ms_per_step,
                                     "flop_per_step": flops_gj, "achieved": achieved_gj}},
-        "roofline_solve": {"kernel": "saddle_apply_bulk_f32, level 0 (one ASM sweep over the factored FP32 inverses, "
-                                     "L^-1 packed, one bulk copy per patch)",
+        "roofline_solve": {"kernel": "saddle_tile_apply, level 0 (one ASM sweep over the factored FP32 inverses, "
+                                     "L^-1 as 4 x 4 tiles, one bulk copy per patch)",
                            "bound": "hbm",
                            "achieved": patch_gbs, "peak": hbm, "unit": "GB/s",
                            "frac": (patch_gbs / hbm) if patch_gbs else None, "bytes_per_launch": patch_bytes,

@@ -1093,11 +1093,11 @@ __global__ void __launch_bounds__(256) saddle_inverse_global(int npatch, int d, 
 // TH P6 and up, SV P4, 3D P3).  One pivot at a time in a global scratch costs a
 // read and a write of the whole block per pivot, from L2; here the upper
 // triangle's 4 x 4 tiles stay in shared memory and a step sweeps four pivots:
-//   U = A[K, :] (4 x n, published), P = A[K, K]^-1 (one warp), V = P U,
+//   U = A[K, :] (4 x n, published), P = A[K, K]^-1 (one warp, a step ahead), V = P U,
 //   A -= U^T V on every tile (64 FMAs between 128 bytes read and written), and
 //   row K becomes V, A[K, K] becomes -P; after the last step A holds -A^-1.
 // The FP64 pipe (2 FMA lanes per SM and clock) bounds it: 1089 patches of the
-// P8 stars on 32 x 32 took 38.2 ms, 24.9 now (79% of the pipe); the padding to tiles adds 4% to the
+// P8 stars on 32 x 32 took 38.2 ms, 24.0 now (79% of the pipe at 24.9); the padding to tiles adds 4% to the
 // FMAs at 217 nodes, the 4 x 4 inverses and V another 8%.
 // A tile's entry (r, c) is double c & 1 of 16-byte group 2 r + c / 2, groups
 // [8][ntile], so that the threads of a warp, on consecutive tiles, read and
@@ -1113,32 +1113,43 @@ __device__ __forceinline__ void tile_map(int n4, ushort2* map) {
         for (int J = I + lane; J < n4; J += 32) map[tile_row(n4, I) + J] = make_ushort2(I, J);
 }
 
-// All threads of the CTA; T, U [4][4 n4], V [4][4 n4], P [16] in shared memory.
-// status <- 1 + step of the first non-positive pivot.
+// P = -(the swept 4 x 4 block v), one entry per lane (r, c) = (lane / 4 % 4, lane % 4)
+// of a whole warp, the upper half-warp repeating the lower; step0: its first pivot
+__device__ __forceinline__ void sweep_4x4(double v, int step0, double* P, int* status) {
+    const int lane = threadIdx.x & 31, r = (lane >> 2) & 3, c = lane & 3;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double piv = __shfl_sync(0xffffffffu, v, 5 * k);
+        const double vrk = __shfl_sync(0xffffffffu, v, 4 * r + k), vkc = __shfl_sync(0xffffffffu, v, 4 * k + c);
+        const double inv = piv > 0.0 ? 1.0 / piv : 0.0;
+        if (lane == 0 && !(piv > 0.0) && *status == 0) *status = step0 + k + 1;
+        const double w = vrk * inv;
+        v = r == k ? (c == k ? flip(inv) : vkc * inv) : (c == k ? w : fma(-w, vkc, v));
+    }
+    if (lane < 16) P[lane] = flip(v);
+}
+
+// All threads of the CTA; T, U [4][4 n4], V [4][4 n4], P [2][16] in shared memory.
+// The 4 x 4 inverse is a chain of some forty dependent FP64 operations (about 4000
+// cycles, against 50,000 for the update of 55 tile rows and 17,000 for 32): warp 0
+// forms the next step's during the update, from its diagonal tile updated on the
+// side, and the warps take the tiles from a counter, 32 at a time, so that it costs
+// nobody a wait: P8 32 x 32 24.9 -> 24.0 ms, SV P4 disk 12.1 -> 11.7.  status <- 1 + step of the first
+// non-positive pivot.
 __device__ void sweep_tiles(double2* T, int n4, const ushort2* map, double* U, double* V, double* P, int* status) {
+    __shared__ int next;
     const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
     const int ntile = n4 * (n4 + 1) / 2, ldu = 4 * n4;
+    const int lr = (lane >> 2) & 3, lc = lane & 3;
+    if (n4 == 0) return;
+    if (warp == 0) sweep_4x4(tile_at(T, ntile, 0, lr, lc), 0, P, status);
     for (int K = 0; K < n4; ++K) {
+        const double* Pk = P + 16 * (K & 1);
+        if (tid == 0) next = 0;
         for (int x = tid; x < 16 * n4; x += nt) {
             const int J = x >> 4, k = (x >> 2) & 3, c = x & 3;
             U[k * ldu + 4 * J + c] = J >= K ? tile_at(T, ntile, tile_row(n4, K) + J, k, c)
                                             : tile_at(T, ntile, tile_row(n4, J) + K, c, k);
-        }
-        __syncthreads();
-        if (warp == 0) {
-            // the 4 x 4 sweep, one entry per lane (the upper half-warp repeats the lower)
-            const int r = (lane >> 2) & 3, c = lane & 3;
-            double v = U[r * ldu + 4 * K + c];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const double piv = __shfl_sync(0xffffffffu, v, 5 * k);
-                const double vrk = __shfl_sync(0xffffffffu, v, 4 * r + k), vkc = __shfl_sync(0xffffffffu, v, 4 * k + c);
-                const double inv = piv > 0.0 ? 1.0 / piv : 0.0;
-                if (lane == 0 && !(piv > 0.0) && *status == 0) *status = 4 * K + k + 1;
-                const double w = vrk * inv;
-                v = r == k ? (c == k ? flip(inv) : vkc * inv) : (c == k ? w : fma(-w, vkc, v));
-            }
-            if (lane < 16) P[lane] = flip(v);
         }
         __syncthreads();
         for (int j = tid; j < ldu; j += nt) {
@@ -1147,14 +1158,28 @@ __device__ void sweep_tiles(double2* T, int n4, const ushort2* map, double* U, d
             for (int l = 0; l < 4; ++l) u[l] = U[l * ldu + j];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                double v = P[4 * k] * u[0];
+                double v = Pk[4 * k] * u[0];
 #pragma unroll
-                for (int l = 1; l < 4; ++l) v = fma(P[4 * k + l], u[l], v);
+                for (int l = 1; l < 4; ++l) v = fma(Pk[4 * k + l], u[l], v);
                 V[k * ldu + j] = v;
             }
         }
+        // the next diagonal tile as it is before this step's update
+        const bool ahead = warp == 0 && K + 1 < n4;
+        double dg = ahead ? tile_at(T, ntile, tile_row(n4, K + 1) + K + 1, lr, lc) : 0.0;
         __syncthreads();
-        for (int t = tid; t < ntile; t += nt) {
+        if (ahead) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) dg = fma(-U[k * ldu + 4 * (K + 1) + lr], V[k * ldu + 4 * (K + 1) + lc], dg);
+            sweep_4x4(dg, 4 * (K + 1), P + 16 * ((K + 1) & 1), status);
+        }
+        for (;;) {
+            int w = 0;
+            if (lane == 0) w = atomicAdd(&next, 32);
+            w = __shfl_sync(0xffffffffu, w, 0);
+            if (w >= ntile) break;
+            const int t = w + lane;
+            if (t >= ntile) continue;
             const int I = map[t].x, J = map[t].y;
             double a[4][4];
             if (I == K || J == K) {
@@ -1162,7 +1187,7 @@ __device__ void sweep_tiles(double2* T, int n4, const ushort2* map, double* U, d
                 for (int r = 0; r < 4; ++r)
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
-                        a[r][c] = I == J ? flip(P[4 * r + c]) : I == K ? V[r * ldu + 4 * J + c] : V[c * ldu + 4 * I + r];
+                        a[r][c] = I == J ? flip(Pk[4 * r + c]) : I == K ? V[r * ldu + 4 * J + c] : V[c * ldu + 4 * I + r];
             } else {
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
@@ -1219,8 +1244,8 @@ __device__ __forceinline__ void saddle_tiles_body(
     double2* T = reinterpret_cast<double2*>(smem);                                     // [8][ntile]
     double* U = reinterpret_cast<double*>(T + 8 * (size_t)maxt);                       // [4][4 max4]
     double* V = U + 16 * max4;                                                         // [4][4 max4]
-    double* P = V + 16 * max4;                                                         // [16]
-    ushort2* map = reinterpret_cast<ushort2*>(P + 16);                                 // [maxt]
+    double* P = V + 16 * max4;                                                         // [2][16]
+    ushort2* map = reinterpret_cast<ushort2*>(P + 32);                                 // [maxt]
     int* coff = reinterpret_cast<int*>(map + maxt);                                    // [np][d + 1]
     int* sd = coff + max_np * (d + 1);                                                 // [n]
     __shared__ int st;
@@ -1388,8 +1413,8 @@ __device__ __forceinline__ void spd_tiles_body(int lo, int hi, const int* __rest
     double2* T = reinterpret_cast<double2*>(smem);                      // [8][ntile]
     double* U = reinterpret_cast<double*>(T + 8 * (size_t)ntile);       // [4][4 n4]
     double* V = U + 16 * n4;                                            // [4][4 n4]
-    double* P = V + 16 * n4;                                            // [16]
-    ushort2* map = reinterpret_cast<ushort2*>(P + 16);                  // [ntile]
+    double* P = V + 16 * n4;                                            // [2][16]
+    ushort2* map = reinterpret_cast<ushort2*>(P + 32);                  // [ntile]
     __shared__ int st;
     if (tid == 0) st = 0;
     tile_map(n4, map);

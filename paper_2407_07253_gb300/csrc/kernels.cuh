@@ -337,7 +337,7 @@ constexpr size_t SADDLE_TILES_SMEM_MAX = 226 * 1024;
 constexpr int SADDLE_TILES_MIN_N = 80;
 __host__ __device__ inline size_t saddle_tiles_smem(int d, int max4, int max_np, int max_n) {
     const size_t nt = (size_t)max4 * (max4 + 1) / 2;
-    return nt * (128 + 4) + sizeof(double) * (32 * (size_t)max4 + 16) + sizeof(int) * ((size_t)max_np * (d + 1) + max_n);
+    return nt * (128 + 4) + sizeof(double) * (32 * (size_t)max4 + 32) + sizeof(int) * ((size_t)max_np * (d + 1) + max_n);
 }
 __host__ __device__ inline long long saddle_tiles_scratch(int d, int n, int nv) {
     const long long dnv = (long long)d * nv, np = n - dnv;
@@ -359,7 +359,7 @@ __global__ void saddle_inverse_tiles_128(SADDLE_TILES_ARGS);
 constexpr int SPD_TILES_SMALL_N = 88, SPD_TILES_MAX_N = 220;
 __host__ __device__ inline size_t spd_tiles_smem(int n) {
     const size_t n4 = (n + 3) / 4, nt = n4 * (n4 + 1) / 2;
-    return nt * (128 + 4) + sizeof(double) * (32 * n4 + 16);
+    return nt * (128 + 4) + sizeof(double) * (32 * n4 + 32);
 }
 #define SPD_TILES_ARGS                                                                                                 \
     int lo, int hi, const int *__restrict__ poff, const long long *__restrict__ moff, const double *__restrict__ work, \
