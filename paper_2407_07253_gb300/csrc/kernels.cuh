@@ -178,12 +178,13 @@ __global__ void __launch_bounds__(256) spmv_stokes(int nvf, int nq, const int* _
 #pragma unroll
         for (int c = 1; c < D; ++c) acc[0] += acc[c];
     }
+    // every live lane takes part in every shuffle: a warp may hold the last
+    // velocity nodes and the first pressure rows
 #pragma unroll
     for (int c = 0; c < D; ++c) {
-        if (c > 0 && !vel) break;
 #pragma unroll
         for (int o = LANES / 2; o > 0; o >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o, LANES);
-        if (lane == 0) {
+        if (lane == 0 && (c == 0 || vel)) {
             const int i = row + c * nvf;
             y[i] = MODE == SPMV_SET ? acc[c] : b[i] - acc[c];
         }
