@@ -219,9 +219,10 @@ int stokes_fgmres_batched(stokes_mg_t h, const double* b_dev, double* x_dev, int
 
 /* Self-test of the bounded mbarrier wait used by the tensor-core kernels
  * (no counterpart in the paper): one CTA waits on a barrier that nothing
- * arrives on, gives up after `polls` polls and returns; *result = 2 then
- * (1 would mean the barrier phase completed, 0 that the kernel never ran).
- * Errors: EINVAL, ECUDA. */
+ * arrives on, gives up after `polls` polls and returns; then its lanes wait
+ * with different numbers of polls and have to come to one outcome.
+ * *result = 2 then (1 would mean that a wait succeeded, 3 that the lanes
+ * disagree, 0 that the kernel never ran).  Errors: EINVAL, ECUDA. */
 int stokes_selftest_bounded_wait(long long polls, int* result);
 
 /* Measurement utility (no counterpart in the paper): the FP64 pipe's peak on

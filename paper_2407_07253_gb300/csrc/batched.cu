@@ -397,22 +397,36 @@ __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile 
     return false;
 }
 
-// self-test of the bounded wait: one CTA waits on an mbarrier that nothing
-// arrives on; *result = 2 when the wait gives up after `limit` polls and the
-// kernel returns (1 would mean the phase completed)
+// the same for a whole converged warp, with one outcome for all its lanes: each
+// polls for itself, so at a timeout some may see the phase complete and others
+// the abort flag, and those that went on would wait in elect.sync, __syncwarp or
+// tcgen05.ld for the ones that left
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t a, uint32_t parity, volatile int* abort_flag,
+                                               long long limit = WAIT_LIMIT) {
+    return __all_sync(0xffffffffu, mbar_wait(a, parity, abort_flag, limit));
+}
+
+// self-test of the bounded waits: one CTA of one warp waits on an mbarrier that
+// nothing arrives on; then the lanes wait for a phase that is over, the odd ones
+// with no polls at all, so that they differ on their own.  *result = 2 when both
+// waits give up for all lanes alike and the kernel returns (1 would mean a
+// completed phase, 3 lanes that disagree)
 __global__ void k_wait_probe(long long limit, int* result) {
-    __shared__ __align__(8) unsigned long long bar;
-    __shared__ int abort_flag;
-    const uint32_t a = smem_u32(&bar);
+    __shared__ __align__(8) unsigned long long bar[2];
+    __shared__ int abort_flag[2];
+    const uint32_t a = smem_u32(bar), b = smem_u32(bar + 1);
     if (threadIdx.x == 0) {
         mbar_init(a, 1);
-        abort_flag = 0;
+        mbar_init(b, 1);
+        abort_flag[0] = abort_flag[1] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        mbar_arrive(b);
     }
     __syncthreads();
-    const bool ok = mbar_wait(a, 0, &abort_flag, limit);
-    __syncthreads();
-    if (threadIdx.x == 0) *result = ok ? 1 : 2;
+    const bool ok = mbar_wait_warp(a, 0, abort_flag, limit);
+    const bool mixed = mbar_wait_warp(b, 0, abort_flag + 1, threadIdx.x & 1 ? 0 : limit);
+    const unsigned agree = __match_any_sync(0xffffffffu, (ok ? 1 : 0) | (mixed ? 2 : 0));
+    if (threadIdx.x == 0) *result = agree != 0xffffffffu ? 3 : ok || mixed ? 1 : 2;
 }
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const void* tmap, uint32_t mbar, int x, int y) {
     asm volatile(
@@ -557,11 +571,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
             item(pc, p, s0, n);
             const int tiles = tiles_of(n), nst = (n + KS - 1) / KS;
             const int b = pc % nbuf;
-            if (pc >= nbuf && !mbar_wait(acce0 + 8 * b, ((pc / nbuf) - 1) & 1, abort_flag)) goto done;
+            if (pc >= nbuf && !mbar_wait_warp(acce0 + 8 * b, ((pc / nbuf) - 1) & 1, abort_flag)) goto done;
             fence_after();
             const uint32_t acc = tmem + (uint32_t)(b * ccols);
             for (int j = 0; j < nst; ++j) {
-                if (!mbar_wait(full0 + 8 * s, ph, abort_flag)) goto done;
+                if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag)) goto done;
                 fence_after();
                 const uint32_t so = (uint32_t)(s * sbytes) >> 4;
                 const uint32_t lo = SPLIT ? (uint32_t)(ls * lo_bytes(maxn)) >> 4 : 0;
@@ -626,7 +640,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
                                        ? __ldg(reinterpret_cast<const float4*>(X + (long long)dof[k4] * M + c))
                                        : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
-                if (it >= ST && !mbar_wait(empty0 + 8 * s, ((it / ST) - 1) & 1, abort_flag)) goto done;
+                if (it >= ST && !mbar_wait_warp(empty0 + 8 * s, ((it / ST) - 1) & 1, abort_flag)) goto done;
                 unsigned char* bp = smem_tc + (stage0 - base) + (size_t)s * sbytes + b_off;
 #pragma unroll
                 for (int k4 = 0; k4 < KS / 4; ++k4) {
@@ -657,7 +671,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
             int p, s0, n;
             item(pc, p, s0, n);
             const int tiles = tiles_of(n), b = pc % nbuf;
-            if (!mbar_wait(accf0 + 8 * b, (pc / nbuf) & 1, abort_flag)) goto done;
+            if (!mbar_wait_warp(accf0 + 8 * b, (pc / nbuf) & 1, abort_flag)) goto done;
             fence_after();
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) {
@@ -697,8 +711,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
             for (int j = 0; j < nst; ++j, ++it) {
                 if (it % ng != grp) continue;
                 const int s = it % ST;
-                if (it >= lr && !mbar_wait(empty0 + 8 * ((it - lr) % ST), ((it - lr) / ST) & 1, abort_flag)) goto done;
-                if (!mbar_wait(raw0 + 8 * s, (it / ST) & 1, abort_flag)) goto done;
+                if (it >= lr && !mbar_wait_warp(empty0 + 8 * ((it - lr) % ST), ((it - lr) / ST) & 1, abort_flag)) goto done;
+                if (!mbar_wait_warp(raw0 + 8 * s, (it / ST) & 1, abort_flag)) goto done;
                 float4* hp = reinterpret_cast<float4*>(smem_tc + (stage0 - base) + (size_t)s * sbytes);
                 float4* lp = reinterpret_cast<float4*>(smem_tc + (lo0 - base) + (size_t)(it % lr) * lo_bytes(maxn));
 #pragma unroll 4

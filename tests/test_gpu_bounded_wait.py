@@ -1,0 +1,14 @@
+"""The bounded waits of the tensor-core patch GEMM at a timeout: a warp whose
+lanes reach the limit at different polls gives up as one (a lane that went on
+alone would wait for the others in the next warp-wide instruction)."""
+import pytest
+
+torch = pytest.importorskip("torch")
+P = pytest.importorskip("paper_2407_07253_gb300")
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("polls", [0, 1, 64, 4096])
+def test_a_warp_gives_up_as_one(polls):
+    assert P._binding.selftest_bounded_wait(polls) == 2
