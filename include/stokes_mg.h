@@ -222,7 +222,9 @@ int stokes_fgmres_batched(stokes_mg_t h, const double* b_dev, double* x_dev, int
  * arrives on, gives up after `polls` polls and returns; then its lanes wait
  * with different numbers of polls and have to come to one outcome.
  * *result = 2 then (1 would mean that a wait succeeded, 3 that the lanes
- * disagree, 0 that the kernel never ran).  Errors: EINVAL, ECUDA. */
+ * disagree, 0 that the kernel never ran).  With polls = 0 the patch GEMM too
+ * runs once with waits that give up at once, which it has to report, and once
+ * as usual (4 and 5 where one of these goes wrong).  Errors: EINVAL, ECUDA. */
 int stokes_selftest_bounded_wait(long long polls, int* result);
 
 /* Measurement utility (no counterpart in the paper): the FP64 pipe's peak on

@@ -5,6 +5,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <climits>
 #include <cstdint>
 #include <stdexcept>
 #include <string>
@@ -292,8 +293,9 @@ __global__ void __launch_bounds__(512, 1) k_patch_gemm(int npatch, const int* __
 //                    warp w % 4) -> Yb.
 // Two accumulators alternate between patches when they fit in the 512
 // tensor-memory columns, so the epilogue of one patch overlaps the MMAs of
-// the next.  All mbarrier waits are bounded; on a timeout the CTA records it
-// in *status, stops every role and returns.
+// the next.  All mbarrier waits are bounded; on a timeout the CTA stops every
+// role, records it in *status, waits (bounded) for its copies and MMAs in flight
+// and returns.
 namespace tc {
 
 constexpr int KS = 16;                    // inverse columns per stage: two K = 8 steps
@@ -309,7 +311,6 @@ __host__ __device__ inline int meta_bytes(int nlist, int grid) {
     const int k = (nlist + grid - 1) / grid;
     return (12 * (k < META_MAX ? k : META_MAX) + 15) & ~15;
 }
-constexpr long long WAIT_LIMIT = 1ll << 22;
 
 __host__ __device__ constexpr int np_of(int m) { return m < 16 ? 16 : m; }
 __host__ __device__ inline int tiles_of(int n) { return (n + 127) >> 7; }
@@ -387,9 +388,8 @@ __device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
 }
 // bounded wait; false (and the CTA's abort flag set) after `limit` polls,
 // or at once if another role has already given up
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int* abort_flag,
-                                          long long limit = WAIT_LIMIT) {
-    for (long long i = 0; i < limit; ++i) {
+__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int* abort_flag, int limit) {
+    for (int i = 0; i < limit; ++i) {
         if (mbar_try(a, parity)) return true;
         if (*abort_flag) return false;
     }
@@ -401,8 +401,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile 
 // polls for itself, so at a timeout some may see the phase complete and others
 // the abort flag, and those that went on would wait in elect.sync, __syncwarp or
 // tcgen05.ld for the ones that left
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t a, uint32_t parity, volatile int* abort_flag,
-                                               long long limit = WAIT_LIMIT) {
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t a, uint32_t parity, volatile int* abort_flag, int limit) {
     return __all_sync(0xffffffffu, mbar_wait(a, parity, abort_flag, limit));
 }
 
@@ -411,7 +410,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t a, uint32_t parity, vola
 // with no polls at all, so that they differ on their own.  *result = 2 when both
 // waits give up for all lanes alike and the kernel returns (1 would mean a
 // completed phase, 3 lanes that disagree)
-__global__ void k_wait_probe(long long limit, int* result) {
+__global__ void k_wait_probe(int limit, int* result) {
     __shared__ __align__(8) unsigned long long bar[2];
     __shared__ int abort_flag[2];
     const uint32_t a = smem_u32(bar), b = smem_u32(bar + 1);
@@ -473,7 +472,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
                                                                         const int* __restrict__ pdofs,
                                                                         const CUtensorMap* __restrict__ tmaps,
                                                                         const float* __restrict__ X,
-                                                                        float* __restrict__ Yb, int* status) {
+                                                                        float* __restrict__ Yb, int* status, int limit) {
     constexpr int NP = np_of(M);
     extern __shared__ __align__(1024) unsigned char smem_tc[];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -482,6 +481,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
     const uint32_t full0 = base, empty0 = base + 8 * ST, accf0 = base + 16 * ST, acce0 = accf0 + 16;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem_tc + 16 * ST + 32);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(smem_tc + 16 * ST + 36);
+    const uint32_t drain0 = base + 16 * ST + 40;              // the MMAs' end after a timeout
     const uint32_t raw0 = base + 16 * ST + 48;                // SPLIT: the TMA's barriers
     int* meta = reinterpret_cast<int*>(smem_tc + HDR);        // [kpatch][3]
     const int sbytes = stage_bytes(maxn, NP, SPLIT);
@@ -529,6 +529,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
             mbar_init(accf0 + 8 * b, 1);           // MMA commit of a patch's last stage
             mbar_init(acce0 + 8 * b, 4);           // epilogue warps
         }
+        mbar_init(drain0, 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -537,19 +538,19 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
     fence_after();
     const uint32_t tmem = *tmem_slot;
 
+    const uint32_t bar0 = SPLIT ? raw0 : full0;    // the copies complete on it
+    int issued = 0;                                // thread 0: stages whose copies were issued
     if (warp == 0) {
         // ---------------------------------------------------------- TMA ---
         if (lane == 0) {
-            const uint32_t bar0 = SPLIT ? raw0 : full0;
-            int it = 0;
             for (int k = 0; k < kpatch; ++k) {
                 int p, s0, n;
                 item(k, p, s0, n);
                 const int tiles = tiles_of(n), nst = (n + KS - 1) / KS;
                 const CUtensorMap* tm = tmaps + p;
-                for (int j = 0; j < nst; ++j, ++it) {
-                    const int s = it % ST;
-                    if (it >= ST && !mbar_wait(empty0 + 8 * s, ((it / ST) - 1) & 1, abort_flag)) goto done;
+                for (int j = 0; j < nst; ++j, ++issued) {
+                    const int s = issued % ST;
+                    if (issued >= ST && !mbar_wait(empty0 + 8 * s, ((issued / ST) - 1) & 1, abort_flag, limit)) goto done;
                     const uint32_t st = stage0 + (uint32_t)(s * sbytes);
                     mbar_expect_tx(bar0 + 8 * s, (uint32_t)(tiles * A_TILE));
                     for (int mt = 0; mt < tiles; ++mt) tma_load_2d(st + mt * A_TILE, tm, bar0 + 8 * s, j * KS, mt * 128);
@@ -571,11 +572,11 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
             item(pc, p, s0, n);
             const int tiles = tiles_of(n), nst = (n + KS - 1) / KS;
             const int b = pc % nbuf;
-            if (pc >= nbuf && !mbar_wait_warp(acce0 + 8 * b, ((pc / nbuf) - 1) & 1, abort_flag)) goto done;
+            if (pc >= nbuf && !mbar_wait_warp(acce0 + 8 * b, ((pc / nbuf) - 1) & 1, abort_flag, limit)) goto done;
             fence_after();
             const uint32_t acc = tmem + (uint32_t)(b * ccols);
             for (int j = 0; j < nst; ++j) {
-                if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag)) goto done;
+                if (!mbar_wait_warp(full0 + 8 * s, ph, abort_flag, limit)) goto done;
                 fence_after();
                 const uint32_t so = (uint32_t)(s * sbytes) >> 4;
                 const uint32_t lo = SPLIT ? (uint32_t)(ls * lo_bytes(maxn)) >> 4 : 0;
@@ -640,7 +641,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
                                        ? __ldg(reinterpret_cast<const float4*>(X + (long long)dof[k4] * M + c))
                                        : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
-                if (it >= ST && !mbar_wait_warp(empty0 + 8 * s, ((it / ST) - 1) & 1, abort_flag)) goto done;
+                if (it >= ST && !mbar_wait_warp(empty0 + 8 * s, ((it / ST) - 1) & 1, abort_flag, limit)) goto done;
                 unsigned char* bp = smem_tc + (stage0 - base) + (size_t)s * sbytes + b_off;
 #pragma unroll
                 for (int k4 = 0; k4 < KS / 4; ++k4) {
@@ -671,7 +672,7 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
             int p, s0, n;
             item(pc, p, s0, n);
             const int tiles = tiles_of(n), b = pc % nbuf;
-            if (!mbar_wait_warp(accf0 + 8 * b, (pc / nbuf) & 1, abort_flag)) goto done;
+            if (!mbar_wait_warp(accf0 + 8 * b, (pc / nbuf) & 1, abort_flag, limit)) goto done;
             fence_after();
 #pragma unroll
             for (int mt = 0; mt < 8; ++mt) {
@@ -711,8 +712,8 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
             for (int j = 0; j < nst; ++j, ++it) {
                 if (it % ng != grp) continue;
                 const int s = it % ST;
-                if (it >= lr && !mbar_wait_warp(empty0 + 8 * ((it - lr) % ST), ((it - lr) / ST) & 1, abort_flag)) goto done;
-                if (!mbar_wait_warp(raw0 + 8 * s, (it / ST) & 1, abort_flag)) goto done;
+                if (it >= lr && !mbar_wait_warp(empty0 + 8 * ((it - lr) % ST), ((it - lr) / ST) & 1, abort_flag, limit)) goto done;
+                if (!mbar_wait_warp(raw0 + 8 * s, (it / ST) & 1, abort_flag, limit)) goto done;
                 float4* hp = reinterpret_cast<float4*>(smem_tc + (stage0 - base) + (size_t)s * sbytes);
                 float4* lp = reinterpret_cast<float4*>(smem_tc + (lo0 - base) + (size_t)(it % lr) * lo_bytes(maxn));
 #pragma unroll 4
@@ -732,9 +733,29 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
         }
     }
 done:
-    if (tid == 0 && *abort_flag) atomicExch(status, 1);
+    __syncwarp();
     fence_before();
     __syncthreads();
+    if (*abort_flag) {
+        // every role has stopped (the flag is final only now: the TMA thread is
+        // through long before the last waits).  Shared and tensor memory go back
+        // once the copies and MMAs in flight are over, or after the limit again
+        // (the TF32 kernel's copies share a phase with a gather that may never
+        // have arrived).
+        auto settle = [&](uint32_t bar, uint32_t parity, int polls) {
+            while (polls > 0 && !mbar_try(bar, parity)) --polls;
+            return polls;
+        };
+        if (tid == 0) {
+            atomicExch(status, 1);
+            int left = (int)GEMM_WAIT_LIMIT;
+            for (int s = 0; s < ST && s < issued; ++s) left = settle(bar0 + 8 * s, ((issued - 1 - s) / ST) & 1, left);
+        } else if (warp == 1) {
+            commit(drain0);
+            settle(drain0, 0, (int)GEMM_WAIT_LIMIT);
+        }
+        __syncthreads();
+    }
     if (warp == 0) {
         fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");
@@ -912,19 +933,20 @@ static TcPlan tc_plan(int maxn, int m, int npatch, bool split = false) {
 
 template <int M, int ST, bool SPLIT>
 static void launch_tc(const TcPlan& pl, int nlist, const int* plist, int maxn, const int* poff, const int* pdofs,
-                      const void* tmaps, const float* X, float* Yb, int* status, cudaStream_t s) {
+                      const void* tmaps, const float* X, float* Yb, int* status, int limit, cudaStream_t s) {
     cudaFuncSetAttribute(tc::k_patch_gemm_tc<M, ST, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
     tc::k_patch_gemm_tc<M, ST, SPLIT><<<pl.grid, tc::threads_of(SPLIT), pl.smem, s>>>(
-        nlist, maxn, pl.lr, pl.gw, plist, poff, pdofs, reinterpret_cast<const CUtensorMap*>(tmaps), X, Yb, status);
+        nlist, maxn, pl.lr, pl.gw, plist, poff, pdofs, reinterpret_cast<const CUtensorMap*>(tmaps), X, Yb, status,
+        limit);
 }
 
 template <int M, bool SPLIT>
 static void launch_tc_st(int nlist, const int* plist, int maxn, const int* poff, const int* pdofs, const void* tmaps,
-                         const float* X, float* Yb, int* status, cudaStream_t s) {
+                         const float* X, float* Yb, int* status, int limit, cudaStream_t s) {
     const TcPlan pl = tc_plan(maxn, M, nlist, SPLIT);
     switch (pl.stages) {
 #define SBAT_TC_CASE(S) \
-    case S: launch_tc<M, S, SPLIT>(pl, nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, s); break;
+    case S: launch_tc<M, S, SPLIT>(pl, nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, limit, s); break;
         SBAT_TC_CASE(2) SBAT_TC_CASE(3) SBAT_TC_CASE(4) SBAT_TC_CASE(5) SBAT_TC_CASE(6) SBAT_TC_CASE(7)
         SBAT_TC_CASE(8) SBAT_TC_CASE(9) SBAT_TC_CASE(10) SBAT_TC_CASE(11) SBAT_TC_CASE(12)
 #undef SBAT_TC_CASE
@@ -935,12 +957,12 @@ static void launch_tc_st(int nlist, const int* plist, int maxn, const int* poff,
 template <int M>
 static void patch_gemm_m(int mode, int kind, int nw, int nlist, const int* plist, int maxn, const int* poff,
                          const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
-                         const float* X, float* Yb, int* status, cudaStream_t s) {
+                         const float* X, float* Yb, int* status, int limit, cudaStream_t s) {
     if (kind == GEMM_KIND_AUTO) kind = gemm_kind(mode, maxn);
     if (kind == GEMM_KIND_TC && mode == GEMM_3XTF32)
-        launch_tc_st<M, true>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, s);
+        launch_tc_st<M, true>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, limit, s);
     else if (kind == GEMM_KIND_TC)
-        launch_tc_st<M, false>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, s);
+        launch_tc_st<M, false>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, limit, s);
     else if (mode == GEMM_3XTF32)
         launch_gemm_st<M, GEMM_3XTF32>(maxn, nw, nlist, plist, poff, pdofs, ioff, inv, X, Yb, s);
     else
@@ -962,7 +984,7 @@ const char* patch_gemm_check(int mode, int maxn, int m) {
 }
 
 int wait_probe(long long polls, int* result_dev, cudaStream_t s) {
-    tc::k_wait_probe<<<1, 32, 0, s>>>(polls, result_dev);
+    tc::k_wait_probe<<<1, 32, 0, s>>>((int)std::min<long long>(polls, INT_MAX), result_dev);
     return (int)cudaGetLastError();
 }
 
@@ -1005,20 +1027,72 @@ void build_tmaps(int npatch, const int* poff_d, const long long* ioff_d, const f
 
 void patch_gemm(int mode, int kind, int nw, int nlist, const int* plist, int maxn, int m, const int* poff,
                 const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
-                const float* X, float* Yb, int* status, cudaStream_t s) {
+                const float* X, float* Yb, int* status, cudaStream_t s, int limit) {
     if (nlist <= 0) return;
     switch (m) {
 #define SBAT_M(MM) \
     case MM: \
         patch_gemm_m<MM>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, X, \
-                         Yb, status, s); \
+                         Yb, status, limit, s); \
         break;
         SBAT_M(8) SBAT_M(16) SBAT_M(32)
 #undef SBAT_M
         default:
             patch_gemm_m<64>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, X,
-                             Yb, status, s);
+                             Yb, status, limit, s);
     }
+}
+
+// identity "inverses" of several row tiles and more stages than the pipeline
+// has, integers as right-hand sides
+int gemm_timeout_probe(int mode, cudaStream_t s) {
+    constexpr int m = 16, np = 3;
+    const int size[np] = {300, 81, 140};
+    std::vector<int> off(1, 0), dofs;
+    std::vector<long long> at;
+    std::vector<float> inv, x;
+    for (int n : size) {
+        const int ld = (n + 3) & ~3;
+        at.push_back((long long)inv.size());
+        inv.resize(inv.size() + (size_t)ld * n, 0.f);
+        for (int a = 0; a < n; ++a) {
+            inv[at.back() + (size_t)a * ld + a] = 1.f;
+            dofs.push_back(off.back() + a);
+        }
+        off.push_back(off.back() + n);
+    }
+    for (size_t i = 0; i < dofs.size() * m; ++i) x.push_back((float)(i % 509) - 254.f);
+    std::vector<float> y(x.size(), 0.f);
+    int flag[2] = {0, 0};
+    std::vector<void*> mem;
+    cudaError_t e = cudaSuccess;
+    auto up = [&](const void* p, size_t bytes) {
+        void* d = nullptr;
+        if (e == cudaSuccess) e = cudaMalloc(&d, bytes);
+        if (e == cudaSuccess) mem.push_back(d);
+        if (e == cudaSuccess && p) e = cudaMemcpy(d, p, bytes, cudaMemcpyHostToDevice);
+        return d;
+    };
+    const int* poff = (const int*)up(off.data(), sizeof(int) * off.size());
+    const int* pdofs = (const int*)up(dofs.data(), sizeof(int) * dofs.size());
+    const long long* ioff = (const long long*)up(at.data(), sizeof(long long) * np);
+    const float* A = (const float*)up(inv.data(), sizeof(float) * inv.size());
+    const float* X = (const float*)up(x.data(), sizeof(float) * x.size());
+    float* Y = (float*)up(y.data(), sizeof(float) * y.size());
+    void* maps = up(nullptr, tmap_bytes(np));
+    int* status = (int*)up(flag, sizeof(flag));
+    if (e == cudaSuccess) {
+        build_tmaps(np, poff, ioff, A, maps);
+        patch_gemm(mode, GEMM_KIND_TC, 0, np, nullptr, 300, m, poff, pdofs, ioff, A, maps, X, Y, status, s, 0);
+        patch_gemm(mode, GEMM_KIND_TC, 0, np, nullptr, 300, m, poff, pdofs, ioff, A, maps, X, Y, status + 1, s);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e == cudaSuccess) e = cudaMemcpy(flag, status, sizeof(flag), cudaMemcpyDeviceToHost);
+    if (e == cudaSuccess) e = cudaMemcpy(y.data(), Y, sizeof(float) * y.size(), cudaMemcpyDeviceToHost);
+    for (void* d : mem) cudaFree(d);
+    if (e != cudaSuccess) throw std::runtime_error(cudaGetErrorString(e));
+    return flag[0] != 1 ? 4 : flag[1] != 0 || y != x ? 5 : 2;
 }
 
 void pull_scatter(int n, int m, const int* soff, const int* sidx, const float* wt, const float* Yb, float alpha,

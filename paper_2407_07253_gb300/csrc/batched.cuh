@@ -37,6 +37,12 @@ const char* patch_gemm_check(int mode, int maxn, int m);
 // whose lanes differ gives up for all of them, and the kernel returns); returns
 // the launch's cudaError_t
 int wait_probe(long long polls, int* result_dev, cudaStream_t s);
+// polls of one of its waits in the tensor-core patch GEMM
+constexpr int GEMM_WAIT_LIMIT = 1 << 22;
+// self-test of that GEMM at a timeout: a launch whose waits give up at once, then
+// one as usual; 2, or 4 if the first one reports no timeout, 5 if the second one
+// does or its product is wrong
+int gemm_timeout_probe(int mode, cudaStream_t s);
 
 // bytes of the per-patch tensor maps of a level, and their construction
 // (host encoding from the device offsets; synchronous)
@@ -63,7 +69,7 @@ int gemm_kind(int mode, int n);
 int gemm_default_warps(int maxn);
 void patch_gemm(int mode, int kind, int nw, int nlist, const int* plist, int maxn, int m, const int* poff,
                 const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
-                const float* X, float* Yb, int* status, cudaStream_t s);
+                const float* X, float* Yb, int* status, cudaStream_t s, int limit = GEMM_WAIT_LIMIT);
 
 // out[j * m + c] = alpha * wt[j] * sum_{q in slots(j)} Yb[sidx[q] * m + c] + beta * out[j * m + c]
 // (slots in increasing order: a fixed summation order; the partition-of-unity

@@ -3154,6 +3154,8 @@ int stokes_selftest_bounded_wait(long long polls, int* result) {
         CK(cudaDeviceSynchronize());
         CK(cudaMemcpy(result, d, sizeof(int), cudaMemcpyDeviceToHost));
         CK(cudaFree(d));
+        for (int mode : {STOKES_BATCH_TF32, STOKES_BATCH_3XTF32})
+            if (polls == 0 && *result == 2) *result = sbat::gemm_timeout_probe(mode, nullptr);
         return STOKES_OK;
     });
 }
