@@ -885,8 +885,11 @@ __device__ void saddle_core_factored(int d, int n, int nv, const double* K, cons
     const int ldl = (nv + vec - 1) / vec * vec;
     const int ldw = (dnv + vec - 1) / vec * vec;
     const int lds = (np + vec - 1) / vec * vec;
-    const long long lenL = saddle_factor_lenL(nv, vec, packed);
-    const long long oW = lenL, oS = oW + (long long)ldw * np;
+    // 32-bit offsets (a patch has at most a few thousand DoFs): 64-bit ones cost
+    // saddle_inverse_smem 62 registers instead of 48, and so its fifth CTA per SM
+    // (P4 64 x 64: 2.59 ms instead of 2.42, P3 128 x 128: 3.52 instead of 3.20)
+    const int lenL = (int)saddle_factor_lenL(nv, vec, packed);
+    const int oW = lenL, oS = oW + ldw * np;
     const int ns = np * (np + 1) / 2;
     if (K) {
         for (int i = warp; i < nv; i += nw)

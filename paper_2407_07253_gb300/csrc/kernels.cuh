@@ -332,9 +332,11 @@ __global__ void saddle_inverse_global(int npatch, int d, const int* __restrict__
 // listed patch's place in the scratch (saddle_tiles_scratch doubles).
 constexpr size_t SADDLE_TILES_SMEM_MAX = 226 * 1024;
 // Patches of max(nv, np) from here on are tiled even where the pivot-pair
-// kernel's shared memory would hold them: the P5 level (91 nodes) of the P8
-// hierarchy takes setup and solve from 50.2 to 48.4 ms; at 61 nodes (P4, where
-// the 4 x 4 inverses and the padding weigh more) it is 2.42 ms against 2.81.
+// kernel's shared memory would hold them.  At 91 nodes (P5 64 x 64) tiles take
+// 7.4 ms against 8.9; at 61 (P4 64 x 64, where the 4 x 4 inverses and the padding
+// weigh more) 2.94 against 2.42, at 37 (P3 128 x 128) 3.65 against 3.20.  The line
+// lies between; 3D P2 stars (65 nodes, one pressure) are on its slower side by
+// 10% (2.40 against 2.16 ms on 16^3).
 constexpr int SADDLE_TILES_MIN_N = 80;
 __host__ __device__ inline size_t saddle_tiles_smem(int d, int max4, int max_np, int max_n) {
     const size_t nt = (size_t)max4 * (max4 + 1) / 2;
