@@ -10,6 +10,7 @@ from paper_2407_07253_gb300 import build as B
 
 # kernel: threads per CTA, CTAs per SM
 WANT = {
+    "gj_inverse_global": (512, 4),      # all of an SM's threads
     "saddle_inverse_smem": (256, 5),    # the 41 KB of a P4 star leave room for five
 }
 
