@@ -98,15 +98,17 @@ void col_dots(int n, int m, int nb, const double* V, long long ldv, const double
 void col_update_dots(int n, int m, int nb, const double* V, long long ldv, const double* H, double* W, double* partial,
                      double* out, double* acc, cudaStream_t s);
 // Vout = (W - V H) / nu per column, hn[c] = nu = sqrt(H[nb][c] - sum_{i < nb} H[i][c]^2)
-// with H[nb][c] = |W_c|^2 (0 where nu == 0)
+// with H[nb][c] = |W_c|^2 (0 where nu == 0); hn[c] = -1 and Vout = W - V H where that
+// difference cancels, for col_givens to finish
 void col_normalise(int n, int m, int nb, const double* V, long long ldv, const double* H, const double* W, double* Vout,
                    double* hn, cudaStream_t s);
 // Vout = W / h[c] per column (0 where h[c] == 0)
 void col_scale(int n, int m, const double* W, const double* h, double* Vout, cudaStream_t s);
-// per column: Hessenberg column j, Givens rotations, g, |residual estimate|;
+// per column: the norm of the new basis vector Vn where col_normalise left it open,
+// Hessenberg column j, Givens rotations, g, |residual estimate|;
 // H [m][ldh][ldh], cs / sn [m][ldh], g [m][ldh + 1], hcol [nb][m], hn / resid [m]
-void col_givens(int j, int m, int ldh, double* H, const double* hcol, const double* hn, double* cs, double* sn,
-                double* g, double* resid, cudaStream_t s);
+void col_givens(int j, int m, int ldh, int n, double* Vn, double* H, const double* hcol, double* hn, double* cs,
+                double* sn, double* g, double* resid, cudaStream_t s);
 void col_backsolve(int jend, int m, int ldh, const double* H, const double* g, double* y, cudaStream_t s);
 // X[r][c] += sum_{j < jend} y[c][j] Z_j[r][c]; y [m][ldy]
 void col_xupdate(int n, int m, int jend, int ldy, const double* Z, long long ldz, const double* y, double* X,

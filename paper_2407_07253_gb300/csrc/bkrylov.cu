@@ -177,10 +177,13 @@ __global__ void __launch_bounds__(1024) k_col_reduce(int nblk, int m, const doub
     if (i < nacc) acc[i * m + c] += s;
 }
 
-// Vout = (W - V H) / nu, hn[c] = nu = sqrt(max(H[nb][c] - sum_i H[i][c]^2, 0))
-// (H[nb] = |W|^2 before the update; Pythagoras: the second pass's H is O(eps)
-// relative to W, so the difference loses no accuracy); 0 where nu = 0 (a
-// column already exact, or padding).
+// Vout = (W - V H) / nu, hn[c] = nu = sqrt(H[nb][c] - sum_i H[i][c]^2), with H[nb] =
+// |W|^2 before the update (Pythagoras); 0 where nu = 0 (padding, a zero column).
+// The second pass's H is O(eps) relative to the vector before the first one, so
+// the difference loses no accuracy unless that vector lay in the span to about
+// eps (a column whose Krylov space has closed while others go on).  Where it
+// cancels by more than a factor of four, Vout stays unscaled, hn[c] = -1, and
+// col_givens measures and scales the vector.
 __global__ void __launch_bounds__(256) k_col_normalise(int n, int m, int nb, const double* __restrict__ V, long long ldv,
                                                        const double* __restrict__ H, const double* __restrict__ W,
                                                        double* __restrict__ Vout, double* __restrict__ hn) {
@@ -190,9 +193,10 @@ __global__ void __launch_bounds__(256) k_col_normalise(int n, int m, int nb, con
     if (threadIdx.x < m) {
         double q = H[nb * m + threadIdx.x];
         for (int i = 0; i < nb; ++i) q = fma(-hs[i * m + threadIdx.x], hs[i * m + threadIdx.x], q);
-        const double nu = sqrt(q > 0.0 ? q : 0.0);
+        const bool exact = q >= 0.25 * H[nb * m + threadIdx.x];     // (false for NaN)
+        const double nu = exact ? sqrt(q) : 1.0;
         hs[nb * m + threadIdx.x] = nu > 0.0 ? 1.0 / nu : 0.0;
-        if (blockIdx.x == 0) hn[threadIdx.x] = nu;
+        if (blockIdx.x == 0) hn[threadIdx.x] = exact ? nu : -1.0;
     }
     __syncthreads();
     const int c = threadIdx.x % m;
@@ -222,20 +226,37 @@ __global__ void k_col_scale(long long nm, int m, const double* __restrict__ W, c
     }
 }
 
-// one column c per thread: append (hcol[.][c], hn[c]) as column j of the
-// column's Hessenberg matrix, apply the previous rotations, form the next,
-// update g and the residual estimate (the single-RHS fgmres_givens per column)
-__global__ void k_col_givens(int j, int m, int ldh, double* __restrict__ H, const double* __restrict__ hcol,
-                             const double* __restrict__ hn, double* __restrict__ cs, double* __restrict__ sn,
-                             double* __restrict__ g, double* __restrict__ resid) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= m) return;
+// one CTA per column c: scale its new basis vector where col_normalise left that
+// open (hn[c] < 0; rare, so one CTA's strided reads will do), then append
+// (hcol[.][c], hn[c]) as column j of the column's Hessenberg matrix, apply the
+// previous rotations, form the next, update g and the residual estimate (the
+// single-RHS fgmres_givens per column)
+__global__ void __launch_bounds__(256) k_col_givens(int j, int m, int ldh, int n, double* __restrict__ Vn,
+                                                    double* __restrict__ H, const double* __restrict__ hcol,
+                                                    double* __restrict__ hn, double* __restrict__ cs,
+                                                    double* __restrict__ sn, double* __restrict__ g,
+                                                    double* __restrict__ resid) {
+    __shared__ double red[256];
+    const int c = blockIdx.x;
+    double nu = hn[c];
+    if (nu < 0.0) {
+        double s = 0.0;
+        for (long long r = threadIdx.x; r < n; r += 256) s = fma(Vn[r * m + c], Vn[r * m + c], s);
+        red[threadIdx.x] = s;
+        __syncthreads();
+        s = 0.0;
+        for (int t = 0; t < 256; ++t) s += red[t];
+        nu = sqrt(s);
+        for (long long r = threadIdx.x; r < n; r += 256) Vn[r * m + c] = nu > 0.0 ? Vn[r * m + c] / nu : 0.0;
+    }
+    if (threadIdx.x > 0) return;
+    hn[c] = nu;
     double* Hc = H + (long long)c * ldh * ldh;
     double* csc = cs + (long long)c * ldh;
     double* snc = sn + (long long)c * ldh;
     double* gc = g + (long long)c * (ldh + 1);
     for (int i = 0; i <= j; ++i) Hc[i * ldh + j] = hcol[i * m + c];
-    Hc[(j + 1) * ldh + j] = hn[c];
+    Hc[(j + 1) * ldh + j] = nu;
     for (int i = 0; i < j; ++i) {
         const double a = Hc[i * ldh + j], b = Hc[(i + 1) * ldh + j];
         Hc[i * ldh + j] = csc[i] * a + snc[i] * b;
@@ -378,9 +399,9 @@ void col_scale(int n, int m, const double* W, const double* h, double* Vout, cud
     k_col_scale<<<grid_of(nm), 256, 0, s>>>(nm, m, W, h, Vout);
 }
 
-void col_givens(int j, int m, int ldh, double* H, const double* hcol, const double* hn, double* cs, double* sn,
-                double* g, double* resid, cudaStream_t s) {
-    k_col_givens<<<(m + 63) / 64, 64, 0, s>>>(j, m, ldh, H, hcol, hn, cs, sn, g, resid);
+void col_givens(int j, int m, int ldh, int n, double* Vn, double* H, const double* hcol, double* hn, double* cs,
+                double* sn, double* g, double* resid, cudaStream_t s) {
+    k_col_givens<<<m, 256, 0, s>>>(j, m, ldh, n, Vn, H, hcol, hn, cs, sn, g, resid);
 }
 
 void col_backsolve(int jend, int m, int ldh, const double* H, const double* g, double* y, cudaStream_t s) {

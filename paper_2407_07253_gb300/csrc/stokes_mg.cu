@@ -3005,7 +3005,9 @@ int fgmres_batched(stokes_mg* h, int nrhs, int mode, const double* B_dev, double
                 sbat::col_normalise(n, m, j + 1, K.V, nm, K.hcol2, K.W, K.V + (long long)(j + 1) * nm, K.hn, s);
             });
             h->launches += 2;              // the two reductions
-            launch(h, -1, s, [&] { sbat::col_givens(j, m, ldh, K.Hc, K.hcol, K.hn, K.cs, K.sn, K.g, K.resid, s); });
+            launch(h, -1, s, [&] {
+                sbat::col_givens(j, m, ldh, n, K.V + (long long)(j + 1) * nm, K.Hc, K.hcol, K.hn, K.cs, K.sn, K.g, K.resid, s);
+            });
             CK(cudaMemcpyAsync(K.host, K.resid, sizeof(double) * m, cudaMemcpyDeviceToHost, s));
             CK(cudaStreamSynchronize(s));
             res.assign(K.host, K.host + m);
