@@ -327,10 +327,15 @@ __global__ void saddle_inverse_global(int npatch, int d, const int* __restrict__
                                       int packed, long long max_scratch, const long long* __restrict__ soff,
                                       double* __restrict__ scratch, int* __restrict__ status);
 // The factored form of the listed patches from the CSR operator, on 4 x 4 tiles
-// in shared memory, one CTA of 512 or 256 threads per patch.  max4: the largest
+// in shared memory, one CTA of 512, 256 or 128 threads per patch.  max4: the largest
 // of nv and np in tiles of four; max_np, max_n: the largest np and n; soff: each
 // listed patch's place in the scratch (saddle_tiles_scratch doubles).
 constexpr size_t SADDLE_TILES_SMEM_MAX = 226 * 1024;
+// A launch's patches take at most this many doubles of scratch (4 GB): about three
+// times what is kept of a patch, so that a level with all its patches at once could
+// fill the memory that its operator and bases need.  Some 5500 patches of P8 and
+// 30,000 of P5 make one launch; a larger level pays a last wave per 40 waves.
+constexpr long long SADDLE_TILES_SCRATCH_MAX = 1LL << 29;
 // Patches of max(nv, np) from here on are tiled even where the pivot-pair
 // kernel's shared memory would hold them.  At 91 nodes (P5 64 x 64) tiles take
 // 7.4 ms against 8.9; at 61 (P4 64 x 64, where the 4 x 4 inverses and the padding

@@ -28,6 +28,7 @@
 #include "fem.hpp"
 #include "assembly.cuh"
 #include "kernels.cuh"
+#include "parts.hpp"
 #include "batched.cuh"
 
 namespace {
@@ -169,6 +170,7 @@ struct DevLevel {
     int* tl_list = nullptr;
     long long* tl_soff = nullptr;   // places in its scratch of tl_scratch doubles
     long long tl_scratch = 0;
+    std::vector<int> tl_first;      // parts of the list that share it (split_parts)
     long long ninv64 = 0, ninv32 = 0;
     double* inv64 = nullptr;            // explicit inverses (Gauss-Jordan patches; FP32 also for the batched path)
     float* inv32 = nullptr;
@@ -1573,7 +1575,7 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
         trace("patch lists uploaded", li, tt);
         // patches of the tiled inversion (factored form, all of a level's large ones or none)
         {
-            std::vector<long long> soff;
+            std::vector<long long> need, soff;
             std::vector<int> list;
             for (int p = 0; p < l.npatch; ++p) {
                 const int n = HL.patch_off[p + 1] - HL.patch_off[p], nv = HL.patch_nv[p], np = n - HL.d * nv;
@@ -1583,9 +1585,9 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
                 l.tl_np = std::max(l.tl_np, np);
                 l.tl_n = std::max(l.tl_n, n);
                 list.push_back(p);
-                soff.push_back(l.tl_scratch);
-                l.tl_scratch += skern::saddle_tiles_scratch(HL.d, n, nv);
+                need.push_back(skern::saddle_tiles_scratch(HL.d, n, nv));
             }
+            l.tl_scratch = split_parts(need, skern::SADDLE_TILES_SCRATCH_MAX, soff, l.tl_first);
             if (!list.empty() &&
                 skern::saddle_tiles_smem(HL.d, l.tl_max4, l.tl_np, l.tl_n) <= skern::SADDLE_TILES_SMEM_MAX) {
                 l.tl_count = (int)list.size();
@@ -2005,18 +2007,21 @@ bool fused_factor(const stokes_mg* h, const DevLevel& l) {
 }
 
 // the tiled inversion of a level's large patches (512 threads a CTA where the
-// tiles fill an SM's shared memory, 256 where two CTAs fit)
+// tiles fill an SM's shared memory, 256 where two CTAs fit, 128 where four do),
+// part by part through one scratch
 void launch_tiles(stokes_mg* h, DevLevel& l, double* f64, float* f32, int* status, cudaStream_t s) {
     const size_t smem = skern::saddle_tiles_smem(h->dim, l.tl_max4, l.tl_np, l.tl_n);
     const int nt = 2 * (smem + 2048) > 227 * 1024 ? 512 : 4 * (smem + 2048) > 227 * 1024 ? 256 : 128;
     auto kern = nt == 512 ? skern::saddle_inverse_tiles_512 : nt == 256 ? skern::saddle_inverse_tiles_256 : skern::saddle_inverse_tiles_128;
     CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)skern::SADDLE_TILES_SMEM_MAX));
     double* scr = palloc<double>(h->device, l.tl_scratch, s);
-    launch(h, PK_GJ, s, [&] {
-        kern<<<l.tl_count, nt, smem, s>>>(h->dim, l.tl_list, l.poff, l.pnv, l.foff64, f64, l.foff32, f32,
-                                                       l.fac_packed, l.pdofs, l.K.rp, l.K.ci, l.K.v64, l.tl_max4,
-                                                       l.tl_np, l.tl_soff, scr, status);
-    });
+    for (size_t k = 0; k + 1 < l.tl_first.size(); ++k) {
+        const int at = l.tl_first[k], count = l.tl_first[k + 1] - at;
+        launch(h, PK_GJ, s, [&] {
+            kern<<<count, nt, smem, s>>>(h->dim, l.tl_list + at, l.poff, l.pnv, l.foff64, f64, l.foff32, f32, l.fac_packed,
+                                         l.pdofs, l.K.rp, l.K.ci, l.K.v64, l.tl_max4, l.tl_np, l.tl_soff + at, scr, status);
+        });
+    }
     CK(cudaFreeAsync(scr, s));
 }
 
