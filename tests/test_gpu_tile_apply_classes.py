@@ -1,0 +1,63 @@
+"""The FP32 apply on tiles in its two widest classes (161 to 256 tiles, one a thread;
+257 to 512, two), which the stars of the structured meshes reach in 2D at P5 alone:
+cones over triangulated spheres and wheels of eight triangles put one vertex of
+high valence in the middle.  In 3D their partial sums lie behind the block instead
+of over it.
+
+Reference and tolerance as the other saddle applies: numpy's LU solves of the
+exported blocks, 2e-4 with FP32 factors."""
+import numpy as np
+import pytest
+from scipy.spatial import ConvexHull
+
+torch = pytest.importorskip("torch")
+P = pytest.importorskip("paper_2407_07253_gb300")
+
+pytestmark = pytest.mark.gpu
+
+
+def cone(n):
+    """Tetrahedra from the origin to the hull of n points spread over the sphere."""
+    i = np.arange(n) + 0.5
+    z, t = 1 - 2 * i / n, np.pi * (1 + 5**0.5) * i
+    s = np.sqrt(1 - z * z)
+    pts = np.stack([s * np.cos(t), s * np.sin(t), z], 1)
+    tri = ConvexHull(pts).simplices + 1
+    return np.vstack([np.zeros(3), pts]), np.hstack([np.zeros((len(tri), 1), int), tri]).astype(np.int32)
+
+
+def wheel(n):
+    t = 2 * np.pi * np.arange(n) / n
+    k = np.arange(n)
+    return (np.vstack([np.zeros(2), np.stack([np.cos(t), np.sin(t)], 1)]),
+            np.stack([0 * k, k + 1, (k + 1) % n + 1], 1).astype(np.int32))
+
+
+CASES = {
+    "3d_one": (cone(17), 2, [2], 160, 256),
+    "3d_two": (cone(24), 2, [2], 256, 512),
+    "2d_one": (wheel(8), 4, [4, 2], 160, 256),
+    "2d_two": (wheel(9), 4, [4, 2], 256, 512),
+}
+
+
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_apply_matches_patch_solves(name):
+    (v, c), k, sched, above, most = CASES[name]
+    h = P.StokesMG(v, c, 1, P.TH, k, hierarchy=P.HIER_EXPLICIT, schedule=sched, precision=P.MIXED, lmax_override=[1.0] * 8)
+    n = h.info()["n_free"][0]
+    off, dofs = h.patches(0)
+    _, comp, _ = h.level_dofs(0)
+    n4 = max(-(-int((comp[dofs[a:b]] == 0).sum()) // 4) for a, b in zip(off, off[1:]))
+    assert above < n4 * (n4 + 1) // 2 <= most
+    flat = h.patch_matrices(0)
+    r = np.random.default_rng(k).standard_normal(n)
+    want, mult, pos = np.zeros(n), np.bincount(dofs, minlength=n), 0
+    for a, b in zip(off, off[1:]):
+        d = dofs[a:b]
+        K = flat[pos:pos + len(d)**2].reshape(len(d), len(d))
+        pos += len(d)**2
+        want[d] += np.linalg.solve(K, r[d]) / mult[d]
+    z = h.asm(0, torch.tensor(r, device="cuda"), P.MIXED).cpu().numpy()
+    h.close()
+    assert np.abs(z - want).max() <= 2e-4 * np.abs(want).max()
