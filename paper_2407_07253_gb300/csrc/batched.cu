@@ -891,9 +891,9 @@ static void launch_gemm_st(int maxn, int nw, int nlist, const int* plist, const 
 }
 
 // Patches of <= TC_MIN_N DoFs fill under half of a 128-row MMA tile; the
-// warp-level kernel is faster there.  The 3xTF32 tensor-core kernel holds
-// twice the operands per stage; up to TC_SPLIT_MAX_N DoFs (6 row tiles) two
-// stages still fit.
+// warp-level kernel is faster there.  The 3xTF32 tensor-core kernel holds R's
+// lo part in every stage and two or more slots of the inverse's; up to
+// TC_SPLIT_MAX_N DoFs (6 row tiles) two stages still fit.
 constexpr int TC_MIN_N = 64, TC_SPLIT_MAX_N = 768;
 
 int gemm_kind(int mode, int n) {

@@ -259,8 +259,9 @@ void maxpy_mdot(int n, int m, const double* V, long long ldv, const double* h, d
 
 // Last update of classical Gram-Schmidt, normalised:
 //   w <- (w - V h) / nu,  nu = sqrt(max(nrm2 - sum_i h_i^2, 0)),  *hn = nu,
-// where nrm2 = ||w||^2 before the update (Pythagoras: the second pass's h is
-// O(eps) relative to w, so the difference loses no accuracy).
+// where nrm2 = ||w||^2 before the update (Pythagoras).  The second pass's h is
+// O(eps) relative to w before the first one, so the difference loses no accuracy
+// unless that w lay in the span to about eps: the Krylov space has closed then.
 __global__ void __launch_bounds__(256) maxpy_normalise(int n, int m, const double* __restrict__ V, long long ldv,
                                                        const double* __restrict__ h, const double* __restrict__ nrm2,
                                                        double* __restrict__ w, double* __restrict__ hn) {
@@ -1461,7 +1462,7 @@ SPD_TILES_KERNEL(512)
 // One ASM sweep.  The patch inverse is column-major with its leading
 // dimension padded to VEC rows; a thread owns VEC consecutive rows (one
 // 16-byte vector per column) and the columns are split among G groups of
-// row-owners (G = blockDim / row groups), each thread keeping 8 independent
+// row-owners (G = threads / row groups), each thread keeping 8 independent
 // 16-byte loads in flight.  The groups' partial sums are added in shared
 // memory in a fixed order.  The gathered residual of the patch sits in
 // shared memory.
@@ -1473,20 +1474,20 @@ __device__ __forceinline__ void patch_apply_body(int p, const int* __restrict__ 
     const int s = poff[p], n = poff[p + 1] - s;
     const int ldv = (n + VEC - 1) / VEC;
     // the map is constant: fetched before the wait for the kernel that wrote r
-    constexpr int PRE = 2;
+    constexpr int PRE = 2, NT = PATCH_APPLY_THREADS;
     int jd[PRE];
 #pragma unroll
-    for (int u = 0; u < PRE; ++u) jd[u] = (int)threadIdx.x + u * 128 < n ? __ldg(pdofs + s + threadIdx.x + u * 128) : -1;
+    for (int u = 0; u < PRE; ++u) jd[u] = (int)threadIdx.x + u * NT < n ? __ldg(pdofs + s + threadIdx.x + u * NT) : -1;
     pdl_wait();
     pdl_release();
 #pragma unroll
     for (int u = 0; u < PRE; ++u)
-        if (jd[u] >= 0) xs[threadIdx.x + u * 128] = r[jd[u]];
-    for (int a = threadIdx.x + PRE * 128; a < n; a += 128) xs[a] = r[pdofs[s + a]];
+        if (jd[u] >= 0) xs[threadIdx.x + u * NT] = r[jd[u]];
+    for (int a = threadIdx.x + PRE * NT; a < n; a += NT) xs[a] = r[pdofs[s + a]];
     __syncthreads();
-    const int G = ldv >= (int)blockDim.x ? 1 : (int)blockDim.x / ldv;
+    const int G = ldv >= NT ? 1 : NT / ldv;
     const V* base = reinterpret_cast<const V*>(inv + ioff[p]);
-    for (int t0 = 0; t0 < ldv; t0 += blockDim.x) {          // more row groups than threads: loop
+    for (int t0 = 0; t0 < ldv; t0 += NT) {          // more row groups than threads: loop
         const int t = threadIdx.x;
         const int rg = t0 + (G == 1 ? t : t % ldv), g = G == 1 ? 0 : t / ldv;
         T a0 = 0, a1 = 0, a2 = 0, a3 = 0;
@@ -1541,24 +1542,24 @@ __device__ __forceinline__ void patch_apply_body(int p, const int* __restrict__ 
     }
 }
 
-__global__ void __launch_bounds__(128) patch_apply_f32(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
+__global__ void __launch_bounds__(PATCH_APPLY_THREADS) patch_apply_f32(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                                        const long long* __restrict__ ioff, const float* __restrict__ inv,
                                                        const float* __restrict__ r, const float* __restrict__ wt,
                                                        float* __restrict__ Y, int n, long long nslot) {
     extern __shared__ __align__(16) unsigned char smem_pa[];
     float4* red = reinterpret_cast<float4*>(smem_pa);
-    float* xs = reinterpret_cast<float*>(smem_pa + sizeof(float4) * (blockDim.x + 4));
+    float* xs = reinterpret_cast<float*>(smem_pa + sizeof(float4) * (PATCH_APPLY_THREADS + 4));
     patch_apply_body<float, float4, 4>(blockIdx.x, poff, pdofs, ioff, inv, r + (long long)blockIdx.y * n, wt,
                                             Y + blockIdx.y * nslot, xs, red);
 }
 
-__global__ void __launch_bounds__(128) patch_apply_f64(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
+__global__ void __launch_bounds__(PATCH_APPLY_THREADS) patch_apply_f64(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                                        const long long* __restrict__ ioff, const double* __restrict__ inv,
                                                        const double* __restrict__ r, const double* __restrict__ wt,
                                                        double* __restrict__ Y, int n, long long nslot) {
     extern __shared__ __align__(16) unsigned char smem_pa[];
     double2* red = reinterpret_cast<double2*>(smem_pa);
-    double* xs = reinterpret_cast<double*>(smem_pa + sizeof(double2) * (blockDim.x + 4));
+    double* xs = reinterpret_cast<double*>(smem_pa + sizeof(double2) * (PATCH_APPLY_THREADS + 4));
     patch_apply_body<double, double2, 2>(blockIdx.x, poff, pdofs, ioff, inv, r + (long long)blockIdx.y * n, wt,
                                             Y + blockIdx.y * nslot, xs, red);
 }

@@ -363,7 +363,7 @@ __global__ void saddle_inverse_tiles_128(SADDLE_TILES_ARGS);
 #undef SADDLE_TILES_ARGS
 // Explicit inverses of SPD blocks of lo < n <= hi (work row-major, kept),
 // outputs and status as gj_inverse_*; spd_tiles_smem(min(hi, largest n)) bytes.
-// Up to SPD_TILES_SMALL_N six CTAs of 128 threads share an SM.
+// Up to SPD_TILES_SMALL_N four CTAs of 128 threads share an SM.
 constexpr int SPD_TILES_SMALL_N = 88, SPD_TILES_MAX_N = 220;
 __host__ __device__ inline size_t spd_tiles_smem(int n) {
     const size_t n4 = (n + 3) / 4, nt = n4 * (n4 + 1) / 2;
@@ -474,8 +474,9 @@ inline int saddle_tile_apply_threads(int n4, int npatch) {
 
 // One ASM sweep (Eq. 3.4): Y[poff[i] + a] = w[dof_a] * sum_b Kinv_i[a][b] r[dof_b].
 // FP32: float4 loads of 4 consecutive rows per thread; FP64: double2 loads
-// of 2 rows.  One CTA per patch and vector (blockIdx.y; vectors of n DoFs and
-// nslot slots); blockDim = round_up(ld / VEC, 32).
+// of 2 rows.  One CTA of PATCH_APPLY_THREADS per patch and vector (blockIdx.y;
+// vectors of n DoFs and nslot slots).
+constexpr int PATCH_APPLY_THREADS = 128;
 __global__ void patch_apply_f32(int npatch, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                 const long long* __restrict__ ioff, const float* __restrict__ inv,
                                 const float* __restrict__ r, const float* __restrict__ wt, float* __restrict__ Y, int n,

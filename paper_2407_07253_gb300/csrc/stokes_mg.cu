@@ -554,9 +554,12 @@ void spmv_lanes(stokes_mg* h, const DevCSR& A, const T* x, T* y, const T* b, cud
 }
 
 // Lanes per node of spmv_stokes: 8, which a small level's latency and long rows
-// want (64 x 64 P4 23.6 us against 25.5 with 4 and 30.8 with 2; 3D P3 16^3, 77
-// entries a row, 56 against 62), 4 where rows of up to 64 entries make so many
-// groups that issue counts (256 x 256 P4, 1.7 M groups: 199 us against 219).
+// want (P4 64 x 64, 0.1 M groups, 24.0 us against 25.1 with 4; 3D P3 16^3, 77 entries
+// a row, 56 against 62), 4 where rows of up to 64 entries make so many groups that
+// issue counts (P4 256 x 256, 1.6 M groups: 199 us against 219; 3D P2 64^3, 2.3 M:
+// 401 against 465).  They break even at 0.4 M groups of 42 entries (P4 128 x 128);
+// between there and the line, 8 lanes cost 4 to 10% (P4 160 x 160 92 us against
+// 88) and keep sums half as long.
 constexpr int kStokesFewLanesFrom = 1 << 20;
 
 template <int MODE, int D>
@@ -695,10 +698,10 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
     } else {
         const T* inv = PO::inv(l);
         if (!inv) throw StokesError(STOKES_EINVAL, PO::none);
-        const size_t smem = PO::red * (128 + 4) + sizeof(T) * l.maxn;
+        const size_t smem = PO::red * (skern::PATCH_APPLY_THREADS + 4) + sizeof(T) * l.maxn;
         launch(h, PK_PATCH, s, [&] {
-            kl(h, PO::expl, dim3(l.npatch, h->nvec), 128, smem, s, l.npatch, poff, pdofs, PO::ioff(l), inv, r, wt, Y, l.n,
-               l.nent);
+            kl(h, PO::expl, dim3(l.npatch, h->nvec), skern::PATCH_APPLY_THREADS, smem, s, l.npatch, poff, pdofs, PO::ioff(l),
+               inv, r, wt, Y, l.n, l.nent);
         });
     }
     const int *soff = l.soff, *sidx = l.sidx;
