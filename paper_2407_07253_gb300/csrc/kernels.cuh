@@ -491,7 +491,12 @@ __global__ void patch_apply_f64(int npatch, const int* __restrict__ poff, const 
 // bookkeeping: xmode PULL_X_SET also sets x[j] = out[j], PULL_X_ADD adds
 // x[j] += out[j]; with rdst != NULL, rdst[j] = bsrc[j].
 enum PullX { PULL_X_NONE = 0, PULL_X_SET = 1, PULL_X_ADD = 2 };
-template <typename T, bool MV>
+// PRE = 8 slots at a time cover every DoF of a structured mesh at once, but cost
+// 48 registers in FP64 (32 in FP32): levels beyond one wave of such CTAs take 4
+// there (256 x 256 P4 73 -> 57 us, 128 x 128 P4 23 -> 19), smaller ones, where the chain
+// of loads counts, 8 (one V-cycle of P2 8 x 8 50.5 us against 51.2).
+constexpr int PULL_WIDE_MAX_64 = 152 * 5 * 256;
+template <typename T, bool MV, int PRE>
 __global__ void __launch_bounds__(256) pull_scatter(int n, const int* __restrict__ soff, const int* __restrict__ sidx,
                                                     const T* __restrict__ Y, T alpha, T beta, T* __restrict__ out,
                                                     T* __restrict__ x, int xmode, const T* __restrict__ bsrc,
@@ -505,9 +510,10 @@ __global__ void __launch_bounds__(256) pull_scatter(int n, const int* __restrict
             rdst += (long long)blockIdx.y * n;
         }
     }
-    // the map is constant: the first DoF's slots (eight at most) and weight are
-    // fetched before the wait for the kernel that wrote Y
-    constexpr int PRE = 8;
+    // the map is constant: the first DoF's slots (PRE at most) are fetched before
+    // the wait for the kernel that wrote Y; the others one by one in the wide FP64
+    // form, whose small levels hardly have any (a loop around them costs it 3 us a
+    // V-cycle of P2 8 x 8), else PRE at a time
     int j = blockIdx.x * blockDim.x + threadIdx.x;
     int q = 0, e = 0, idx[PRE];
     if (j < n) {
@@ -519,14 +525,28 @@ __global__ void __launch_bounds__(256) pull_scatter(int n, const int* __restrict
     pdl_wait();
     pdl_release();
     for (; j < n;) {
-        T y[PRE], s = 0;
+        T s = 0;
+        auto slots = [&] {
+            T y[PRE];
 #pragma unroll
-        for (int u = 0; u < PRE; ++u)
-            if (q + u < e) y[u] = Y[idx[u]];
+            for (int u = 0; u < PRE; ++u)
+                if (q + u < e) y[u] = Y[idx[u]];
 #pragma unroll
-        for (int u = 0; u < PRE; ++u)
-            if (q + u < e) s += y[u];
-        for (int k = q + PRE; k < e; ++k) s += Y[__ldg(sidx + k)];
+            for (int u = 0; u < PRE; ++u)
+                if (q + u < e) s += y[u];
+        };
+        if constexpr (sizeof(T) == 8 && PRE == 8) {
+            slots();
+            for (int k = q + PRE; k < e; ++k) s += Y[__ldg(sidx + k)];
+        } else {
+            for (;;) {
+                slots();
+                q += PRE;
+                if (q >= e) break;
+#pragma unroll
+                for (int u = 0; u < PRE; ++u) idx[u] = q + u < e ? __ldg(sidx + q + u) : 0;
+            }
+        }
         const T o = beta == T(0) ? alpha * s : alpha * s + beta * out[j];
         out[j] = o;
         if (xmode == PULL_X_SET) x[j] = o;

@@ -705,9 +705,12 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
         });
     }
     const int *soff = l.soff, *sidx = l.sidx;
+    const bool wide = sizeof(T) == 4 || (long long)l.n * h->nvec <= skern::PULL_WIDE_MAX_64;
+    const auto pull = h->nvec > 1 ? (wide ? skern::pull_scatter<T, true, 8> : skern::pull_scatter<T, true, 4>)
+                                  : (wide ? skern::pull_scatter<T, false, 8> : skern::pull_scatter<T, false, 4>);
     launch(h, PK_PULL, s, [&] {
-        kl(h, h->nvec > 1 ? skern::pull_scatter<T, true> : skern::pull_scatter<T, false>, dim3(grid_for(l.n), h->nvec), 256,
-           0, s, l.n, soff, sidx, (const T*)Y, (T)alpha, (T)beta, out, x, xmode, bsrc, rdst, l.nent);
+        kl(h, pull, dim3(grid_for(l.n), h->nvec), 256, 0, s, l.n, soff, sidx, (const T*)Y, (T)alpha, (T)beta, out, x, xmode,
+           bsrc, rdst, l.nent);
     });
 }
 
