@@ -553,23 +553,36 @@ void spmv_lanes(stokes_mg* h, const DevCSR& A, const T* x, T* y, const T* b, cud
     }
 }
 
-// Lanes per node of spmv_stokes: 8, which a small level's latency and long rows
-// want (P4 64 x 64, 0.1 M groups, 24.0 us against 25.1 with 4; 3D P3 16^3, 77 entries
-// a row, 56 against 62), 4 where rows of up to 64 entries make so many groups that
-// issue counts (P4 256 x 256, 1.6 M groups: 199 us against 219; 3D P2 64^3, 2.3 M:
-// 401 against 465).  They break even at 0.4 M groups of 42 entries (P4 128 x 128);
-// between there and the line, 8 lanes cost 4 to 10% (P4 160 x 160 92 us against
-// 88) and keep sums half as long.
+// Lanes per node of spmv_stokes.  Long rows on few nodes are a chain of rounds of
+// gathers, which more lanes shorten while the SMs have threads to spare.  With
+// g = groups / average entries of a row: 16 lanes up to g = 1600, 32 up to 800 /
+// components (us with 8, 16, 32 lanes: SV P4 disk, g = 343, 25.8, 18.1, 13.8; P4 16 x 16,
+// 159, 13.4, 11.4, 10.0; P6 disk, 399, 26.2, 18.9, 17.5; 3D P3 8^3, 238, 20.1, 16.6, 17.0;
+// P7 32 x 32, 970, 38.6, 33.4, 39.5; SV P4 disk refined, 1358, 27.3, 19.7, 22.8; 3D P3
+// 16^3, 1819, 56.2, 57.5, 75.5; P4 64 x 64, 2471, 23.6, 26.1, 38.3).  Rows of up to 20
+// entries (P2 in 2D) measured no better with more than 8.  4 where rows
+// of up to 64 entries make so many groups that issue counts (P4 256 x 256, 1.6 M
+// groups: 199 us against 219; 3D P2 64^3, 2.3 M: 401 against 465).  4 and 8 break even at
+// 0.4 M groups of 42 entries (P4 128 x 128); between there and the line, 8 lanes cost
+// 4 to 10% (P4 160 x 160 92 us against 88) and keep sums half as long.
 constexpr int kStokesFewLanesFrom = 1 << 20;
+
+int stokes_lanes(const DevCSR& A) {
+    const long long groups = A.nr - (long long)(A.dim - 1) * A.nvf;
+    if (groups >= kStokesFewLanesFrom && A.nnz <= 64LL * A.nr) return 4;
+    if (A.nnz <= 20LL * A.nr) return 8;
+    const double g = (double)groups * A.nr / A.nnz;
+    return g * A.dim <= 800 ? 32 : g <= 1600 ? 16 : 8;
+}
 
 template <int MODE, int D>
 void spmv_stokes_lanes(stokes_mg* h, const DevCSR& A, const float* x, float* y, const float* b, cudaStream_t s) {
-    const int nq = A.nr - D * A.nvf;
-    const bool few = A.nvf + nq >= kStokesFewLanesFrom && A.nnz <= 64LL * A.nr;
-    const int lanes = few ? 4 : 8, grid = (int)(((long long)(A.nvf + nq) * lanes + 255) / 256);
     if (A.nr == 0) return;
-    if (few) kl(h, skern::spmv_stokes<4, MODE, D>, grid, 256, 0, s, A.nvf, nq, A.rp, A.ci, A.v32, x, y, b);
-    else kl(h, skern::spmv_stokes<8, MODE, D>, grid, 256, 0, s, A.nvf, nq, A.rp, A.ci, A.v32, x, y, b);
+    const int nq = A.nr - D * A.nvf, lanes = stokes_lanes(A);
+    const int grid = (int)(((long long)(A.nvf + nq) * lanes + 255) / 256);
+    const auto kern = lanes == 4 ? skern::spmv_stokes<4, MODE, D> : lanes == 8 ? skern::spmv_stokes<8, MODE, D>
+                    : lanes == 16 ? skern::spmv_stokes<16, MODE, D> : skern::spmv_stokes<32, MODE, D>;
+    kl(h, kern, grid, 256, 0, s, A.nvf, nq, A.rp, A.ci, A.v32, x, y, b);
 }
 
 template <typename T>

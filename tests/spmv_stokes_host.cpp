@@ -99,6 +99,7 @@ int main() {
         for (int nq : {1, 6, 11}) {
             same &= check<8, 2>(nvf, nq, 70, &worst) & check<8, 3>(nvf, nq, 70, &worst);
             same &= check<4, 2>(nvf, nq, 40, &worst) & check<4, 3>(nvf, nq, 40, &worst);
+            same &= check<16, 2>(nvf, nq, 70, &worst) & check<32, 3>(nvf, nq, 70, &worst);
         }
     std::printf("%.3e\n", worst);
     return same ? 0 : 1;

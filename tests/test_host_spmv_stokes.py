@@ -1,6 +1,6 @@
 """spmv_stokes as a warp sees it, on the CPU (spmv_stokes_host.cpp): every lane
 of a warp that holds velocity nodes and pressure rows takes part in every
-full-mask shuffle, with 4 and 8 lanes per group, in 2D and 3D, and the rows'
+full-mask shuffle, with 4 to 32 lanes per group, in 2D and 3D, and the rows'
 sums agree with sums in double to 2^-24 times their length (at most 3 * 70
 products and the residual's own term)."""
 import os
