@@ -2165,6 +2165,15 @@ __device__ __forceinline__ void saddle_apply_bulk_body(
     for (int q = tid; q < np; q += NT) Y[s0 + dnv + q] = -wq[dnv + q] * sq[q];
 }
 
+__global__ void __launch_bounds__(SA_BULK_THREADS) saddle_apply_bulk_f32(
+    int d, const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
+    const long long* __restrict__ foff, const float* __restrict__ fac, const float* __restrict__ r,
+    const float* __restrict__ wt, float* __restrict__ Y, int buf_bytes, int xs_len, int* __restrict__ status) {
+    extern __shared__ __align__(128) unsigned char smem_sb[];
+    __shared__ __align__(8) unsigned long long bar;
+    saddle_apply_bulk_body<float>(d, poff, pdofs, pnv, foff, fac, r, wt, Y, buf_bytes, xs_len, status, smem_sb, &bar);
+}
+
 __global__ void __launch_bounds__(SA_BULK_THREADS) saddle_apply_bulk_f64(
     int d, const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,
     const long long* __restrict__ foff, const double* __restrict__ fac, const double* __restrict__ r,

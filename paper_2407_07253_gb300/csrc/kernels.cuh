@@ -379,9 +379,9 @@ __global__ void spd_inverse_tiles_512(SPD_TILES_ARGS);
 // Elements of one patch's factored inverse (Li, W, Si with leading
 // dimensions rounded up to vec = 2 (FP64) or 4 (FP32)).  Li's form, packed:
 // 0 column-major; 1 its upper triangle row by row (nv (nv + 1) / 2 entries,
-// rounded up to vec: the FP64 bulk-copy apply); 2 the 4 x 4 tiles of its upper
+// rounded up to vec: the row-wise bulk-copy apply); 2 the 4 x 4 tiles of its upper
 // triangle, zero padded, 16-byte group r ntile + t holding row r of tile t (the
-// FP32 bulk-copy apply).
+// FP32 apply on tiles).
 __host__ __device__ inline long long saddle_factor_lenL(int nv, int vec, int packed) {
     const long long n4 = (nv + 3) / 4;
     if (packed == 2) return 8 * n4 * (n4 + 1);
@@ -430,6 +430,11 @@ constexpr long long SA_WAIT_LIMIT = 1ll << 22;
 __host__ __device__ inline size_t saddle_apply_bulk_smem(int buf_bytes, int elem_bytes, int xs_len) {
     return (size_t)buf_bytes + (size_t)elem_bytes * 5 * xs_len;
 }
+__global__ void saddle_apply_bulk_f32(int d, const int* __restrict__ poff, const int* __restrict__ pdofs,
+                                      const int* __restrict__ pnv, const long long* __restrict__ foff,
+                                      const float* __restrict__ fac, const float* __restrict__ r,
+                                      const float* __restrict__ wt, float* __restrict__ Y, int buf_bytes,
+                                      int xs_len, int* __restrict__ status);
 __global__ void saddle_apply_bulk_f64(int d, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                       const int* __restrict__ pnv, const long long* __restrict__ foff,
                                       const double* __restrict__ fac, const double* __restrict__ r,
@@ -470,6 +475,20 @@ inline int saddle_tile_apply_threads(int n4, int npatch) {
     const int t = n4 * (n4 + 1) / 2;
     if (t <= 64) return t <= 32 && npatch >= SADDLE_TILE_APPLY_WARP_MIN ? 32 : 64;
     return t <= 128 ? 128 : t <= 160 ? 160 : t <= SADDLE_TILE_APPLY_MAX ? 256 : 0;
+}
+// Levels that keep the row-wise bulk-copy apply in FP32: one pressure per patch (P2),
+// a largest patch, which sets threads and shared memory for all, with far more tiles
+// than most, and enough patches for the SMs' places to count.  Mean over largest 0.23: the P2 level
+// of SV on the refined disk (5671 patches, 91 tiles) 18.1 us against 22.3, 3D P2 with one
+// star of 115 nodes (4505) 38.7 against 57.8; 0.33: 3D P2, 95 nodes (2465) 24.7 against
+// 28.6; 0.39 (2057 patches) 22.5 on both sides; 0.47: P4 around a vertex of nine cells 52.5
+// against 44.5 on tiles.  With 1438 patches or fewer there is no such loss (0.22: 11.4
+// against 11.7 us; 669 patches, 0.23: 17.8 against 16.7), and with many pressures the
+// tiles' products with W outweigh it (SV P3, up to 73 nodes, 3137 patches: 84 against 55).
+constexpr int SADDLE_TILE_UNEVEN_FROM = 152 * 8;
+inline bool saddle_tile_uneven(long long sum_tiles, int n4, int max_np, int npatch) {
+    const int t = n4 * (n4 + 1) / 2;
+    return max_np <= 1 && t > 64 && npatch > SADDLE_TILE_UNEVEN_FROM && 5 * sum_tiles < 2LL * t * npatch;
 }
 
 // One ASM sweep (Eq. 3.4): Y[poff[i] + a] = w[dof_a] * sum_b Kinv_i[a][b] r[dof_b].

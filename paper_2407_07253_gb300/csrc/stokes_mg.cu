@@ -661,6 +661,7 @@ template <> struct PatchOf<float> {
                 return dim == 3 ? skern::saddle_tile_apply_3d_256_1 : skern::saddle_tile_apply_2d_256_1;
         }
     }
+    static constexpr auto bulk = skern::saddle_apply_bulk_f32;
     static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f32_3d : skern::saddle_apply_f32_2d; }
     static constexpr auto expl = skern::patch_apply_f32;
     static constexpr size_t red = sizeof(float4);
@@ -673,6 +674,7 @@ template <> struct PatchOf<double> {
     static const long long* ioff(const DevLevel& l) { return l.ioff64; }
     static const double* wt(const DevLevel& l) { return l.wt64; }
     static double* Y(const DevLevel& l) { return l.Y64; }
+    static constexpr auto bulk = skern::saddle_apply_bulk_f64;
     static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f64_3d : skern::saddle_apply_f64_2d; }
     static constexpr auto expl = skern::patch_apply_f64;
     static constexpr size_t red = sizeof(double2);
@@ -694,13 +696,14 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
     if (fac && l.sa_buf > 0) {
         launch(h, PK_PATCH, s, [&] {
             if constexpr (sizeof(T) == 4)
-                kl(h, PO::tiles(h->dim, l.sa_n4, l.npatch), l.npatch, skern::saddle_tile_apply_threads(l.sa_n4, l.npatch),
-                   skern::saddle_tile_apply_smem(l.sa_buf, h->dim, l.sa_xs), s, poff, pdofs, pnv, foff, fac, r, wt, Y,
-                   (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
-            else
-                kl(h, skern::saddle_apply_bulk_f64, l.npatch, skern::SA_BULK_THREADS,
-                   skern::saddle_apply_bulk_smem(l.sa_buf, sizeof(T), l.sa_xs), s, h->dim, poff, pdofs, pnv, foff, fac, r,
-                   wt, Y, (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
+                if (l.fac_packed == 2) {
+                    kl(h, PO::tiles(h->dim, l.sa_n4, l.npatch), l.npatch, skern::saddle_tile_apply_threads(l.sa_n4, l.npatch),
+                       skern::saddle_tile_apply_smem(l.sa_buf, h->dim, l.sa_xs), s, poff, pdofs, pnv, foff, fac, r, wt, Y,
+                       (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
+                    return;
+                }
+            kl(h, PO::bulk, l.npatch, skern::SA_BULK_THREADS, skern::saddle_apply_bulk_smem(l.sa_buf, sizeof(T), l.sa_xs), s,
+               h->dim, poff, pdofs, pnv, foff, fac, r, wt, Y, (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
         });
     } else if (fac) {
         const size_t smem = skern::saddle_apply_smem(sizeof(T), h->dim, l.sa_xs);
@@ -1679,33 +1682,49 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
             };
             opt_in(PatchOf<float>::fact(HL.d));
             opt_in(PatchOf<double>::fact(HL.d));
-            opt_in(skern::saddle_apply_bulk_f64);
-            // the bulk-copy apply, with L^-1 stored as its upper triangle (FP32:
-            // in 4 x 4 tiles, at most SADDLE_TILE_APPLY_MAX), when the level's largest
-            // block fits in shared memory with room for at least two CTAs per SM
+            opt_in(PatchOf<float>::bulk);
+            opt_in(PatchOf<double>::bulk);
+            // the bulk-copy applies, with L^-1 stored as its upper triangle, when the
+            // level's largest block fits in shared memory with room for at least two
+            // CTAs per SM.  FP32: in 4 x 4 tiles, at most SADDLE_TILE_APPLY_MAX, or row
+            // by row where such a level's patches are too uneven for them.
             {
-                const int eb = want32 ? 4 : 8, vec = 16 / eb, packed = want32 ? 2 : 1;
-                long long mb = 0;
-                int n4 = 0;
-                std::vector<long long> fp(l.npatch + 1, 0);
+                const int eb = want32 ? 4 : 8;
+                long long sum_tiles = 0, buf = 0;
+                int n4 = 0, max_np = 0;
                 for (int p = 0; p < l.npatch; ++p) {
-                    const long long len = skern::saddle_factor_len(HL.d, HL.patch_off[p + 1] - HL.patch_off[p],
-                                                                   HL.patch_nv[p], vec, packed);
-                    fp[p + 1] = fp[p] + len;
-                    mb = std::max(mb, len);
-                    n4 = std::max(n4, (HL.patch_nv[p] + 3) / 4);
+                    max_np = std::max(max_np, HL.patch_off[p + 1] - HL.patch_off[p] - HL.d * HL.patch_nv[p]);
+                    const long long t = (HL.patch_nv[p] + 3) / 4;
+                    sum_tiles += t * (t + 1) / 2;
+                    n4 = std::max(n4, (int)t);
                 }
-                const bool tiles = skern::saddle_tile_apply_threads(n4, l.npatch) > 0;
-                long long buf = (mb * eb + 127) & ~127LL;
-                if (want32 && HL.d == 3) buf += (skern::tile_part_bytes(3, std::min(n4, 64)) + 127) & ~127;
-                buf = std::min<long long>(buf, 1 << 30);
-                const size_t smem = want32 ? skern::saddle_tile_apply_smem((int)buf, HL.d, l.sa_xs)
-                                           : skern::saddle_apply_bulk_smem((int)buf, eb, l.sa_xs);
-                if (mb > 0 && smem <= skern::SADDLE_APPLY_SMEM_MAX / 2 && (!want32 || tiles) &&
-                    !std::getenv("STOKES_NO_BULK_APPLY")) {
+                std::vector<long long> fp(l.npatch + 1, 0);
+                auto fits = [&](int packed) {
+                    long long mb = 0;
+                    for (int p = 0; p < l.npatch; ++p) {
+                        const long long len = skern::saddle_factor_len(HL.d, HL.patch_off[p + 1] - HL.patch_off[p],
+                                                                       HL.patch_nv[p], 16 / eb, packed);
+                        fp[p + 1] = fp[p] + len;
+                        mb = std::max(mb, len);
+                    }
+                    buf = (mb * eb + 127) & ~127LL;
+                    if (packed == 2 && HL.d == 3) buf += (skern::tile_part_bytes(3, std::min(n4, 64)) + 127) & ~127;
+                    buf = std::min<long long>(buf, 1 << 30);
+                    const size_t smem = packed == 2 ? skern::saddle_tile_apply_smem((int)buf, HL.d, l.sa_xs)
+                                                    : skern::saddle_apply_bulk_smem((int)buf, eb, l.sa_xs);
+                    return mb > 0 && smem <= skern::SADDLE_APPLY_SMEM_MAX / 2;
+                };
+                int packed = 0;
+                if (std::getenv("STOKES_NO_BULK_APPLY")) {
+                } else if (!want32) {
+                    packed = fits(1) ? 1 : 0;
+                } else if (skern::saddle_tile_apply_threads(n4, l.npatch) > 0 && fits(2)) {
+                    packed = skern::saddle_tile_uneven(sum_tiles, n4, max_np, l.npatch) && fits(1) ? 1 : 2;
+                }
+                if (packed) {
                     l.sa_buf = (int)buf;
                     l.sa_n4 = n4;
-                    if (want32)
+                    if (packed == 2)
                         CK(cudaFuncSetAttribute(PatchOf<float>::tiles(HL.d, n4, l.npatch), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                 (int)skern::SADDLE_APPLY_SMEM_MAX));
                     l.fac_packed = packed;

@@ -12,6 +12,8 @@ import numpy as np
 import pytest
 from scipy.spatial import ConvexHull
 
+import workloads as W
+
 torch = pytest.importorskip("torch")
 P = pytest.importorskip("paper_2407_07253_gb300")
 
@@ -76,3 +78,29 @@ def test_apply_matches_patch_solves(name):
 def test_streamed_apply_matches_patch_solves(name, precision, monkeypatch):
     monkeypatch.setenv("STOKES_NO_BULK_APPLY", "1")
     check(name, precision)
+
+
+@pytest.mark.parametrize("precision", [P.FP64, P.MIXED])
+@pytest.mark.parametrize("name", ["sv_p2_level", "3d"])
+def test_uneven_levels(name, precision, monkeypatch):
+    """Over 1216 patches, most of them far smaller than the largest: the row-wise
+    bulk-copy apply, in FP32 too, against the streamed one (the same factors, rounded
+    the same; the sums of up to 3 * 95 terms in another order)."""
+    (v, c), nref, fam, k, sched, level = {"sv_p2_level": (W.delaunay_disk_mesh(0, h=0.16), 1, P.SV, 3, [3, 2], 1),
+                                          "3d": (cone(13), 3, P.TH, 2, [2], 0)}[name]
+    z = []
+    for stream in (False, True):
+        if stream:
+            monkeypatch.setenv("STOKES_NO_BULK_APPLY", "1")
+        h = P.StokesMG(v, c, nref, fam, k, barycentric=fam == P.SV, hierarchy=P.HIER_EXPLICIT, schedule=sched,
+                       precision=precision, lmax_override=[1.0] * 8)
+        off, dofs = h.patches(level)
+        _, comp, _ = h.level_dofs(level)
+        n4 = np.array([-(-int((comp[dofs[a:b]] == 0).sum()) // 4) for a, b in zip(off, off[1:])])
+        t = n4 * (n4 + 1) // 2
+        assert len(t) > 1216 and t.mean() < 0.4 * t.max() and t.max() > 64
+        r = np.random.default_rng(3).standard_normal(len(comp))
+        z.append(h.asm(level, torch.tensor(r, device="cuda"), precision).cpu().numpy())
+        h.close()
+    eps = 2.0**-24 if precision == P.MIXED else 2.0**-53
+    assert np.abs(z[0] - z[1]).max() <= 600 * eps * np.abs(z[1]).max()
