@@ -1567,7 +1567,7 @@ __global__ void __launch_bounds__(PATCH_APPLY_THREADS) patch_apply_f64(int npatc
 // One ASM sweep with factored saddle inverses (saddle_core's factored form):
 //   t = r_p - W^T r_u,  s = Si t,  z_u = blockdiag(Li) r_u + W s,  z_p = -s,
 //   Y[poff[i] + a] = w[dof_a] z_a.
-// One CTA of SADDLE_APPLY_THREADS threads per patch.  Only vectors live in
+// One CTA of 128 or 256 threads per patch (saddle_apply_threads).  Only vectors live in
 // shared memory; Li, W and Si stream from global memory into registers, so
 // that seven CTAs share an SM and one's loads cover the others' barriers and
 // dependent loads.  Staging W in shared memory, to read it once, left one to
@@ -1575,8 +1575,8 @@ __global__ void __launch_bounds__(PATCH_APPLY_THREADS) patch_apply_f64(int npatc
 // square (1089 patches; bound by the FP64 pipe at 116 us), 176 against 135 us on
 // 3D P3 16^3 (3.9 TB/s), 155 against 130 us on P8 (5.4 TB/s: there W, 220 KB a
 // patch, comes from DRAM both times), 184 against 131 us on the SV P4 disk.
-// Fewer, larger CTAs (256 or 512 threads), 64 threads, and a bulk prefetch of
-// the block into L2 were each measured no faster.
+// On such levels fewer, larger CTAs (256 or 512 threads), 64 threads, and a bulk
+// prefetch of the block into L2 were each measured no faster; small ones take 256.
 template <typename T, int D> struct ColVec;              // x of one column, all components
 template <> struct __align__(4) ColVec<float, 1> { float v[1]; };
 template <> struct __align__(8) ColVec<float, 2> { float v[2]; };
@@ -1611,10 +1611,10 @@ __device__ __forceinline__ Vec16<T> load16(const Vec16<T>* p) {
 // groups' sums are added in red in a fixed order and handed to
 // out(row group, acc) by the first group.  Ends with every read of red done
 // by its reader only: the caller separates two calls by a barrier.
-template <bool ONCE, typename T, int D, typename F>
+template <bool ONCE, typename T, int D, int NT, typename F>
 __device__ __forceinline__ void columns_times(const T* __restrict__ M, int ld, int ncol, const ColVec<T, D>* x,
                                               Vec16<T>* red, F&& out) {
-    constexpr int NT = SADDLE_APPLY_THREADS, VEC = Vec16<T>::N, U = 8;
+    constexpr int VEC = Vec16<T>::N, U = 8;
     const int tid = threadIdx.x, ldv = ld / VEC;
     // no more groups than columns: the others' zeros would only lengthen the sum
     // over the groups, in series (3D P2 stars have one pressure: 127 additions; with
@@ -1678,13 +1678,13 @@ __device__ __forceinline__ void columns_times(const T* __restrict__ M, int ld, i
     }
 }
 
-template <typename T, int D>
+template <typename T, int D, int NT>
 __device__ __forceinline__ void saddle_apply_body(int p, const int* __restrict__ poff, const int* __restrict__ pdofs,
                                                   const int* __restrict__ pnv, const long long* __restrict__ foff,
                                                   const T* __restrict__ fac, const T* __restrict__ r,
                                                   const T* __restrict__ wt, T* __restrict__ Y, int xs_len,
                                                   unsigned char* smem) {
-    constexpr int NT = SADDLE_APPLY_THREADS, VEC = Vec16<T>::N;
+    constexpr int VEC = Vec16<T>::N;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int s0 = poff[p], n = poff[p + 1] - s0, nv = pnv[p], dnv = D * nv, np = n - dnv;
     if (n == 0) return;
@@ -1756,7 +1756,7 @@ __device__ __forceinline__ void saddle_apply_body(int p, const int* __restrict__
     }
     __syncthreads();
     // y_c = Li r_c for every component
-    columns_times<true, T, D>(Li, ldl, nv, xi, red, [&](int rg, const T (&acc)[D][VEC]) {
+    columns_times<true, T, D, NT>(Li, ldl, nv, xi, red, [&](int rg, const T (&acc)[D][VEC]) {
 #pragma unroll
         for (int c = 0; c < D; ++c)
 #pragma unroll
@@ -1765,14 +1765,14 @@ __device__ __forceinline__ void saddle_apply_body(int p, const int* __restrict__
     });
     __syncthreads();
     // s = Si t (Si symmetric)
-    columns_times<true, T, 1>(Sg, lds, np, reinterpret_cast<const ColVec<T, 1>*>(tq), red, [&](int rg, const T (&acc)[1][VEC]) {
+    columns_times<true, T, 1, NT>(Sg, lds, np, reinterpret_cast<const ColVec<T, 1>*>(tq), red, [&](int rg, const T (&acc)[1][VEC]) {
 #pragma unroll
         for (int e = 0; e < VEC; ++e)
             if (VEC * rg + e < np) sq[VEC * rg + e] = acc[0][e];
     });
     __syncthreads();
     // z_u = y + W s, z_p = -s, weighted
-    columns_times<false, T, 1>(Wg, ldw, np, reinterpret_cast<const ColVec<T, 1>*>(sq), red, [&](int rg, const T (&acc)[1][VEC]) {
+    columns_times<false, T, 1, NT>(Wg, ldw, np, reinterpret_cast<const ColVec<T, 1>*>(sq), red, [&](int rg, const T (&acc)[1][VEC]) {
 #pragma unroll
         for (int e = 0; e < VEC; ++e) {
             const int a = VEC * rg + e;
@@ -1782,20 +1782,24 @@ __device__ __forceinline__ void saddle_apply_body(int p, const int* __restrict__
     for (int q = tid; q < np; q += NT) Y[s0 + dnv + q] = -wt[pdofs[s0 + dnv + q]] * sq[q];
 }
 
-// seven CTAs per SM (at most 72 registers): left to itself the compiler takes
-// 77, six CTAs, and the 3D P3 apply takes 160 us instead of 135
-#define SADDLE_APPLY_KERNEL(NAME, T, D)                                                                             \
-    __global__ void __launch_bounds__(SADDLE_APPLY_THREADS, 7) NAME(                                                \
+// seven CTAs of 128 threads per SM (at most 72 registers): left to itself the
+// compiler takes 77, six CTAs, and the 3D P3 apply takes 160 us instead of 135
+#define SADDLE_APPLY_KERNEL(NAME, T, D, NT)                                                                         \
+    __global__ void __launch_bounds__(NT, NT == 128 ? 7 : 3) NAME##_##NT(                                           \
         const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,                   \
         const long long* __restrict__ foff, const T* __restrict__ fac, const T* __restrict__ r,                     \
         const T* __restrict__ wt, T* __restrict__ Y, int xs_len) {                                                  \
         extern __shared__ __align__(16) unsigned char smem_sa[];                                                    \
-        saddle_apply_body<T, D>(blockIdx.x, poff, pdofs, pnv, foff, fac, r, wt, Y, xs_len, smem_sa);                \
+        saddle_apply_body<T, D, NT>(blockIdx.x, poff, pdofs, pnv, foff, fac, r, wt, Y, xs_len, smem_sa);            \
     }
-SADDLE_APPLY_KERNEL(saddle_apply_f32_2d, float, 2)
-SADDLE_APPLY_KERNEL(saddle_apply_f32_3d, float, 3)
-SADDLE_APPLY_KERNEL(saddle_apply_f64_2d, double, 2)
-SADDLE_APPLY_KERNEL(saddle_apply_f64_3d, double, 3)
+SADDLE_APPLY_KERNEL(saddle_apply_f32_2d, float, 2, 128)
+SADDLE_APPLY_KERNEL(saddle_apply_f32_3d, float, 3, 128)
+SADDLE_APPLY_KERNEL(saddle_apply_f64_2d, double, 2, 128)
+SADDLE_APPLY_KERNEL(saddle_apply_f64_3d, double, 3, 128)
+SADDLE_APPLY_KERNEL(saddle_apply_f32_2d, float, 2, 256)
+SADDLE_APPLY_KERNEL(saddle_apply_f32_3d, float, 3, 256)
+SADDLE_APPLY_KERNEL(saddle_apply_f64_2d, double, 2, 256)
+SADDLE_APPLY_KERNEL(saddle_apply_f64_3d, double, 3, 256)
 #undef SADDLE_APPLY_KERNEL
 
 // ---- the same sweep with each patch's factored block brought into shared

@@ -393,34 +393,38 @@ __host__ __device__ inline long long saddle_factor_len(int d, int n, int nv, int
     return saddle_factor_lenL(nv, vec, packed) + ldw * np + lds * np;
 }
 // One ASM sweep with the factored inverses streamed from global memory, one
-// CTA per patch, D = 2 or 3 components; xs_len >= the largest patch.  Shared
+// CTA of 128 or 256 threads per patch, D = 2 or 3 components; xs_len >= the largest patch.  Shared
 // memory (bytes): the groups' partial sums and the patch's vectors (the
 // residual in two orders, y, t and s).  A level whose largest patch needs more
 // than SADDLE_APPLY_SMEM_MAX (the kernels' shared-memory attribute) by
 // saddle_apply_limit is refused.
-constexpr int SADDLE_APPLY_THREADS = 128;
 constexpr size_t SADDLE_APPLY_SMEM_MAX = 200 * 1024;
-__host__ __device__ inline size_t saddle_apply_smem(int elem_bytes, int d, long long xs_len) {
+__host__ __device__ inline size_t saddle_apply_smem(int elem_bytes, int d, long long xs_len, int threads) {
     const long long xl = (xs_len + 3) & ~3LL;
-    return (size_t)16 * SADDLE_APPLY_THREADS * d + (size_t)elem_bytes * ((d == 3 ? 4 : d) * ((xl / d + 4) & ~3LL) + 3 * xl + 4);
+    return (size_t)16 * threads * d + (size_t)elem_bytes * ((d == 3 ? 4 : d) * ((xl / d + 4) & ~3LL) + 3 * xl + 4);
 }
 __host__ __device__ inline size_t saddle_apply_limit(long long xs_len) { return (size_t)(6144 + 40 * xs_len); }
-__global__ void saddle_apply_f32_2d(const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                    const float* __restrict__ fac, const float* __restrict__ r, const float* __restrict__ wt,
-                                    float* __restrict__ Y, int xs_len);
-__global__ void saddle_apply_f32_3d(const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                    const float* __restrict__ fac, const float* __restrict__ r, const float* __restrict__ wt,
-                                    float* __restrict__ Y, int xs_len);
-__global__ void saddle_apply_f64_2d(const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                    const double* __restrict__ fac, const double* __restrict__ r, const double* __restrict__ wt,
-                                    double* __restrict__ Y, int xs_len);
-__global__ void saddle_apply_f64_3d(const int* __restrict__ poff, const int* __restrict__ pdofs,
-                                    const int* __restrict__ pnv, const long long* __restrict__ foff,
-                                    const double* __restrict__ fac, const double* __restrict__ r, const double* __restrict__ wt,
-                                    double* __restrict__ Y, int xs_len);
+// Threads per patch: 256 while all patches fit in about one wave of the CTAs of 128
+// (seven per SM), where a patch's own chain is what takes the time (FP32, 3D P3, 369
+// patches 32.5 us against 71; SV P4, 370, 32.5 against 55.6; P8 16 x 16, 289, 45 against 71;
+// P8 32 x 32, 1089, 130 against 143; FP64 P6 16 x 16, 289, 53 against 59).  Beyond it the
+// smaller CTAs cover each other's barriers better (3D P3 16^3, 4913, 144 against 170; SV P3
+// disk, 1438, 32.6 against 38.9; FP64 P5 stars, 1089, 90 against 117).  In FP32, with half as
+// many row groups a patch, the line is eight per SM.
+inline int saddle_apply_threads(int elem_bytes, int npatch) { return npatch <= 152 * (elem_bytes == 4 ? 8 : 7) ? 256 : 128; }
+#define SADDLE_APPLY_DECL(T, NAME)                                                                                     \
+    __global__ void NAME(const int* __restrict__ poff, const int* __restrict__ pdofs, const int* __restrict__ pnv,     \
+                         const long long* __restrict__ foff, const T* __restrict__ fac, const T* __restrict__ r,       \
+                         const T* __restrict__ wt, T* __restrict__ Y, int xs_len);
+SADDLE_APPLY_DECL(float, saddle_apply_f32_2d_128)
+SADDLE_APPLY_DECL(float, saddle_apply_f32_3d_128)
+SADDLE_APPLY_DECL(double, saddle_apply_f64_2d_128)
+SADDLE_APPLY_DECL(double, saddle_apply_f64_3d_128)
+SADDLE_APPLY_DECL(float, saddle_apply_f32_2d_256)
+SADDLE_APPLY_DECL(float, saddle_apply_f32_3d_256)
+SADDLE_APPLY_DECL(double, saddle_apply_f64_2d_256)
+SADDLE_APPLY_DECL(double, saddle_apply_f64_3d_256)
+#undef SADDLE_APPLY_DECL
 // The same sweep with one CTA per patch whose factored block is brought into
 // shared memory by one bulk copy (buf_bytes >= the largest block, a
 // multiple of 128; xs_len >= the largest patch).  *status = 1 if a CTA gave

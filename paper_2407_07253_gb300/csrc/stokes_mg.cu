@@ -662,7 +662,10 @@ template <> struct PatchOf<float> {
         }
     }
     static constexpr auto bulk = skern::saddle_apply_bulk_f32;
-    static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f32_3d : skern::saddle_apply_f32_2d; }
+    static auto fact(int dim, int threads) {
+        if (threads == 256) return dim == 3 ? skern::saddle_apply_f32_3d_256 : skern::saddle_apply_f32_2d_256;
+        return dim == 3 ? skern::saddle_apply_f32_3d_128 : skern::saddle_apply_f32_2d_128;
+    }
     static constexpr auto expl = skern::patch_apply_f32;
     static constexpr size_t red = sizeof(float4);
     static constexpr const char* none = "no FP32 patch inverses on this handle (FP64 handle)";
@@ -675,7 +678,10 @@ template <> struct PatchOf<double> {
     static const double* wt(const DevLevel& l) { return l.wt64; }
     static double* Y(const DevLevel& l) { return l.Y64; }
     static constexpr auto bulk = skern::saddle_apply_bulk_f64;
-    static auto fact(int dim) { return dim == 3 ? skern::saddle_apply_f64_3d : skern::saddle_apply_f64_2d; }
+    static auto fact(int dim, int threads) {
+        if (threads == 256) return dim == 3 ? skern::saddle_apply_f64_3d_256 : skern::saddle_apply_f64_2d_256;
+        return dim == 3 ? skern::saddle_apply_f64_3d_128 : skern::saddle_apply_f64_2d_128;
+    }
     static constexpr auto expl = skern::patch_apply_f64;
     static constexpr size_t red = sizeof(double2);
     static constexpr const char* none = "no FP64 patch inverses on this handle (MIXED handle)";
@@ -706,9 +712,10 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
                h->dim, poff, pdofs, pnv, foff, fac, r, wt, Y, (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
         });
     } else if (fac) {
-        const size_t smem = skern::saddle_apply_smem(sizeof(T), h->dim, l.sa_xs);
+        const int nt = skern::saddle_apply_threads(sizeof(T), l.npatch);
+        const size_t smem = skern::saddle_apply_smem(sizeof(T), h->dim, l.sa_xs, nt);
         launch(h, PK_PATCH, s, [&] {
-            kl(h, PO::fact(h->dim), l.npatch, skern::SADDLE_APPLY_THREADS, smem, s, poff, pdofs, pnv, foff, fac, r, wt, Y,
+            kl(h, PO::fact(h->dim, nt), l.npatch, nt, smem, s, poff, pdofs, pnv, foff, fac, r, wt, Y,
                (int)l.sa_xs);
         });
     } else {
@@ -1680,8 +1687,10 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
                 CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         (int)skern::SADDLE_APPLY_SMEM_MAX));
             };
-            opt_in(PatchOf<float>::fact(HL.d));
-            opt_in(PatchOf<double>::fact(HL.d));
+            for (int nt : {128, 256}) {
+                opt_in(PatchOf<float>::fact(HL.d, nt));
+                opt_in(PatchOf<double>::fact(HL.d, nt));
+            }
             opt_in(PatchOf<float>::bulk);
             opt_in(PatchOf<double>::bulk);
             // the bulk-copy applies, with L^-1 stored as its upper triangle, when the
