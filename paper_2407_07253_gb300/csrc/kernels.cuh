@@ -343,6 +343,14 @@ constexpr long long SADDLE_TILES_SCRATCH_MAX = 1LL << 29;
 // lies between; 3D P2 stars (65 nodes, one pressure) are on its slower side by
 // 10% (2.40 against 2.16 ms on 16^3).
 constexpr int SADDLE_TILES_MIN_N = 80;
+// and from this many on, unless the level's larger ones need the tiles anyway: they
+// are a launch of their own behind the others', whose time a small level pays on top
+// (P5 16 x 16 0.74 ms on pivot pairs, 0.45 + 0.59 with tiles; 28 x 28 1.93, 0.46 + 1.77; 32 x 32
+// with 961 stars 2.57, 0.46 + 2.18, its setup 5.50 and 5.90; 64 x 64 8.9, 0.49 + 7.4; P4 on the
+// disk, a few stars of 81 nodes among 1943, 1.50, 1.37 + 0.27).  Below another level,
+// beside whose inversion it runs, half as many: under P8 32 x 32 the 961 P5 stars are
+// better on tiles (setup 31.4 ms against 33.1).
+constexpr int SADDLE_TILES_MIN_COUNT = 152 * 8, SADDLE_TILES_MIN_BELOW = 152 * 4;
 __host__ __device__ inline size_t saddle_tiles_smem(int d, int max4, int max_np, int max_n) {
     const size_t nt = (size_t)max4 * (max4 + 1) / 2;
     return nt * (128 + 4) + sizeof(double) * (32 * (size_t)max4 + 32) + sizeof(int) * ((size_t)max_np * (d + 1) + max_n);

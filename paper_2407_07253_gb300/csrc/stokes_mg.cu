@@ -1606,10 +1606,22 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
         {
             std::vector<long long> need, soff;
             std::vector<int> list;
+            int large = 0, medium = 0;
+            auto size_class = [&](int p) {
+                const int n = HL.patch_off[p + 1] - HL.patch_off[p], nv = HL.patch_nv[p];
+                return skern::saddle_scratch(HL.d, n, nv) > skern::SADDLE_SMEM_MAX_DOUBLES ? 2
+                       : std::max(nv, n - HL.d * nv) >= skern::SADDLE_TILES_MIN_N          ? 1
+                                                                                           : 0;
+            };
+            for (int p = 0; p < l.npatch; ++p) {
+                const int c = size_class(p);
+                large += c == 2;
+                medium += c == 1;
+            }
+            const int from = large > 0 || medium >= (li > 0 ? skern::SADDLE_TILES_MIN_BELOW : skern::SADDLE_TILES_MIN_COUNT) ? 1 : 2;
             for (int p = 0; p < l.npatch; ++p) {
                 const int n = HL.patch_off[p + 1] - HL.patch_off[p], nv = HL.patch_nv[p], np = n - HL.d * nv;
-                if (skern::saddle_scratch(HL.d, n, nv) <= skern::SADDLE_SMEM_MAX_DOUBLES && std::max(nv, np) < skern::SADDLE_TILES_MIN_N)
-                    continue;
+                if (size_class(p) < from) continue;
                 l.tl_max4 = std::max(l.tl_max4, (std::max(nv, np) + 3) / 4);
                 l.tl_np = std::max(l.tl_np, np);
                 l.tl_n = std::max(l.tl_n, n);
@@ -1620,7 +1632,7 @@ void upload_level_patches(stokes_mg* h, int li, bool want32, cudaStream_t s) {
             if (!list.empty() &&
                 skern::saddle_tiles_smem(HL.d, l.tl_max4, l.tl_np, l.tl_n) <= skern::SADDLE_TILES_SMEM_MAX) {
                 l.tl_count = (int)list.size();
-                l.tl_min = skern::SADDLE_TILES_MIN_N;
+                if (from == 1) l.tl_min = skern::SADDLE_TILES_MIN_N;
                 l.tl_list = hupload(h, list, s);
                 l.tl_soff = hupload(h, soff, s);
             }
@@ -2054,16 +2066,21 @@ bool fused_factor(const stokes_mg* h, const DevLevel& l) {
 }
 
 // the tiled inversion of a level's large patches (512 threads a CTA where the
-// tiles fill an SM's shared memory, 256 where two CTAs fit, 128 where four do),
-// part by part through one scratch
+// tiles fill an SM's shared memory, 256 where two CTAs fit, 128 where four do, and
+// more where there are fewer patches than that: 225 stars of P5 0.70 ms with 128
+// threads, 0.59 with 256, 49 of them 0.60 and with 512 0.35), part by part through one
+// scratch
 void launch_tiles(stokes_mg* h, DevLevel& l, double* f64, float* f32, int* status, cudaStream_t s) {
     const size_t smem = skern::saddle_tiles_smem(h->dim, l.tl_max4, l.tl_np, l.tl_n);
-    const int nt = 2 * (smem + 2048) > 227 * 1024 ? 512 : 4 * (smem + 2048) > 227 * 1024 ? 256 : 128;
-    auto kern = nt == 512 ? skern::saddle_inverse_tiles_512 : nt == 256 ? skern::saddle_inverse_tiles_256 : skern::saddle_inverse_tiles_128;
-    CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)skern::SADDLE_TILES_SMEM_MAX));
+    const int nt_smem = 2 * (smem + 2048) > 227 * 1024 ? 512 : 4 * (smem + 2048) > 227 * 1024 ? 256 : 128;
     double* scr = palloc<double>(h->device, l.tl_scratch, s);
     for (size_t k = 0; k + 1 < l.tl_first.size(); ++k) {
         const int at = l.tl_first[k], count = l.tl_first[k + 1] - at;
+        const int nt = std::max(nt_smem, count <= 152 ? 512 : count <= 304 ? 256 : 128);
+        auto kern = nt == 512   ? skern::saddle_inverse_tiles_512
+                    : nt == 256 ? skern::saddle_inverse_tiles_256
+                                : skern::saddle_inverse_tiles_128;
+        CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)skern::SADDLE_TILES_SMEM_MAX));
         launch(h, PK_GJ, s, [&] {
             kern<<<count, nt, smem, s>>>(h->dim, l.tl_list + at, l.poff, l.pnv, l.foff64, f64, l.foff32, f32, l.fac_packed,
                                          l.pdofs, l.K.rp, l.K.ci, l.K.v64, l.tl_max4, l.tl_np, l.tl_soff + at, scr, status);
