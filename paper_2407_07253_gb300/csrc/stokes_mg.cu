@@ -852,27 +852,6 @@ void vcycle_body(stokes_mg* h, int prec, cudaStream_t s, bool pdl = true) {
     h->pdl_chain = h->pdl_armed = false;
 }
 
-// vout = B_MG vin for nvec vectors (1 or nvec_max), by the graph if there is one
-void vcycle_run(stokes_mg* h, int prec, cudaStream_t s, int nvec = 1) {
-    // per-launch events cannot sit inside a replayed graph: profiling any
-    // V-cycle kernel class runs the V-cycle as plain launches
-    const bool any_prof = h->prof[PK_PATCH].on || h->prof[PK_SPMV].on || h->prof[PK_PULL].on || h->prof[PK_TRANSFER].on;
-    const cudaGraphExec_t g = nvec > 1 ? h->vgraph : h->graph[prec];
-    if (g && !any_prof) {
-        CK(cudaGraphLaunch(g, s));
-        h->launches += nvec > 1 ? h->vgraph_launches : h->graph_launches[prec];
-    } else {
-        h->nvec = nvec;
-        try {
-            vcycle_body(h, prec, s, !any_prof);
-        } catch (...) {
-            h->nvec = 1;
-            throw;
-        }
-        h->nvec = 1;
-    }
-}
-
 void capture_graph(stokes_mg* h, int prec, int nvec, cudaGraphExec_t* out, long long* n_launches) {
     cudaStream_t cs;
     CK(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
@@ -899,6 +878,34 @@ void capture_graph(stokes_mg* h, int prec, int nvec, cudaGraphExec_t* out, long 
     CK(cudaGraphInstantiate(out, g, 0));
     CK(cudaGraphDestroy(g));
     CK(cudaStreamDestroy(cs));
+}
+
+// vout = B_MG vin for nvec vectors (1 or nvec_max), by the graph if there is one.
+// An FBF handle's setup captures the graph that its solves use; the one of a single
+// vector follows on the first call (not into a capture of the caller's).
+void vcycle_run(stokes_mg* h, int prec, cudaStream_t s, int nvec = 1) {
+    // per-launch events cannot sit inside a replayed graph: profiling any
+    // V-cycle kernel class runs the V-cycle as plain launches
+    const bool any_prof = h->prof[PK_PATCH].on || h->prof[PK_SPMV].on || h->prof[PK_PULL].on || h->prof[PK_TRANSFER].on;
+    if (nvec == 1 && h->nvec_max > 1 && !h->graph[prec] && h->opts.use_graph && !any_prof) {
+        cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(s, &st));
+        if (st == cudaStreamCaptureStatusNone) capture_graph(h, prec, 1, &h->graph[prec], &h->graph_launches[prec]);
+    }
+    const cudaGraphExec_t g = nvec > 1 ? h->vgraph : h->graph[prec];
+    if (g && !any_prof) {
+        CK(cudaGraphLaunch(g, s));
+        h->launches += nvec > 1 ? h->vgraph_launches : h->graph_launches[prec];
+    } else {
+        h->nvec = nvec;
+        try {
+            vcycle_body(h, prec, s, !any_prof);
+        } catch (...) {
+            h->nvec = 1;
+            throw;
+        }
+        h->nvec = 1;
+    }
 }
 
 // ---- batched V-cycle (m interleaved right-hand sides, FP32 operators) -----
@@ -2925,8 +2932,8 @@ int setup_impl(const stokes_mesh* coarse, int n_refine, int barycentric_finest, 
         h->st.t_eig_ms = host_ms() - t1;
         t1 = host_ms();
         if (o.use_graph) {
-            capture_graph(h.get(), o.precision, 1, &h->graph[o.precision], &h->graph_launches[o.precision]);
             if (h->nvec_max > 1) capture_graph(h.get(), o.precision, h->nvec_max, &h->vgraph, &h->vgraph_launches);
+            else capture_graph(h.get(), o.precision, 1, &h->graph[o.precision], &h->graph_launches[o.precision]);
         }
         h->st.t_graph_ms = host_ms() - t1;
         h->st.t_total_ms = host_ms() - t0;
