@@ -143,6 +143,7 @@ inline int grid_for(long long n, int block = 256) {
 struct DevCSR {
     int nr = 0, nc = 0;
     int dim = 0, nvf = 0;      // a Stokes operator in the device assembly's order (spmv_stokes): velocity nodes per component
+    bool by_size = true;       // spmv_stokes: lanes by the level's size (stokes_lanes); false: as a large level
     long long nnz = 0;
     int lanes = 16;
     int *rp = nullptr, *ci = nullptr;
@@ -570,7 +571,7 @@ constexpr int kStokesFewLanesFrom = 1 << 20;
 int stokes_lanes(const DevCSR& A) {
     const long long groups = A.nr - (long long)(A.dim - 1) * A.nvf;
     if (groups >= kStokesFewLanesFrom && A.nnz <= 64LL * A.nr) return 4;
-    if (A.nnz <= 20LL * A.nr) return 8;
+    if (A.nnz <= 20LL * A.nr || !A.by_size) return 8;
     const double g = (double)groups * A.nr / A.nnz;
     return g * A.dim <= 800 ? 32 : g <= 1600 ? 16 : 8;
 }
@@ -689,10 +690,12 @@ template <> struct PatchOf<double> {
 
 // one ASM sweep: Y = W_i K_i^{-1} I_i r for every patch, then
 // out = alpha * sum_i I_i^T Y_i + beta * out in the same pass as the
-// Chebyshev bookkeeping: x = out or x += out (xmode), rdst = bsrc (if rdst)
+// Chebyshev bookkeeping: x = out or x += out (xmode), rdst = bsrc (if rdst);
+// stream_threads: the streamed apply's threads per patch (0: by the level's size)
 template <typename T>
 void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, double beta, cudaStream_t s,
-               T* x = nullptr, int xmode = skern::PULL_X_NONE, const T* bsrc = nullptr, T* rdst = nullptr) {
+               T* x = nullptr, int xmode = skern::PULL_X_NONE, const T* bsrc = nullptr, T* rdst = nullptr,
+               int stream_threads = 0) {
     using PO = PatchOf<T>;
     const T* fac = PO::fac(l);
     const long long* foff = PO::foff(l);
@@ -712,7 +715,7 @@ void asm_apply(stokes_mg* h, DevLevel& l, const T* r, T* out, double alpha, doub
                h->dim, poff, pdofs, pnv, foff, fac, r, wt, Y, (int)l.sa_buf, (int)l.sa_xs, h->sa_status);
         });
     } else if (fac) {
-        const int nt = skern::saddle_apply_threads(sizeof(T), l.npatch);
+        const int nt = stream_threads ? stream_threads : skern::saddle_apply_threads(sizeof(T), l.npatch);
         const size_t smem = skern::saddle_apply_smem(sizeof(T), h->dim, l.sa_xs, nt);
         launch(h, PK_PATCH, s, [&] {
             kl(h, PO::fact(h->dim, nt), l.npatch, nt, smem, s, poff, pdofs, pnv, foff, fac, r, wt, Y,
@@ -1319,16 +1322,22 @@ int arnoldi_launch(stokes_mg* h, int li, const double* v0, int steps, double* Hs
     // the estimate serves (FP32 K and inverses in mixed mode); the basis and
     // its orthogonalisation stay FP64
     const bool f32 = h->opts.precision == STOKES_MIXED && (l.inv32 || l.fac32) && l.K.v32 && l.t32 && l.u32;
+    // A few steps leave the Ritz value unconverged, and at high degrees FP32 rounding
+    // then moves it by some 1e-6, and every cycle with it: the products keep one order
+    // of summation, whatever a level's size makes of the cycle's.
+    constexpr int threads = 128;
+    DevCSR K = l.K;
+    K.by_size = false;
     for (int j = 0; j < m; ++j) {
         double* w = V + (long long)(j + 1) * n;
         if (f32) {
             launch(h, -1, s, [&] { skern::convert_vec<float, double><<<grid_for(n), 256, 0, s>>>(n, V + (long long)j * n, l.t32); });
-            spmv<float>(h, PK_SPMV, l.K, skern::SPMV_SET, l.t32, l.u32, nullptr, s);
-            asm_apply<float>(h, l, l.u32, l.t32, 1.0, 0.0, s);
+            spmv<float>(h, PK_SPMV, K, skern::SPMV_SET, l.t32, l.u32, nullptr, s);
+            asm_apply<float>(h, l, l.u32, l.t32, 1.0, 0.0, s, nullptr, skern::PULL_X_NONE, nullptr, nullptr, threads);
             launch(h, -1, s, [&] { skern::convert_vec<double, float><<<grid_for(n), 256, 0, s>>>(n, l.t32, w); });
         } else {
             spmv<double>(h, PK_SPMV, l.K, skern::SPMV_SET, V + (long long)j * n, l.t64, nullptr, s);
-            asm_apply<double>(h, l, l.t64, w, 1.0, 0.0, s);
+            asm_apply<double>(h, l, l.t64, w, 1.0, 0.0, s, nullptr, skern::PULL_X_NONE, nullptr, nullptr, threads);
         }
         cgs2(h, n, j + 1, V, w, hh, yy, hn, s, ws);
         launch(h, -1, s, [&] { skern::arnoldi_store<<<1, 1, 0, s>>>(j, m, Hs, hh, hn); });
@@ -1469,7 +1478,7 @@ void fbf_apply(stokes_mg* h, const double* r, double* z, cudaStream_t s) {
     const int nu = F.nu, nS = F.nS, d = F.S0.d, np = nS - nu, prec = h->opts.precision;
     // the components in one pass of the cycle: one after another its launches,
     // whose work on the coarse levels is far below what a launch takes, came d
-    // times (setup and solve of SV P4 on the disk, mixed: 52.5 ms, 46.7 ms now)
+    // times (setup and solve of SV P4 on the disk, mixed: 52.5 -> 46.7 ms)
     auto vcycles = [&](const double* in, double* out) {
         CK(cudaMemcpyAsync(h->vin, in, sizeof(double) * nu, cudaMemcpyDeviceToDevice, s));
         vcycle_run(h, prec, s, d);
