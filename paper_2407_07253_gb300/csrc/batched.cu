@@ -388,8 +388,8 @@ __device__ __forceinline__ bool mbar_try(uint32_t a, uint32_t parity) {
 }
 // bounded wait; false (and the CTA's abort flag set) after `limit` polls,
 // or at once if another role has already given up
-__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int* abort_flag, int limit) {
-    for (int i = 0; i < limit; ++i) {
+__device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile int* abort_flag, long long limit) {
+    for (long long i = 0; i < limit; ++i) {
         if (mbar_try(a, parity)) return true;
         if (*abort_flag) return false;
     }
@@ -401,7 +401,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t a, uint32_t parity, volatile 
 // polls for itself, so at a timeout some may see the phase complete and others
 // the abort flag, and those that went on would wait in elect.sync, __syncwarp or
 // tcgen05.ld for the ones that left
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t a, uint32_t parity, volatile int* abort_flag, int limit) {
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t a, uint32_t parity, volatile int* abort_flag, long long limit) {
     return __all_sync(0xffffffffu, mbar_wait(a, parity, abort_flag, limit));
 }
 
@@ -466,13 +466,15 @@ __device__ __forceinline__ void ld16(uint32_t taddr, uint32_t (&v)[16]) {
 // 3xTF32, 32 right-hand sides, 16,129 patches of 81 DoFs and less: 434 -> 263 us;
 // 64 right-hand sides, 16^3 P3 (4817 patches of up to 540 DoFs, 3.9 GB of
 // inverses): 1664 -> 1262 us (3.1 TB/s; two to three stages of 40 KB fit).
-template <int M, int ST, bool SPLIT>
+template <int M, int ST, bool SPLIT, bool GIVE_UP>
 __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npatch, int maxn, int lr, int gw, const int* __restrict__ plist,
                                                                         const int* __restrict__ poff,
                                                                         const int* __restrict__ pdofs,
                                                                         const CUtensorMap* __restrict__ tmaps,
                                                                         const float* __restrict__ X,
-                                                                        float* __restrict__ Yb, int* status, int limit) {
+                                                                        float* __restrict__ Yb, int* status) {
+    // polls of a wait; a constant, since the loop's bound is on the way of every stage
+    constexpr long long limit = GIVE_UP ? 0 : GEMM_WAIT_LIMIT;
     constexpr int NP = np_of(M);
     extern __shared__ __align__(1024) unsigned char smem_tc[];
     const int tid = threadIdx.x, lane = tid & 31;
@@ -539,23 +541,25 @@ __global__ void __launch_bounds__(threads_of(SPLIT), 1) k_patch_gemm_tc(int npat
     const uint32_t tmem = *tmem_slot;
 
     const uint32_t bar0 = SPLIT ? raw0 : full0;    // the copies complete on it
-    int issued = 0;                                // thread 0: stages whose copies were issued
+    volatile int* issued = reinterpret_cast<volatile int*>(smem_tc + 24 * ST + 48);   // stages whose copies were issued
     if (warp == 0) {
         // ---------------------------------------------------------- TMA ---
         if (lane == 0) {
-            for (int k = 0; k < kpatch; ++k) {
+            int it = 0;
+            for (int k = 0; k < kpatch && !*abort_flag; ++k) {
                 int p, s0, n;
                 item(k, p, s0, n);
                 const int tiles = tiles_of(n), nst = (n + KS - 1) / KS;
                 const CUtensorMap* tm = tmaps + p;
-                for (int j = 0; j < nst; ++j, ++issued) {
-                    const int s = issued % ST;
-                    if (issued >= ST && !mbar_wait(empty0 + 8 * s, ((issued / ST) - 1) & 1, abort_flag, limit)) goto done;
+                for (int j = 0; j < nst; ++j, ++it) {
+                    const int s = it % ST;
+                    if (it >= ST && !mbar_wait(empty0 + 8 * s, ((it / ST) - 1) & 1, abort_flag, limit)) break;
                     const uint32_t st = stage0 + (uint32_t)(s * sbytes);
                     mbar_expect_tx(bar0 + 8 * s, (uint32_t)(tiles * A_TILE));
                     for (int mt = 0; mt < tiles; ++mt) tma_load_2d(st + mt * A_TILE, tm, bar0 + 8 * s, j * KS, mt * 128);
                 }
             }
+            *issued = it;
         }
     } else if (warp == 1) {
         // ---------------------------------------------------------- MMA ---
@@ -749,7 +753,7 @@ done:
         if (tid == 0) {
             atomicExch(status, 1);
             int left = (int)GEMM_WAIT_LIMIT;
-            for (int s = 0; s < ST && s < issued; ++s) left = settle(bar0 + 8 * s, ((issued - 1 - s) / ST) & 1, left);
+            for (int s = 0, n = *issued; s < ST && s < n; ++s) left = settle(bar0 + 8 * s, ((n - 1 - s) / ST) & 1, left);
         } else if (warp == 1) {
             commit(drain0);
             settle(drain0, 0, (int)GEMM_WAIT_LIMIT);
@@ -933,20 +937,24 @@ static TcPlan tc_plan(int maxn, int m, int npatch, bool split = false) {
 
 template <int M, int ST, bool SPLIT>
 static void launch_tc(const TcPlan& pl, int nlist, const int* plist, int maxn, const int* poff, const int* pdofs,
-                      const void* tmaps, const float* X, float* Yb, int* status, int limit, cudaStream_t s) {
-    cudaFuncSetAttribute(tc::k_patch_gemm_tc<M, ST, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
-    tc::k_patch_gemm_tc<M, ST, SPLIT><<<pl.grid, tc::threads_of(SPLIT), pl.smem, s>>>(
-        nlist, maxn, pl.lr, pl.gw, plist, poff, pdofs, reinterpret_cast<const CUtensorMap*>(tmaps), X, Yb, status,
-        limit);
+                      const void* tmaps, const float* X, float* Yb, int* status, bool give_up, cudaStream_t s) {
+    auto go = [&](auto kern) {
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem);
+        kern<<<pl.grid, tc::threads_of(SPLIT), pl.smem, s>>>(nlist, maxn, pl.lr, pl.gw, plist, poff, pdofs,
+                                                             reinterpret_cast<const CUtensorMap*>(tmaps), X, Yb, status);
+    };
+    if (!give_up) go(tc::k_patch_gemm_tc<M, ST, SPLIT, false>);
+    // the waits that give up at once: for gemm_timeout_probe's sizes alone
+    else if constexpr (M == 16 && ST == (SPLIT ? 6 : 8)) go(tc::k_patch_gemm_tc<M, ST, SPLIT, true>);
 }
 
 template <int M, bool SPLIT>
 static void launch_tc_st(int nlist, const int* plist, int maxn, const int* poff, const int* pdofs, const void* tmaps,
-                         const float* X, float* Yb, int* status, int limit, cudaStream_t s) {
+                         const float* X, float* Yb, int* status, bool give_up, cudaStream_t s) {
     const TcPlan pl = tc_plan(maxn, M, nlist, SPLIT);
     switch (pl.stages) {
 #define SBAT_TC_CASE(S) \
-    case S: launch_tc<M, S, SPLIT>(pl, nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, limit, s); break;
+    case S: launch_tc<M, S, SPLIT>(pl, nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, give_up, s); break;
         SBAT_TC_CASE(2) SBAT_TC_CASE(3) SBAT_TC_CASE(4) SBAT_TC_CASE(5) SBAT_TC_CASE(6) SBAT_TC_CASE(7)
         SBAT_TC_CASE(8) SBAT_TC_CASE(9) SBAT_TC_CASE(10) SBAT_TC_CASE(11) SBAT_TC_CASE(12)
 #undef SBAT_TC_CASE
@@ -957,12 +965,12 @@ static void launch_tc_st(int nlist, const int* plist, int maxn, const int* poff,
 template <int M>
 static void patch_gemm_m(int mode, int kind, int nw, int nlist, const int* plist, int maxn, const int* poff,
                          const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
-                         const float* X, float* Yb, int* status, int limit, cudaStream_t s) {
+                         const float* X, float* Yb, int* status, bool give_up, cudaStream_t s) {
     if (kind == GEMM_KIND_AUTO) kind = gemm_kind(mode, maxn);
     if (kind == GEMM_KIND_TC && mode == GEMM_3XTF32)
-        launch_tc_st<M, true>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, limit, s);
+        launch_tc_st<M, true>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, give_up, s);
     else if (kind == GEMM_KIND_TC)
-        launch_tc_st<M, false>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, limit, s);
+        launch_tc_st<M, false>(nlist, plist, maxn, poff, pdofs, tmaps, X, Yb, status, give_up, s);
     else if (mode == GEMM_3XTF32)
         launch_gemm_st<M, GEMM_3XTF32>(maxn, nw, nlist, plist, poff, pdofs, ioff, inv, X, Yb, s);
     else
@@ -1027,19 +1035,19 @@ void build_tmaps(int npatch, const int* poff_d, const long long* ioff_d, const f
 
 void patch_gemm(int mode, int kind, int nw, int nlist, const int* plist, int maxn, int m, const int* poff,
                 const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
-                const float* X, float* Yb, int* status, cudaStream_t s, int limit) {
+                const float* X, float* Yb, int* status, cudaStream_t s, bool give_up) {
     if (nlist <= 0) return;
     switch (m) {
 #define SBAT_M(MM) \
     case MM: \
         patch_gemm_m<MM>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, X, \
-                         Yb, status, limit, s); \
+                         Yb, status, give_up, s); \
         break;
         SBAT_M(8) SBAT_M(16) SBAT_M(32)
 #undef SBAT_M
         default:
             patch_gemm_m<64>(mode, kind, nw, nlist, plist, maxn, poff, pdofs, ioff, inv, tmaps, X,
-                             Yb, status, limit, s);
+                             Yb, status, give_up, s);
     }
 }
 
@@ -1083,7 +1091,7 @@ int gemm_timeout_probe(int mode, cudaStream_t s) {
     int* status = (int*)up(flag, sizeof(flag));
     if (e == cudaSuccess) {
         build_tmaps(np, poff, ioff, A, maps);
-        patch_gemm(mode, GEMM_KIND_TC, 0, np, nullptr, 300, m, poff, pdofs, ioff, A, maps, X, Y, status, s, 0);
+        patch_gemm(mode, GEMM_KIND_TC, 0, np, nullptr, 300, m, poff, pdofs, ioff, A, maps, X, Y, status, s, true);
         patch_gemm(mode, GEMM_KIND_TC, 0, np, nullptr, 300, m, poff, pdofs, ioff, A, maps, X, Y, status + 1, s);
         e = cudaGetLastError();
     }

@@ -69,7 +69,7 @@ int gemm_kind(int mode, int n);
 int gemm_default_warps(int maxn);
 void patch_gemm(int mode, int kind, int nw, int nlist, const int* plist, int maxn, int m, const int* poff,
                 const int* pdofs, const long long* ioff, const float* inv, const void* tmaps,
-                const float* X, float* Yb, int* status, cudaStream_t s, int limit = GEMM_WAIT_LIMIT);
+                const float* X, float* Yb, int* status, cudaStream_t s, bool give_up = false);
 
 // out[j * m + c] = alpha * wt[j] * sum_{q in slots(j)} Yb[sidx[q] * m + c] + beta * out[j * m + c]
 // (slots in increasing order: a fixed summation order; the partition-of-unity
